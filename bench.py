@@ -25,7 +25,7 @@ requests by a 40 GB budget and batches them continuously.
   roofline       HBM roofline of the whole update step: algorithmic bytes
                  B = 12 N + 24 U per round (every point read once; every cell
                  updated or cleared read and written once) over the step time.
-  ray            the ray march (k_ray), the dominant kernel: samples/s and its
+  ray            the points and their ray march (k_points), the dominant kernel: samples/s and its
                  event-timed share of a round.
   load_sweep     p50 / p99 latency and mean batch size, served vs plain, at
                  several Poisson loads.
@@ -169,13 +169,9 @@ def file_hash(*paths) -> str:
 
 
 CSRC = "paper_2204_12876_gb300/csrc/"
-KERNEL_SOURCES = {"ray": [CSRC + "k_ray.cu", CSRC + "ray_pass.cuh", CSRC + "em_point.cuh", CSRC + "em_internal.cuh"],
-                  "count": [CSRC + "k_sort.cu", CSRC + "sort_pass.cuh", CSRC + "em_point.cuh", CSRC + "em_internal.cuh"],
-                  "scatter": [CSRC + "k_sort.cu", CSRC + "sort_pass.cuh", CSRC + "em_point.cuh",
-                              CSRC + "em_internal.cuh"],
-                  "alloc": [CSRC + "k_sort.cu", CSRC + "sort_pass.cuh", CSRC + "em_point.cuh", CSRC + "em_internal.cuh"],
-                  "fuse": [CSRC + "k_fuse.cu", CSRC + "fuse_pass.cuh", CSRC + "em_point.cuh", CSRC + "em_internal.cuh"],
-                  "clear": [CSRC + "k_ray.cu", CSRC + "ray_pass.cuh", CSRC + "em_point.cuh", CSRC + "em_internal.cuh"]}
+_POINT = [CSRC + "k_point.cu", CSRC + "point_pass.cuh", CSRC + "em_point.cuh", CSRC + "em_internal.cuh"]
+_CELL = [CSRC + "k_cell.cu", CSRC + "cell_pass.cuh", CSRC + "em_point.cuh", CSRC + "em_internal.cuh"]
+KERNEL_SOURCES = {"scatter": _POINT, "ray": _POINT, "count": _CELL, "fuse": _CELL}  # by profile slot
 
 
 def ncu_traffic(kernel: str, workload: str):
@@ -407,9 +403,9 @@ def run_ours(args, rank: int, world: int):
                 "per_round": {"points": round_pts, "points_in_map": in_map, "cells_updated": cells_upd,
                               "cells_cleared": cells_clr}}
     ray_ms = prof["ray"][0] / prof["ray"][1] if prof.get("ray", (0, 0))[1] else None
-    ray = {"kernel": "k_ray", "samples_per_launch": samples, "ms_per_launch": ray_ms,
+    ray = {"kernel": "k_points", "samples_per_launch": samples, "ms_per_launch": ray_ms,
            "samples_per_s": samples / (ray_ms / 1e3) if ray_ms else None,
-           "share_of_round": kernels.get("k_ray", {}).get("share"), "traffic": ncu_traffic("ray", "served_round")}
+           "share_of_round": kernels.get("k_points", {}).get("share"), "traffic": ncu_traffic("ray", "served_round")}
 
     # ---- end to end through the library: each round's 32 clouds lie in page-locked
     # host memory (a client's ring of input buffers; the pools repeat every 8 rounds);

@@ -129,7 +129,7 @@ typedef struct em_info {
   int32_t t_now;           /* number of updates fused so far */
   int64_t shift_x, shift_y;/* cumulative em_shift in cells; the map centre is (shift_x r, shift_y r) */
   double x0, y0;           /* lower-left corner of the map in the map frame */
-  int64_t point_capacity;  /* points per update the workspace holds without growing */
+  int64_t point_capacity;  /* points per update reserved for (em_reserve); the trace holds as many */
   int64_t device_bytes;    /* device memory held by the map */
 } em_info;
 
@@ -226,17 +226,17 @@ int em_get_trace(em_map* map, int32_t* ix, int32_t* iy, uint8_t* status, int64_t
  * for the previous update's events (so timing adds a host wait per update).
  * Slots of em_profile_read, in this order: */
 enum {
-  EM_PROF_COUNT = 0,   /* k_count: transform + bin + per-tile counts; ray thresholds */
-  EM_PROF_RAY,         /* k_ray: visibility ray march */
-  EM_PROF_ALLOC,       /* k_alloc: record ranges of the tiles */
-  EM_PROF_SCATTER,     /* k_scatter: records into their tile's range */
-  EM_PROF_FUSE,        /* k_fuse: per-cell gate + fusion, one tile per block */
-  EM_PROF_CLEAR,       /* k_clear: removal of penetrated cells */
+  EM_PROF_COUNT = 0,   /* k_cells: drift compensation of the estimates, ray thresholds */
+  EM_PROF_RAY,         /* k_points: gate and sums of every point, visibility ray march */
+  EM_PROF_ALLOC,       /* (no kernel) */
+  EM_PROF_SCATTER,     /* k_pre: points per cell for the wall rule, drift sums */
+  EM_PROF_FUSE,        /* k_write: new state of every cell, removal, overlap clearance */
+  EM_PROF_CLEAR,       /* (no kernel) */
   EM_PROF_NORMALS,
   EM_PROF_SMOOTH,
   EM_PROF_INPAINT,
-  EM_PROF_DRIFT,       /* k_drift: drift compensation of the estimates (and the ray thresholds) */
-  EM_PROF_OVERLAP,     /* k_overlap: overlap clearance near the robot */
+  EM_PROF_DRIFT,       /* (no kernel) */
+  EM_PROF_OVERLAP,     /* (no kernel) */
   EM_PROF_PERSIST,     /* k_persist: the passes of a batched update in one launch (EM_BATCH_PERSISTENT) */
   EM_PROF_SLOTS
 };
@@ -249,8 +249,7 @@ int em_profile_read(em_map* map, double* ms, int64_t* launches);
  * sequence of kernels over all of them -- the per-point and per-cell work of
  * every map shares each launch, so small updates no longer pay a launch
  * sequence each.  The arithmetic per map is exactly em_update's.
- * A batch object owns the record workspace (max_points records), a ring of
- * device descriptors, and -- with EM_BATCH_GRAPH -- one captured CUDA graph
+ * A batch object owns a ring of device descriptors and -- with EM_BATCH_GRAPH -- one captured CUDA graph
  * per descriptor slot, replayed with a single cudaGraphLaunch per batch (grids
  * are sized from the capacities; actual sizes are read from the descriptor). */
 typedef struct em_batch em_batch;
@@ -278,12 +277,9 @@ int em_wait_selftest(int device, int32_t wait_us);
 typedef struct em_tuning {
   int32_t ray_group;    /* ray march: samples per chunk tested against the coarse threshold grid,
                            and lanes per marched chunk: 1, 2, 4, 8, 16 or 32 */
-  int32_t fuse_chunk;   /* threads per fusion block (one tile of 1024 cells per block): 64 .. 1024, a
-                           power of two; 512 and more run 512-thread blocks (three resident per SM
-                           when the cell space has at least three tiles per SM -- for a graph-
-                           replayed batch the capacity's, else the update's -- otherwise two),
-                           the rest 256-thread ones */
-  int32_t big_thresh;   /* tiles with more than 16 x big_thresh records are fused first: 32 .. 1023 */
+  int32_t fuse_chunk;   /* 64 .. 1024, a power of two; checked and kept, picks nothing (the points are
+                           added to their cells without grouping) */
+  int32_t big_thresh;   /* 32 .. 1023; checked and kept, picks nothing */
 } em_tuning;
 
 /* Capacities: at most max_maps distinct maps, max_clouds clouds and
@@ -309,7 +305,7 @@ int em_batch_profile(em_batch* batch, int enable);
 int em_batch_profile_read(em_batch* batch, double* ms, int64_t* launches);
 
 /* Autotuner: times candidate launch shapes on this workload (median of `reps`
- * runs each, coordinate by coordinate) on scratch copies of the maps -- the
+ * runs each) on scratch copies of the maps -- the
  * maps themselves are not changed -- and keeps the fastest.  Synchronous.
  * *out (may be NULL) receives the choice. */
 int em_batch_autotune(em_batch* batch, em_map* const* maps, const em_cloud* clouds, int32_t count,
@@ -331,9 +327,8 @@ typedef struct em_server em_server;
 
 enum { EM_SERVE_BATCHED = 0, EM_SERVE_PLAIN = 1 };
 
-/* Admission accounting: each admitted request holds this many bytes per point
- * (one grouped record per point), and each batch stream a workspace of
- * max_batch_points records. */
+/* Admission accounting: each admitted request counts this many bytes per point,
+ * and each batch stream as many for max_batch_points points. */
 enum { EM_SERVE_RECORD_BYTES = 16 };
 
 typedef struct em_server_cfg {
@@ -430,7 +425,7 @@ int em_server_destroy(em_server* srv); /* NULL-safe: drains, stops the worker, f
  * The paper has no counterpart: this entry point exists for callers that
  * cannot allocate device memory when they update a map -- a real-time loop
  * that forbids allocation after start-up, or a framework whose own allocator
- * already holds the device memory.  It runs the update of em_update (binning, counting sort by cell,
+ * already holds the device memory.  It runs the update of em_update (binning,
  * wall rule, Mahalanobis gate, Eq. 1/2 fusion, ray march and removal; not the
  * per-cell filters) on layers the caller owns, in logical row-major order
  * without a ring offset:
@@ -443,7 +438,7 @@ int em_server_destroy(em_server* srv); /* NULL-safe: drains, stops the worker, f
  *   shift_x/y   the map centre is (shift_x r, shift_y r) (see em_info)
  *   t_now       index of this update (>= 1): cells it writes get t_last = t_now
  *   clouds[]    host array; clouds[i].points device memory
- * All scratch lives in one static device array of the library (about 6.1 MiB,
+ * All scratch lives in one static device array of the library (about 2.9 MiB,
  * held by every GPU that loads the library until the process exits).  The
  * first call on a device looks up that array's address with the device
  * current; make that first call before any stream capture.  Every call uses

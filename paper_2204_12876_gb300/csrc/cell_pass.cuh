@@ -1,0 +1,214 @@
+// cell_pass.cuh -- the device passes over the cells (k_cell.cu):
+//
+//   cells_pass  before the points: estimates moved by the drift, ray thresholds
+//               of the pre-update map and their largest per coarse block
+//   write_pass  after them: every cell's new state from its sums, removal of
+//               marked cells, overlap clearance
+//
+// Each pass runs on the blocks of a Grid: its own kernel's, or the persistent
+// kernel's (k_persist.cu).
+#pragma once
+
+#include "em_point.cuh"
+
+namespace em {
+
+constexpr int kCellThreads = 256;
+
+// One warp per item of kItemW x kItemH logical cells: a lane's column of 8
+// cells gives 24 independent loads, rows are coalesced in both layouts, and the
+// item's four coarse blocks are maxima over 8 lanes.  The thresholds go to
+// logical order, so the march indexes them without the ring wrap.
+static_assert(kItemH == kCoarse && kItemW == 32 && kItemW % kCoarse == 0, "items hold whole coarse blocks");
+__device__ __forceinline__ void cells_pass(const BatchDev& b, Grid gr) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  for (int64_t g = (int64_t)gr.bid * warps + warp; g < b.n_items; g += (int64_t)gr.nb * warps) {
+    int lo = 0, hi = b.n_maps - 1;  // the last map whose items start at or before g
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (b.maps[mid].ibegin <= g) lo = mid; else hi = mid - 1;
+    }
+    const MapDev& m = b.maps[lo];
+    const int32_t q = (int32_t)(g - m.ibegin);
+    const int32_t ty = q / m.IW, tx = q - ty * m.IW;
+    const int32_t W = m.W, lx = tx * kItemW + lane, y0 = ty * kItemH;
+    const int32_t rows = lx < W ? min(kItemH, m.H - y0) : 0;
+    int32_t px = lx + m.ox;
+    px -= px >= W ? W : 0;
+    const bool drift = m.drift_flat > 0.f, ray = m.ray_step > 0.f;
+    float var[kItemH], h[kItemH];
+    int32_t tl[kItemH], p[kItemH];
+#pragma unroll
+    for (int r = 0; r < kItemH; ++r) {  // all loads first
+      int32_t py = y0 + r + m.oy;
+      py -= py >= m.H ? m.H : 0;
+      p[r] = py * W + px;
+      var[r] = r < rows ? m.var[p[r]] : __int_as_float(0x7f800000);
+      h[r] = r < rows ? m.h[p[r]] : 0.f;
+      tl[r] = r < rows ? m.t_last[p[r]] : 0;
+    }
+    if (drift) {
+      // height drift compensation (Section II-D): every estimate moves by the mean
+      // error of this update's points in flat cells (k_pre summed them exactly, so
+      // every thread derives the same mean)
+      const unsigned long long n = m.ctl->drift_n;
+      const float mean = n ? __fdiv_rn(fixed_to_float(fix128(m.ctl->drift_h, m.ctl->drift_l)), (float)n) : 0.f;
+      if (q == 0 && lane == 0) {  // once per map
+        atomicAdd(&m.ctl->stats[kStDriftPoints], n);
+        m.ctl->drift_last = mean;
+      }
+#pragma unroll
+      for (int r = 0; r < kItemH; ++r) {
+        if (r < rows && isfinite(var[r]) && n) {
+          h[r] = __fadd_rn(h[r], mean);
+          m.h[p[r]] = h[r];
+        }
+      }
+    }
+    if (!ray) continue;
+    // Eq. 3: h - sqrt(var_eff); an empty cell is never penetrated (-inf).  With
+    // the upper-bound layer it holds the cell's bound instead, so a ray sample
+    // below the bound takes the march's candidate path and lowers it (Section II-H)
+    float mx = __int_as_float(0xff800000);
+#pragma unroll
+    for (int r = 0; r < kItemH; ++r) {
+      if (r >= rows) continue;
+      float t = __int_as_float(0xff800000);
+      if (isfinite(var[r])) t = __fsub_rn(h[r], __fsqrt_rn(var_eff(m, var[r], tl[r])));
+      else if (m.upper) t = m.upper[p[r]];
+      m.thr[(y0 + r) * W + lx] = t;
+      mx = fmaxf(mx, t);  // a NaN never marks: skipped
+    }
+#pragma unroll
+    for (int o = 1; o < kCoarse; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
+    const int32_t cx = tx * (kItemW / kCoarse) + lane / kCoarse;
+    if (lane % kCoarse == 0 && cx < m.CW) m.cthr[ty * m.CW + cx] = mx;
+  }
+}
+
+// New state of a cell from its complete sums; acc: some point was accepted, rej:
+// rejected points (Section II-C: every rejection adds outlier_variance; then
+// Eq. 1 and Eq. 2 for all accepted points at once in information form).
+__device__ __forceinline__ void fused_state(const MapDev& m, float h, float var, int32_t tl, __int128 qw, __int128 qt,
+                                            bool acc, uint32_t rej, float& h_new, float& var_new) {
+  const float sw = fixed_to_float(qw), st = fixed_to_float(qt);
+  if (isfinite(var)) {
+    const float vprior = __fadd_rn(var_eff(m, var, tl), __fmul_rn((float)(int)rej, m.v_out));
+    if (!acc) {
+      h_new = h;
+      var_new = vprior;
+    } else {
+      const float lam = __fadd_rn(__frcp_rn(vprior), sw);
+      h_new = __fadd_rn(h, __fdiv_rn(st, lam));
+      var_new = __frcp_rn(lam);
+    }
+  } else {
+    h_new = __fadd_rn(m.z_ref, __fdiv_rn(st, sw));
+    var_new = __frcp_rn(sw);
+  }
+}
+
+// A cell's accumulator with one 32-byte load.
+__device__ __forceinline__ CellAcc load_acc(const CellAcc* p) {
+  CellAcc a;
+  asm volatile("ld.global.v4.u64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(a.wh), "=l"(a.wl), "=l"(a.th), "=l"(a.tl)
+               : "l"(p)
+               : "memory");
+  return a;
+}
+__device__ __forceinline__ void clear_acc(CellAcc* p) {
+  asm volatile("st.global.v4.u64 [%0], {%1, %1, %1, %1};" ::"l"(p), "l"(0ull) : "memory");
+}
+
+// One block per tile of kTile cells, a cell per thread and round: the sums of
+// the tile's four rounds are in flight together.  Sums, counts, marks and the
+// tile's flag go back to zero for the next update.  Tiles start on multiples of
+// kTile cells, so a tile owns whole mark words.
+constexpr int kWriteRounds = kTile / kCellThreads;
+__device__ __forceinline__ void write_pass(const BatchDev& b, Grid gr) {
+  const int lane = threadIdx.x & 31;
+  if (gr.bid == 0 && threadIdx.x == 0) b.ctl->next = 0;
+  for_each_tile(b, gr, [&](const MapDev& m, int, int32_t p0, int32_t count) {
+    const int32_t tile = p0 / kTile;
+    if (p0 == 0 && threadIdx.x == 0) {  // once per map
+      atomicAdd(&m.ctl->stats[kStUpdates], 1ull);
+      m.ctl->drift_h = 0;
+      m.ctl->drift_l = 0;
+      m.ctl->drift_n = 0;
+    }
+    const bool touched = m.touched[tile] != 0;
+    const bool overlap = m.ovl_dz > 0.f;
+    CellAcc a[kWriteRounds];
+    uint32_t rej[kWriteRounds], mark[kWriteRounds];
+#pragma unroll
+    for (int k = 0; k < kWriteRounds; ++k) {
+      const int32_t i = k * kCellThreads + threadIdx.x, c = p0 + i;
+      a[k] = CellAcc{0, 0, 0, 0};
+      rej[k] = 0;
+      mark[k] = i < count ? m.mark[c >> 5] : 0u;
+      if (touched && i < count) {
+        a[k] = load_acc(m.acc + c);
+        rej[k] = m.rej[c];
+        if (m.cnt && m.cnt[c]) m.cnt[c] = 0;
+      }
+    }
+    unsigned updated = 0, cleared = 0;
+#pragma unroll
+    for (int k = 0; k < kWriteRounds; ++k) {
+      const int32_t i = k * kCellThreads + threadIdx.x, c = p0 + i;
+      const bool acc = (a[k].wh | a[k].wl) != 0;  // (an accepted point leaves a weight or kAccTouched)
+      const bool mk = (mark[k] >> (c & 31)) & 1u;
+      const bool fused = acc || rej[k] != 0;
+      // overlap clearance (Section II-F): an estimate whose cell centre lies within
+      // overlap_radius of the robot (the first cloud's sensor origin) and whose
+      // height is more than overlap_dz from the robot's belongs to another floor
+      bool near = false;
+      if (overlap && i < count) {
+        int32_t lx, ly;
+        logical_of(m, c, lx, ly);
+        const float cx = __fsub_rn(__fmaf_rn(__fadd_rn((float)lx, 0.5f), m.res, m.x0), m.ref_x);
+        const float cy = __fsub_rn(__fmaf_rn(__fadd_rn((float)ly, 0.5f), m.res, m.y0), m.ref_y);
+        near = __fmaf_rn(cx, cx, __fmul_rn(cy, cy)) <= m.ovl_r2;
+      }
+      if (!(fused || mk || near)) continue;
+      float h = m.h[c], var = m.var[c];
+      int32_t tl = m.t_last[c];
+      bool gone = false;
+      if (fused) {
+        if (acc) clear_acc(m.acc + c);
+        if (rej[k]) m.rej[c] = 0;
+        float hn, vn;
+        fused_state(m, h, var, tl, fix128((long long)a[k].wh, a[k].wl & ~kAccTouched),
+                    fix128((long long)a[k].th, a[k].tl), acc, rej[k], hn, vn);
+        h = hn;
+        var = vn;
+        m.h[c] = h;
+        m.var[c] = var;
+        m.t_last[c] = m.t_now;
+        if (m.upper) m.upper[c] = __int_as_float(0x7f800000);  // observed: no bound (Section II-H)
+        ++updated;
+      } else if (mk && isfinite(var) && m.t_now - tl >= (m.min_age > 1 ? m.min_age : 1)) {
+        gone = true;  // penetrated and not written recently (a cell written now has age 0)
+        ++cleared;
+      }
+      if (!gone && near && isfinite(var) && fabsf(__fsub_rn(h, m.z_ref)) > m.ovl_dz) gone = true;
+      if (gone) {
+        m.h[c] = __int_as_float(0x7fc00000);
+        m.var[c] = __int_as_float(0x7f800000);
+      }
+    }
+    // the mark words are reset after their readers (one warp each) have read them
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < kWriteRounds; ++k)
+      if (lane == 0 && mark[k]) m.mark[(p0 + k * kCellThreads + (int)threadIdx.x) >> 5] = 0u;
+    const unsigned nu = __reduce_add_sync(kFull, updated), nc = __reduce_add_sync(kFull, cleared);
+    if (lane == 0 && nu) atomicAdd(&m.ctl->stats[kStCellsUpdated], (unsigned long long)nu);
+    if (lane == 0 && nc) atomicAdd(&m.ctl->stats[kStCleared], (unsigned long long)nc);
+    __syncthreads();  // every thread has read the tile's flag
+    if (threadIdx.x == 0 && touched) m.touched[tile] = 0;
+  });
+}
+
+}  // namespace em

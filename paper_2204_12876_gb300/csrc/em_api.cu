@@ -71,29 +71,18 @@ struct em_map {
   uint32_t* mark = nullptr;
   float* thr = nullptr;
   float* cthr = nullptr;  // coarse grid of the ray thresholds (maps with the ray march)
-  int32_t* tile_cnt = nullptr;   // per tile of 1024 cells: record counts, ranges, claims
-  int32_t* tile_base = nullptr;
-  int32_t* tile_cur = nullptr;
-  int32_t* tile_map = nullptr;
-  FuseItem* heavy = nullptr;                // the fusion's work lists (one entry per tile)
-  FuseItem* light = nullptr;
-  unsigned long long* split_acc = nullptr;  // accumulator slots of split tiles (zero between updates)
-  int32_t* split_done = nullptr;
-  int32_t split_slots = 0;
-  FuseItem* pieces = nullptr;               // piece list (with the record workspace)
-  int32_t max_pieces = 0;
+  CellAcc* acc = nullptr;        // the fusion's sums, rejected points, wall-rule counts (zero between updates)
+  uint32_t* rej = nullptr;
+  uint32_t* cnt = nullptr;       // maps with the wall rule
+  uint8_t* touched = nullptr;    // per tile of 1024 cells
   MapCtl* ctl = nullptr;
   BatchCtl* bctl = nullptr;
   // geometry
   int32_t ox = 0, oy = 0;
   int64_t shift_x = 0, shift_y = 0;
   int32_t t_now = 0;
-  // per-update workspace
+  // points per update reserved for (only the trace needs memory per point)
   int64_t cap = 0;
-  float* rz = nullptr;
-  float* rv = nullptr;
-  uint16_t* rc = nullptr;
-  int32_t* idx_sorted = nullptr;
   int32_t* tr_ix = nullptr;
   int32_t* tr_iy = nullptr;
   uint8_t* tr_status = nullptr;
@@ -112,13 +101,9 @@ struct em_map {
   float* layer_stage = nullptr;
   size_t layer_stage_cap = 0;
   cudaStream_t last_stream = nullptr;
-  cudaStream_t side = nullptr;  // the ray march, beside the sort and fusion (maps with a ray step)
-  cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   int64_t layer_bytes = 0;
   int64_t work_bytes = 0;
-  int fuse_threads = 512;
   int ray_group = 8;
-  int heavy_thresh = 256 * 16;
   int64_t points_in = 0;
   // per-kernel profiling
   bool prof = false;
@@ -143,10 +128,8 @@ MapDev make_mapdev(const em_map* m) {
   d.h = m->h; d.var = m->var; d.t_last = m->t_last;
   d.nx = m->nx; d.ny = m->ny; d.nz = m->nz; d.smooth = m->smooth; d.inpaint = m->inpaint; d.upper = m->upper;
   d.mark = m->mark; d.thr = m->thr; d.cthr = m->cthr;
-  if (m->cthr) {
-    d.CW = coarse_dim(m->p.width);
-    d.CH = coarse_dim(m->p.height);
-  }
+  d.acc = m->acc; d.rej = m->rej; d.cnt = m->cnt; d.touched = m->touched;
+  set_item_grid(d, m->p.width, m->p.height, m->p.ray_step > 0.f, m->p.drift_flatness > 0.f);
   d.ctl = m->ctl;
   d.cell_begin = 0;
   d.W = m->p.width; d.H = m->p.height; d.ox = m->ox; d.oy = m->oy;
@@ -193,12 +176,9 @@ bool params_ok(const em_params* p) {
 }
 
 void free_workspace(em_map* m) {
-  cudaFree(m->rz); cudaFree(m->rv); cudaFree(m->rc); cudaFree(m->idx_sorted);
-  cudaFree(m->tr_ix); cudaFree(m->tr_iy); cudaFree(m->tr_status); cudaFree(m->pieces);
-  m->rz = m->rv = nullptr; m->rc = nullptr; m->idx_sorted = nullptr; m->tr_ix = m->tr_iy = nullptr;
+  cudaFree(m->tr_ix); cudaFree(m->tr_iy); cudaFree(m->tr_status);
+  m->tr_ix = m->tr_iy = nullptr;
   m->tr_status = nullptr;
-  m->pieces = nullptr;
-  m->max_pieces = 0;
   m->cap = 0;
   m->work_bytes = 0;
 }
@@ -209,25 +189,16 @@ int grow_workspace(em_map* m, int64_t n) {
   int64_t want = n + n / 4;
   if (want < 4096) want = 4096;
   if (want > (int64_t(1) << 31) - 1) want = (int64_t(1) << 31) - 1;
-  EM_TRY(cudaDeviceSynchronize(), "cudaDeviceSynchronize");
-  free_workspace(m);
-  const bool trace = (m->p.flags & EM_F_TRACE) != 0;
-  int64_t tot = 0;
-  EM_TRY(dev_alloc(&m->rz, (size_t)want, &tot), "alloc workspace");
-  EM_TRY(dev_alloc(&m->rv, (size_t)want, &tot), "alloc workspace");
-  EM_TRY(dev_alloc(&m->rc, (size_t)want, &tot), "alloc workspace");
-  // pieces: a split tile has more than 16 kMinHeavy records per piece but its last
-  const int64_t np = want / (kMinHeavy * 16) + kMaxSplit + 1;
-  EM_TRY(dev_alloc(&m->pieces, (size_t)np, &tot), "alloc workspace");
-  m->max_pieces = (int32_t)np;
-  if (trace) {
-    EM_TRY(dev_alloc(&m->idx_sorted, (size_t)want, &tot), "alloc trace");
+  if (m->p.flags & EM_F_TRACE) {
+    EM_TRY(cudaDeviceSynchronize(), "cudaDeviceSynchronize");
+    free_workspace(m);
+    int64_t tot = 0;
     EM_TRY(dev_alloc(&m->tr_ix, (size_t)want, &tot), "alloc trace");
     EM_TRY(dev_alloc(&m->tr_iy, (size_t)want, &tot), "alloc trace");
     EM_TRY(dev_alloc(&m->tr_status, (size_t)want, &tot), "alloc trace");
+    m->work_bytes = tot;
   }
   m->cap = want;
-  m->work_bytes = tot;
   return EM_OK;
 }
 
@@ -238,13 +209,8 @@ void release(em_map* m) {
   cudaFree(m->h); cudaFree(m->var); cudaFree(m->t_last);
   cudaFree(m->nx); cudaFree(m->ny); cudaFree(m->nz); cudaFree(m->smooth); cudaFree(m->inpaint); cudaFree(m->upper);
   cudaFree(m->mark); cudaFree(m->thr); cudaFree(m->cthr);
-  cudaFree(m->tile_cnt); cudaFree(m->tile_base); cudaFree(m->tile_cur); cudaFree(m->tile_map);
-  cudaFree(m->heavy); cudaFree(m->light);
-  cudaFree(m->split_acc); cudaFree(m->split_done);
+  cudaFree(m->acc); cudaFree(m->rej); cudaFree(m->cnt); cudaFree(m->touched);
   cudaFree(m->ctl); cudaFree(m->bctl);
-  if (m->side) cudaStreamDestroy(m->side);
-  if (m->fork_ev) cudaEventDestroy(m->fork_ev);
-  if (m->join_ev) cudaEventDestroy(m->join_ev);
   free_workspace(m);
   cudaFree(m->desc_dev);
   cudaFreeHost(m->desc_host);
@@ -301,29 +267,12 @@ int upload_desc(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t tot
   b->n_points = total;
   b->maps = reinterpret_cast<const MapDev*>(db + sizeof(BatchDev));
   b->clouds = reinterpret_cast<const CloudDev*>(db + sizeof(BatchDev) + sizeof(MapDev));
-  b->rz = m->rz;
-  b->rv = m->rv;
-  b->rc = m->rc;
-  b->idx_sorted = m->idx_sorted;
   b->tr_ix = m->tr_ix;
   b->tr_iy = m->tr_iy;
   b->tr_status = m->tr_status;
   b->n_cells = pad_tile((int64_t)m->p.width * m->p.height);
-  b->n_coarse = (int64_t)md->CW * md->CH;
+  b->n_items = (int64_t)md->IW * md->IH;
   b->ctl = m->bctl;
-  b->tile_cnt = m->tile_cnt;
-  b->tile_base = m->tile_base;
-  b->tile_cur = m->tile_cur;
-  b->tile_map = m->tile_map;
-  b->heavy = m->heavy;
-  b->light = m->light;
-  b->pieces = m->pieces;
-  b->max_pieces = m->max_pieces;
-  b->split_acc = m->split_acc;
-  b->split_done = m->split_done;
-  b->split_slots = m->split_slots;
-  b->heavy_thresh = m->heavy_thresh;
-  b->fuse_threads = m->fuse_threads;
   const size_t bytes = sizeof(BatchDev) + sizeof(MapDev) + (size_t)n_clouds * sizeof(CloudDev);
   EM_TRY(cudaMemcpyAsync(db, hb, bytes, cudaMemcpyHostToDevice, s), "upload descriptor");
   *out = reinterpret_cast<const BatchDev*>(db);
@@ -470,29 +419,24 @@ int em_create(const em_params* params, int device, em_map** out) {
   if (params->flags & EM_F_INPAINT) { EM_ALLOC(m->inpaint, nc) }
   if (params->flags & EM_F_UPPER) { EM_ALLOC(m->upper, nc) }
   const size_t ntile = (size_t)(pad_tile((int64_t)nc) / kTile);
-  EM_ALLOC(m->mark, (nc + 31) / 32) EM_ALLOC(m->thr, nc)
-  if (params->ray_step > 0.f) { EM_ALLOC(m->cthr, (size_t)coarse_dim(params->width) * coarse_dim(params->height)) }
-  EM_ALLOC(m->tile_cnt, ntile + 1) EM_ALLOC(m->tile_base, ntile + 1) EM_ALLOC(m->tile_cur, ntile + 1)
-  EM_ALLOC(m->tile_map, ntile) EM_ALLOC(m->heavy, ntile) EM_ALLOC(m->light, ntile)
-  m->split_slots = (int32_t)(ntile < (size_t)kMaxSplit ? ntile : (size_t)kMaxSplit);
-  EM_ALLOC(m->split_acc, (size_t)m->split_slots * kSplitWords * kTile) EM_ALLOC(m->split_done, m->split_slots)
+  EM_ALLOC(m->mark, (nc + 31) / 32)
+  if (params->ray_step > 0.f) {
+    EM_ALLOC(m->thr, nc) EM_ALLOC(m->cthr, (size_t)coarse_dim(params->width) * coarse_dim(params->height))
+  }
+  EM_ALLOC(m->acc, nc) EM_ALLOC(m->rej, nc) EM_ALLOC(m->touched, ntile)
+  if (params->wall_num_thresh > 0) { EM_ALLOC(m->cnt, nc) }
   EM_ALLOC(m->ctl, 1) EM_ALLOC(m->bctl, 1)
   EM_ALLOC(m->desc_dev, kDescBytes * kSlots)
 #undef EM_ALLOC
   if (e == cudaSuccess) e = cudaMallocHost((void**)&m->desc_host, kDescBytes * kSlots);
   for (int i = 0; i < kSlots && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&m->desc_ev[i], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->stage_ev, cudaEventDisableTiming);
-  if (e == cudaSuccess && params->ray_step > 0.f) {
-    e = cudaStreamCreateWithFlags(&m->side, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->fork_ev, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->join_ev, cudaEventDisableTiming);
-  }
   if (e == cudaSuccess) e = cudaMemset(m->ctl, 0, sizeof(MapCtl));
-  if (e == cudaSuccess) e = cudaMemset(m->tile_cnt, 0, (ntile + 1) * sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMemset(m->bctl, 0, sizeof(BatchCtl));
-  if (e == cudaSuccess)
-    e = cudaMemset(m->split_acc, 0, (size_t)m->split_slots * kSplitWords * kTile * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMemset(m->split_done, 0, (size_t)m->split_slots * sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMemset(m->acc, 0, nc * sizeof(CellAcc));
+  if (e == cudaSuccess) e = cudaMemset(m->rej, 0, nc * sizeof(uint32_t));
+  if (e == cudaSuccess && m->cnt) e = cudaMemset(m->cnt, 0, nc * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMemset(m->touched, 0, ntile);
   if (e == cudaSuccess) e = cuda_status(launch_fill_map(make_mapdev(m), nullptr), "fill") ? cudaErrorUnknown : cudaSuccess;
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
@@ -501,18 +445,10 @@ int em_create(const em_params* params, int device, em_map** out) {
     return code;
   }
   m->layer_bytes = tot;
-  // tuning knobs (defaults chosen by measurement; the environment overrides them)
-  if (const char* g = getenv("EM_FUSE_THREADS")) {
-    int v = atoi(g);
-    if (v == 256 || v == 512) m->fuse_threads = v;
-  }
+  // tuning knob (the default chosen by measurement; the environment overrides it)
   if (const char* g = getenv("EM_RAY_GROUP")) {
     int v = atoi(g);
     if (v == 1 || v == 2 || v == 4 || v == 8 || v == 16 || v == 32) m->ray_group = v;
-  }
-  if (const char* g = getenv("EM_HEAVY_THRESH")) {
-    int v = atoi(g);
-    if (v >= kMinHeavy && v <= kMaxHeavy) m->heavy_thresh = v * 16;
   }
   *out = m;
   return EM_OK;
@@ -551,32 +487,13 @@ static int update_impl(em_map* m, const em_cloud* clouds, int32_t n_clouds, cuda
   }
   const int64_t ncell = pad_tile((int64_t)m->p.width * m->p.height);
   const bool ext = m->p.excl_d > 0.f || (m->p.flags & EM_F_UPPER);  // kernels with the extended features
-  EM_TRY(timed(m, EM_PROF_COUNT, s, [&] { return launch_bin(bd, total, ncell, ext, s); }), "k_count");
-  if (m->p.drift_flatness > 0.f)
-    EM_TRY(timed(m, EM_PROF_DRIFT, s, [&] { return launch_drift(bd, total, ncell, ext, s); }), "k_drift");
-  if (total > 0) {
-    // the ray march reads only the ray thresholds and the points and writes only
-    // the marks (read by k_clear): it runs on the side stream beside the sort and
-    // the fusion, unless the map has the upper-bound layer (both write it)
-    auto ray = [&](cudaStream_t rs) {
-      return timed(m, EM_PROF_RAY, rs, [&] { return launch_ray(bd, total, ncell, m->ray_group, ext, rs); });
-    };
-    auto rest = [&] {
-      cudaError_t r = timed(m, EM_PROF_ALLOC, s, [&] { return launch_alloc(bd, ncell, s); });
-      if (r == cudaSuccess) r = timed(m, EM_PROF_SCATTER, s, [&] { return launch_scatter(bd, total, ext, s); });
-      if (r == cudaSuccess) r = timed(m, EM_PROF_FUSE, s, [&] { return launch_fuse(bd, ncell, m->fuse_threads, s); });
-      return r;
-    };
-    if (m->p.ray_step > 0.f && !(m->p.flags & EM_F_UPPER)) {
-      EM_TRY(launch_beside(s, m->side, m->fork_ev, m->join_ev, ray, rest), "k_ray / k_alloc / k_scatter / k_fuse");
-    } else {
-      if (m->p.ray_step > 0.f) EM_TRY(ray(s), "k_ray");
-      EM_TRY(rest(), "k_alloc / k_scatter / k_fuse");
-    }
-  }
-  EM_TRY(timed(m, EM_PROF_CLEAR, s, [&] { return launch_clear(bd, ncell, s); }), "k_clear");
-  if (m->p.overlap_dz > 0.f && n_clouds > 0)
-    EM_TRY(timed(m, EM_PROF_OVERLAP, s, [&] { return launch_overlap(bd, ncell, s); }), "k_overlap");
+  const bool ray = m->p.ray_step > 0.f, drift = m->p.drift_flatness > 0.f;
+  if (drift || m->p.wall_num_thresh > 0)
+    EM_TRY(timed(m, EM_PROF_SCATTER, s, [&] { return launch_pre(bd, total, ext, s); }), "k_pre");
+  if (ray || drift) EM_TRY(timed(m, EM_PROF_COUNT, s, [&] { return launch_cells(bd, ncell, s); }), "k_cells");
+  if (total > 0)
+    EM_TRY(timed(m, EM_PROF_RAY, s, [&] { return launch_points(bd, total, m->ray_group, ray, ext, s); }), "k_points");
+  EM_TRY(timed(m, EM_PROF_FUSE, s, [&] { return launch_write(bd, ncell, s); }), "k_write");
   if (m->p.flags & EM_F_NORMALS)
     EM_TRY(timed(m, EM_PROF_NORMALS, s, [&] { return launch_normals(bd, ncell, s); }), "k_normals");
   if (m->p.flags & (EM_F_SMOOTH | EM_F_MEDIAN | EM_F_GAUSS))

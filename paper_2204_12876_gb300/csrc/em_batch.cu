@@ -33,21 +33,19 @@ constexpr int kSlots = 3;
 bool tuning_ok(const em_tuning& t) {
   const int r = t.ray_group, f = t.fuse_chunk;
   return (r == 1 || r == 2 || r == 4 || r == 8 || r == 16 || r == 32) && f >= 64 && f <= 1024 && (f & (f - 1)) == 0 &&
-         t.big_thresh >= kMinHeavy && t.big_thresh <= kMaxHeavy;
+         t.big_thresh >= 32 && t.big_thresh <= 1023;
 }
 
 // what a captured graph depends on besides the slot
 struct GraphKey {
-  em_tuning t;
+  int32_t ray_group;
   bool ray;
   bool drift;
-  bool overlap;
-  bool ext;    // some map uses the exclusion area or the upper-bound layer
-  bool upper;  // some map has the upper-bound layer (the ray march then runs before the fusion)
+  bool wall;
+  bool ext;  // some map uses the exclusion area or the upper-bound layer
   uint32_t stencils;
   bool operator==(const GraphKey& o) const {
-    return t.ray_group == o.t.ray_group && t.fuse_chunk == o.t.fuse_chunk && t.big_thresh == o.t.big_thresh &&
-           ray == o.ray && drift == o.drift && overlap == o.overlap && ext == o.ext && upper == o.upper &&
+    return ray_group == o.ray_group && ray == o.ray && drift == o.drift && wall == o.wall && ext == o.ext &&
            stencils == o.stencils;
   }
 };
@@ -59,22 +57,7 @@ struct em_batch {
   int32_t max_maps = 0, max_clouds = 0, max_cells = 0;
   int64_t max_points = 0;
   uint32_t flags = 0;
-  float* rz = nullptr;  // records (k_sort.cu layout), max_points of each
-  float* rv = nullptr;
-  uint16_t* rc = nullptr;
   BatchCtl* bctl = nullptr;
-  int64_t max_tiles = 0;  // tiles of the padded cell space of a full batch
-  int32_t* tile_cnt = nullptr;
-  int32_t* tile_base = nullptr;
-  int32_t* tile_cur = nullptr;
-  int32_t* tile_map = nullptr;
-  FuseItem* heavy = nullptr;  // the fusion's work lists (one entry per tile)
-  FuseItem* light = nullptr;
-  unsigned long long* split_acc = nullptr;  // accumulator slots of split tiles (zero between updates)
-  int32_t* split_done = nullptr;
-  int32_t split_slots = 0;
-  FuseItem* pieces = nullptr;
-  int32_t max_pieces = 0;
   size_t desc_bytes = 0;
   unsigned char* desc_host = nullptr;
   unsigned char* desc_dev = nullptr;
@@ -82,8 +65,6 @@ struct em_batch {
   int slot = 0;
   em_tuning tune{8, 512, 256};
   cudaStream_t capture_stream = nullptr;
-  cudaStream_t side = nullptr;  // the ray march, beside the sort and fusion
-  cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   cudaGraphExec_t graph[kSlots] = {};
   GraphKey graph_key[kSlots] = {};
   // host scratch for grouping
@@ -127,11 +108,7 @@ int prof_collect(em_batch* b) {
   return EM_OK;
 }
 
-// The kernel sequence of one update over the descriptor at `bd`.  The ray
-// march reads only the ray thresholds (k_count / k_drift) and the points, and
-// writes only the visibility marks (read by k_clear), so it runs on the side
-// stream beside the sort and the fusion -- unless a map has the upper-bound
-// layer, which both the march and the fusion write.
+// The kernel sequence of one update over the descriptor at `bd`.
 cudaError_t launch_sequence(em_batch* b, const BatchDev* bd, int64_t grid_points, int64_t grid_cells,
                             const GraphKey& k, cudaStream_t s, em_batch* prof = nullptr) {
   cudaError_t e = cudaSuccess;
@@ -139,7 +116,7 @@ cudaError_t launch_sequence(em_batch* b, const BatchDev* bd, int64_t grid_points
   // the device can run it and no map needs the drift compensation
   bool persisted = false;
   if ((b->flags & EM_BATCH_PERSISTENT) && !k.drift) {
-    e = timed(prof, EM_PROF_PERSIST, s, [&] { return launch_persist(bd, k.t.ray_group, k.ext, EM_PERSIST_WAIT_MS, s); });
+    e = timed(prof, EM_PROF_PERSIST, s, [&] { return launch_persist(bd, k.ray_group, k.ext, EM_PERSIST_WAIT_MS, s); });
     persisted = e != cudaErrorNotSupported;
     if (!persisted) {
       cudaGetLastError();
@@ -147,34 +124,12 @@ cudaError_t launch_sequence(em_batch* b, const BatchDev* bd, int64_t grid_points
     }
   }
   if (!persisted) {
-    e = timed(prof, EM_PROF_COUNT, s, [&] { return launch_bin(bd, grid_points, grid_cells, k.ext, s); });
-    if (e == cudaSuccess && k.drift)
-      e = timed(prof, EM_PROF_DRIFT, s, [&] { return launch_drift(bd, grid_points, grid_cells, k.ext, s); });
-    if (grid_points > 0) {
-      auto ray = [&](cudaStream_t rs) {
-        return timed(prof, EM_PROF_RAY, rs,
-                     [&] { return launch_ray(bd, grid_points, grid_cells, k.t.ray_group, k.ext, rs); });
-      };
-      auto rest = [&] {
-        cudaError_t r = timed(prof, EM_PROF_ALLOC, s, [&] { return launch_alloc(bd, grid_cells, s); });
-        if (r == cudaSuccess)
-          r = timed(prof, EM_PROF_SCATTER, s, [&] { return launch_scatter(bd, grid_points, k.ext, s); });
-        if (r == cudaSuccess)
-          r = timed(prof, EM_PROF_FUSE, s, [&] { return launch_fuse(bd, grid_cells, k.t.fuse_chunk, s); });
-        return r;
-      };
-      if (e == cudaSuccess) {
-        if (k.ray && !k.upper) {
-          e = launch_beside(s, b->side, b->fork_ev, b->join_ev, ray, rest);
-        } else {
-          if (k.ray) e = ray(s);
-          if (e == cudaSuccess) e = rest();
-        }
-      }
-    }
-    if (e == cudaSuccess) e = timed(prof, EM_PROF_CLEAR, s, [&] { return launch_clear(bd, grid_cells, s); });
-    if (e == cudaSuccess && k.overlap)
-      e = timed(prof, EM_PROF_OVERLAP, s, [&] { return launch_overlap(bd, grid_cells, s); });
+    if (k.drift || k.wall) e = timed(prof, EM_PROF_SCATTER, s, [&] { return launch_pre(bd, grid_points, k.ext, s); });
+    if (e == cudaSuccess && (k.ray || k.drift))
+      e = timed(prof, EM_PROF_COUNT, s, [&] { return launch_cells(bd, grid_cells, s); });
+    if (e == cudaSuccess && grid_points > 0)
+      e = timed(prof, EM_PROF_RAY, s, [&] { return launch_points(bd, grid_points, k.ray_group, k.ray, k.ext, s); });
+    if (e == cudaSuccess) e = timed(prof, EM_PROF_FUSE, s, [&] { return launch_write(bd, grid_cells, s); });
   }
   if (e == cudaSuccess && (k.stencils & EM_F_NORMALS))
     e = timed(prof, EM_PROF_NORMALS, s, [&] { return launch_normals(bd, grid_cells, s); });
@@ -237,19 +192,18 @@ int prepare(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t co
   MapDev* md = reinterpret_cast<MapDev*>(hb + sizeof(BatchDev));
   CloudDev* cd = reinterpret_cast<CloudDev*>(hb + sizeof(BatchDev) + (size_t)b->max_maps * sizeof(MapDev));
   memset(bd, 0, sizeof(BatchDev));
-  GraphKey key{tune, false, false, false, false, false, 0u};
-  int64_t cells = 0, coarse = 0;
+  GraphKey key{tune.ray_group, false, false, false, false, 0u};
+  int64_t cells = 0, items = 0;
   for (int u = 0; u < nm; ++u) {
     md[u] = map_begin_update(b->uniq[u], map_pts[u]);
     md[u].cell_begin = cells;
     cells += pad_tile(map_cells(b->uniq[u]));
-    md[u].cbegin = coarse;
-    coarse += (int64_t)md[u].CW * md[u].CH;
+    md[u].ibegin = items;
+    items += (int64_t)md[u].IW * md[u].IH;
     key.ray |= md[u].ray_step > 0.f;
     key.drift |= md[u].drift_flat > 0.f;
-    key.overlap |= md[u].ovl_dz > 0.f;
+    key.wall |= md[u].cnt != nullptr;
     key.ext |= md[u].excl_d > 0.f || md[u].upper != nullptr;
-    key.upper |= md[u].upper != nullptr;
     key.stencils |= map_flags(b->uniq[u]) & (EM_F_NORMALS | EM_F_SMOOTH | EM_F_MEDIAN | EM_F_GAUSS | EM_F_INPAINT);
   }
   // clouds ordered by map (stable), so each map's points are contiguous
@@ -282,26 +236,11 @@ int prepare(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t co
   bd->n_points = total;
   bd->maps = reinterpret_cast<const MapDev*>(db + sizeof(BatchDev));
   bd->clouds = reinterpret_cast<const CloudDev*>(db + sizeof(BatchDev) + (size_t)b->max_maps * sizeof(MapDev));
-  bd->rz = b->rz;
-  bd->rv = b->rv;
-  bd->rc = b->rc;
   bd->n_cells = cells;
-  bd->n_coarse = coarse;
+  bd->n_items = items;
   bd->ctl = b->bctl;
-  bd->tile_cnt = b->tile_cnt;
-  bd->tile_base = b->tile_base;
-  bd->tile_cur = b->tile_cur;
-  bd->tile_map = b->tile_map;
-  bd->heavy = b->heavy;
-  bd->light = b->light;
-  bd->pieces = b->pieces;
-  bd->max_pieces = b->max_pieces;
-  bd->split_acc = b->split_acc;
-  bd->split_done = b->split_done;
-  bd->split_slots = b->split_slots;
-  bd->heavy_thresh = tune.big_thresh * 16;
-  bd->passes = (key.ray ? kPassRay : 0u) | (key.overlap ? kPassOverlap : 0u);
-  bd->fuse_threads = tune.fuse_chunk;
+  bd->passes = (key.ray ? kPassRay : 0u) | (key.wall || key.drift ? kPassPre : 0u) |
+               (key.ray || key.drift ? kPassCells : 0u);
   // upload header + maps, and the clouds at their fixed offset
   cudaError_t e = cudaMemcpyAsync(db, hb, sizeof(BatchDev) + (size_t)nm * sizeof(MapDev), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
@@ -325,51 +264,6 @@ void finish(em_batch* b, const Prepared& p, cudaStream_t s) {
   cudaEventRecord(b->ev[p.slot], s);
 }
 
-// A captured sequence is one chain of kernel nodes.  Let the ray march
-// (k_coarse -> k_ray) hang off the node before it and join again at k_clear, so
-// it runs beside k_alloc -> k_scatter -> k_fuse (the ray march reads only the
-// ray thresholds and the points and writes only the marks, which k_clear reads).
-// Anything but the expected chain is left as it is.  False when an edit failed
-// half way (the graph must not be used).
-bool overlap_ray_march(cudaGraph_t g) {
-  cudaGraphNode_t root = nullptr;
-  size_t n = 0;
-  if (cudaGraphGetRootNodes(g, nullptr, &n) != cudaSuccess || n != 1) return true;
-  if (cudaGraphGetRootNodes(g, &root, &n) != cudaSuccess) return true;
-  std::vector<cudaGraphNode_t> chain;
-  for (cudaGraphNode_t cur = root; cur && chain.size() < 64;) {
-    chain.push_back(cur);
-    size_t nd = 0;
-    if (cudaGraphNodeGetDependentNodes(cur, nullptr, nullptr, &nd) != cudaSuccess || nd > 1) return true;
-    cudaGraphNode_t next = nullptr;
-    if (nd == 1 && cudaGraphNodeGetDependentNodes(cur, &next, nullptr, &nd) != cudaSuccess) return true;
-    cur = nd == 1 ? next : nullptr;
-  }
-  auto fn = [](cudaGraphNode_t node) -> const void* {
-    cudaGraphNodeType t;
-    if (cudaGraphNodeGetType(node, &t) != cudaSuccess || t != cudaGraphNodeTypeKernel) return nullptr;
-    cudaKernelNodeParams kp = {};
-    if (cudaGraphKernelNodeGetParams(node, &kp) != cudaSuccess) return nullptr;
-    return kp.func;
-  };
-  for (size_t i = 1; i + 5 < chain.size(); ++i) {
-    if (fn(chain[i]) != coarse_kernel()) continue;
-    // chain: prev -> coarse -> ray -> alloc -> scatter -> fuse -> clear
-    if (fn(chain[i + 2]) != alloc_kernel() || !is_fuse_kernel(fn(chain[i + 4])) || fn(chain[i + 5]) != clear_kernel())
-      return true;
-    cudaGraphNode_t prev = chain[i - 1], ray = chain[i + 1], alloc = chain[i + 2], clear = chain[i + 5];
-    if (cudaGraphRemoveDependencies(g, &ray, &alloc, nullptr, 1) != cudaSuccess) {
-      cudaGetLastError();
-      return true;  // nothing changed
-    }
-    const bool ok = cudaGraphAddDependencies(g, &prev, &alloc, nullptr, 1) == cudaSuccess &&
-                    cudaGraphAddDependencies(g, &ray, &clear, nullptr, 1) == cudaSuccess;
-    if (!ok) cudaGetLastError();
-    return ok;
-  }
-  return true;
-}
-
 int run_graph(em_batch* b, const Prepared& p, cudaStream_t s) {
   if (!b->graph[p.slot] || !(b->graph_key[p.slot] == p.key)) {
     if (b->graph[p.slot]) {
@@ -388,11 +282,6 @@ int run_graph(em_batch* b, const Prepared& p, cudaStream_t s) {
       if (g) cudaGraphDestroy(g);
       cudaGetLastError();
       EB_TRY(launch_sequence(b, p.bd, p.points, p.cells, p.key, s), "launch (capture failed)");
-      return EM_OK;
-    }
-    if (p.key.ray && !p.key.upper && !overlap_ray_march(g)) {  // a half-edited graph is not used
-      cudaGraphDestroy(g);
-      EB_TRY(launch_sequence(b, p.bd, p.points, p.cells, p.key, s), "launch (graph edit failed)");
       return EM_OK;
     }
     cudaGraphExec_t ex = nullptr;
@@ -420,22 +309,7 @@ void release(em_batch* b) {
     if (b->ev[i]) cudaEventDestroy(b->ev[i]);
   }
   if (b->capture_stream) cudaStreamDestroy(b->capture_stream);
-  if (b->side) cudaStreamDestroy(b->side);
-  if (b->fork_ev) cudaEventDestroy(b->fork_ev);
-  if (b->join_ev) cudaEventDestroy(b->join_ev);
-  cudaFree(b->rz);
-  cudaFree(b->rv);
-  cudaFree(b->rc);
   cudaFree(b->bctl);
-  cudaFree(b->tile_cnt);
-  cudaFree(b->tile_base);
-  cudaFree(b->tile_cur);
-  cudaFree(b->tile_map);
-  cudaFree(b->heavy);
-  cudaFree(b->light);
-  cudaFree(b->split_acc);
-  cudaFree(b->split_done);
-  cudaFree(b->pieces);
   cudaFree(b->desc_dev);
   cudaFreeHost(b->desc_host);
   delete b;
@@ -491,38 +365,12 @@ int em_batch_create(int device, int32_t max_maps, int32_t max_clouds, int64_t ma
   b->flags = flags;
   b->desc_bytes = (sizeof(BatchDev) + (size_t)max_maps * sizeof(MapDev) + (size_t)max_clouds * sizeof(CloudDev) + 255) &
                   ~size_t(255);
-  const size_t np = (size_t)(max_points > 0 ? max_points : 1);
-  b->max_tiles = (int64_t)max_maps * (pad_tile(max_cells) / kTile);
-  const size_t nt = (size_t)b->max_tiles + 1;
-  cudaError_t e = cudaMalloc((void**)&b->rz, np * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->rv, np * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->rc, np * sizeof(uint16_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->bctl, sizeof(BatchCtl));
+  cudaError_t e = cudaMalloc((void**)&b->bctl, sizeof(BatchCtl));
   if (e == cudaSuccess) e = cudaMemset(b->bctl, 0, sizeof(BatchCtl));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->tile_cnt, nt * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMemset(b->tile_cnt, 0, nt * sizeof(int32_t));  // k_alloc keeps it zero after
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->tile_base, nt * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->tile_cur, nt * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->tile_map, nt * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->heavy, nt * sizeof(FuseItem));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->light, nt * sizeof(FuseItem));
-  // split tiles: at most kMaxSplit slots of kSplitWords x kTile words; pieces of
-  // more than 16 kMinHeavy records but the last of each tile
-  b->split_slots = (int32_t)(b->max_tiles < kMaxSplit ? b->max_tiles : kMaxSplit);
-  b->max_pieces = (int32_t)(np / (kMinHeavy * 16) + kMaxSplit + 1);
-  const size_t acc_bytes = (size_t)b->split_slots * kSplitWords * kTile * sizeof(unsigned long long);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->split_acc, acc_bytes);
-  if (e == cudaSuccess) e = cudaMemset(b->split_acc, 0, acc_bytes);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->split_done, (size_t)b->split_slots * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMemset(b->split_done, 0, (size_t)b->split_slots * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->pieces, (size_t)b->max_pieces * sizeof(FuseItem));
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->desc_dev, b->desc_bytes * kSlots);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->desc_host, b->desc_bytes * kSlots);
   for (int i = 0; i < kSlots && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&b->ev[i], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->capture_stream, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join_ev, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     release(b);
     return map_record_error("em_batch_create", e);
@@ -660,31 +508,21 @@ int em_batch_autotune(em_batch* b, em_map* const* maps, const em_cloud* clouds, 
   em_tuning best = b->tune;
   float best_ms = 0.f;
   rc = time_one(best, &best_ms);
-  const int ray_c[] = {1, 2, 4, 8, 16};
-  const int chunk_c[] = {256, 512, 256, 512, 256};  // fusion block sizes (repeats are skipped)
-  const int big_c[] = {64, 128, 256, 512, 1023};
   const bool any_ray = [&] {
     for (em_map* m : uniq)
       if (map_params(m).ray_step > 0.f) return true;
     return false;
   }();
-  // coordinate descent: ray group, then fusion block size, then the heavy-tile threshold
-  for (int pass = 0; pass < 3 && rc == EM_OK; ++pass) {
-    if (pass == 0 && !any_ray) continue;
-    const int* cand = pass == 0 ? ray_c : pass == 1 ? chunk_c : big_c;
-    for (int i = 0; i < 5 && rc == EM_OK; ++i) {
-      em_tuning t = best;
-      if (pass == 0) t.ray_group = cand[i];
-      if (pass == 1) t.fuse_chunk = cand[i];
-      if (pass == 2) t.big_thresh = cand[i];
-      if (t.ray_group == best.ray_group && t.fuse_chunk == best.fuse_chunk && t.big_thresh == best.big_thresh)
-        continue;
-      float ms = 0.f;
-      rc = time_one(t, &ms);
-      if (rc == EM_OK && ms < best_ms) {
-        best_ms = ms;
-        best = t;
-      }
+  for (int g : {1, 2, 4, 8, 16}) {
+    if (!any_ray || rc != EM_OK) break;
+    em_tuning t = best;
+    t.ray_group = g;
+    if (t.ray_group == best.ray_group) continue;
+    float ms = 0.f;
+    rc = time_one(t, &ms);
+    if (rc == EM_OK && ms < best_ms) {
+      best_ms = ms;
+      best = t;
     }
   }
   cudaStreamSynchronize(s);

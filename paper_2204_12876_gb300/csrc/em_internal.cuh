@@ -10,22 +10,23 @@
 //   points  the clouds of all maps concatenated (per-point kernels, 1D grid);
 //   cells   the cells of all maps concatenated, each map's range padded to a
 //           multiple of kTile cells, so every tile of kTile cells lies in one
-//           map (per-cell kernels, 1D grid over tiles: uneven maps balance).
+//           map (per-cell kernels, 1D grid over tiles: uneven maps balance);
+//   items   logical blocks of 32 x 8 cells, one warp's work in k_cells.
 //
 // Pipeline of one update (Section II-A of the paper: transform, height update
 // and ray casting in the same iteration, then per-cell passes):
-//   k_count    transform + noise variance + cell binning, per-tile record
-//              counts; per cell: ray thresholds of the pre-update map
-//                                                              (Section II-C)
-//   k_ray      visibility ray march against the pre-update map (Section II-E)
-//   k_alloc    one range of the record arrays per tile of 1024 cells; the
-//              fusion's work lists (dense tiles cut into pieces)
-//   k_scatter  records into their tile's range (counting sort by tile)
-//   k_fuse     per work item, one block: the tile's state in shared memory;
-//              per cell: wall rule, Mahalanobis gate, Eq. 1/2 in information
-//              form with exact integer accumulation (Section II-C)
-//   k_clear    remove penetrated cells not written recently   (Section II-E)
-//   k_normals / k_smooth / k_inpaint                          (Section II-A, II-I)
+//   k_pre      only with the wall rule or the drift compensation: points per
+//              cell, and the drift sums                (Section II-C, II-D)
+//   k_cells    only with the ray march or the drift compensation: moves the
+//              estimates by the drift, ray thresholds of the pre-update map and
+//              their largest per block of 8 x 8 cells  (Section II-D, II-E)
+//   k_points   per point: transform, noise variance, cell, wall rule and
+//              Mahalanobis gate against the pre-update map, exact integer sums
+//              into the cell's accumulator (Section II-C); then its ray, marched
+//              against the pre-update thresholds       (Section II-E)
+//   k_write    per cell: Eq. 1/2 in information form from the sums; removal of
+//              penetrated cells not written recently   (Section II-C, II-E, II-F)
+//   k_normals / k_smooth / k_inpaint                   (Section II-A, II-I)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -54,54 +55,34 @@ struct MapCtl {
   int32_t err;         // first device-side error code of this map (sticky until read)
   float drift_last;    // height error added by the last drift compensation
   int32_t pad[2];
-  // drift-compensation sums, one slot per update parity: update t accumulates
-  // into slot t & 1 (k_count) and reads it (k_drift); k_count of update t clears
-  // slot (t + 1) & 1, last read by update t - 1, which has completed
-  long long drift_h[2];           // sum of the errors' fixed-point high parts
-  unsigned long long drift_l[2];  // ... and low parts (value h 2^27 + l, 2^-44 m units)
-  unsigned long long drift_n[2];  // points in the sum
+  // drift-compensation sums (k_pre; read by k_cells, zero between updates)
+  long long drift_h;           // sum of the errors' fixed-point high parts
+  unsigned long long drift_l;  // ... and low parts (value h 2^27 + l, 2^-44 m units)
+  unsigned long long drift_n;  // points in the sum
 };
 
-// per-batch device control block (reset by k_count and k_alloc)
+// per-batch device control block (zero between updates)
 struct BatchCtl {
-  int32_t rec_total;         // records of this update (all maps)
-  int32_t fuse_next;         // work counter of the fusion: pieces, heavy tiles, then light tiles
-  int32_t n_split;           // tiles split into pieces (one accumulator slot each)
-  int32_t n_pieces;          // entries of the three work lists of the fusion
-  int32_t n_heavy;
-  int32_t n_light;
-  int32_t ray_next;          // work counter of the ray march: runs of kRayRun 32-point batches
-  int32_t pad;
-  // grid barrier of the persistent kernel (k_persist.cu): block tickets, blocks
-  // done, and the abort flag of a barrier wait that ran out; zero between launches
-  unsigned long long bar_ticket;
+  int32_t next;              // work counter of k_points: runs of at most kRayRun 32-point batches
+  // grid barrier of the persistent kernel (k_persist.cu): blocks done, the abort
+  // flag of a barrier wait that ran out, and block tickets
   int32_t bar_done;
   int32_t bar_abort;
+  int32_t pad;
+  unsigned long long bar_ticket;
 };
 
-// A tile with more than heavy_thresh records is split, while accumulator
-// slots last, into pieces of at most heavy_thresh records, fused by different
-// blocks: each adds its exact sums to the tile's slot (kSplitWords 64-bit words
-// per cell) and the last piece to finish writes the cells.
-constexpr int kMaxSplit = 512;       // accumulator slots at most
-constexpr int kSplitWords = 5;       // per cell: weight sum (high, low), term sum (high, low), counts
-
-// One work item of the fusion, written by k_alloc: a non-empty tile (whole) or
-// a piece of a split tile.  The tile's records are [r0, r1); the item fuses
-// [q0, q1) of them (the whole range unless it is a piece).
-struct FuseItem {
-  int32_t tile, map;                 // tile of the batch cell space, and the map it lies in
-  int32_t r0, r1, q0, q1;
-  int32_t slot, np;                  // accumulator slot and pieces of a split tile; -1 and 1 otherwise
+// Accumulator of one cell: the exact fixed-point sums of its accepted points'
+// weights and weighted heights (value h 2^27 + l each), one 32-byte sector, so
+// the four words of a run of points go to L2 as one sector's reductions.  Zero
+// between updates.  kAccTouched in wl: a point was accepted whose weight is
+// zero in fixed point (the low parts' sum stays below 2^58).
+struct __align__(32) CellAcc {
+  unsigned long long wh, wl, th, tl;
 };
-static_assert(sizeof(FuseItem) == 32, "work items are read as two 16-byte words");
+constexpr unsigned long long kAccTouched = 1ull << 63;
 
-// Records: one per in-map point, grouped by tile of kTile cells of the batch
-// cell space (a tile lies in one map: map cell ranges are padded to whole
-// tiles).  Structure of arrays: z (map frame), sigma_p^2, and the cell's index
-// within its tile.  Tile t's records fill [tile_base[t], tile_base[t + 1]).
-constexpr int kMinHeavy = 32;        // tuning bounds of the heavy-tile threshold (x 16 records)
-constexpr int kMaxHeavy = 1023;
+constexpr int kItemW = 32, kItemH = 8;  // k_cells: logical cells per warp item
 
 // device-side error word value for a failed internal consistency check (EM_ERR_CUDA)
 constexpr int32_t kErrInternal = -3;
@@ -126,7 +107,12 @@ struct MapDev {
   float* thr;       // per LOGICAL cell [iy][ix]: h - sqrt(var_eff) of the pre-update map, -inf if empty
   float* cthr;      // per coarse block [by][bx] (CW x CH of them): the largest thr of its cells
   MapCtl* ctl;
-  int64_t cbegin;   // this map's first block in the batch's coarse space (maps with the ray march)
+  CellAcc* acc;     // per physical cell
+  uint32_t* rej;    // rejected points per physical cell, zero between updates
+  uint32_t* cnt;    // wall rule: points per physical cell, zero between updates; null without the rule
+  uint8_t* touched; // per tile of kTile cells: some point of this update fell into it
+  int64_t ibegin;   // this map's first item in the batch's item space (maps with the ray march or drift)
+  int32_t IW, IH;   // items per row and column; 0 x 0 without the ray march and the drift compensation
   int32_t CW, CH;   // coarse blocks per row and column; 0 x 0 without the ray march
   int64_t cell_begin;  // this map's first cell in the batch cell space (multiple of kTile)
   int32_t W, H, ox, oy;
@@ -158,43 +144,24 @@ struct BatchDev {
   int32_t n_maps, n_clouds;
   int64_t n_points;
   int64_t n_cells;     // padded size of the cell space
-  int64_t n_coarse;    // blocks of the coarse grids of all maps
+  int64_t n_items;     // k_cells items of all maps
   const MapDev* maps;
   const CloudDev* clouds;
-  // records grouped by tile (layout above); capacity: the points of the batch
-  float* rz;
-  float* rv;
-  uint16_t* rc;
-  int32_t* idx_sorted; // original point index per record (trace only, else null)
   int32_t* tr_ix;      // trace (null unless EM_F_TRACE)
   int32_t* tr_iy;
   uint8_t* tr_status;
   BatchCtl* ctl;
-  // per tile of the cell space (n_cells / kTile tiles): the records counted by
-  // k_count (zero between updates), their first record (k_alloc; one more
-  // entry holds the total), k_scatter's claims (zeroed by k_alloc), and the
-  // map of every non-empty tile (k_count)
-  int32_t* tile_cnt;
-  int32_t* tile_base;
-  int32_t* tile_cur;
-  int32_t* tile_map;
-  // the fusion's work lists (k_alloc): pieces of split tiles (max_pieces
-  // entries), tiles with more than heavy_thresh records fused whole when the
-  // slots ran out, and the other non-empty tiles (one entry per tile each)
-  FuseItem* pieces;
-  FuseItem* heavy;
-  FuseItem* light;
-  // split tiles: per slot kSplitWords x kTile accumulator words and a count of
-  // finished pieces, both zero between updates
-  unsigned long long* split_acc;
-  int32_t* split_done;
-  int32_t split_slots; // 0: no tile is split
-  int32_t max_pieces;
-  int32_t heavy_thresh;
-  int32_t fuse_threads;  // threads per fusion block: 256 or 512
-  uint32_t passes;       // kPass* bits: optional passes some map of the batch needs
+  uint32_t passes;     // kPass* bits: optional passes some map of the batch needs
 };
-enum : uint32_t { kPassRay = 1u, kPassOverlap = 2u };
+enum : uint32_t { kPassRay = 1u, kPassPre = 2u, kPassCells = 4u };
+
+// The coarse grid and the items of k_cells of a map of W x H cells.
+inline void set_item_grid(MapDev& d, int32_t W, int32_t H, bool ray, bool drift) {
+  d.CW = ray ? coarse_dim(W) : 0;
+  d.CH = ray ? coarse_dim(H) : 0;
+  d.IW = ray || drift ? (W + kItemW - 1) / kItemW : 0;
+  d.IH = ray || drift ? (H + kItemH - 1) / kItemH : 0;
+}
 
 inline int64_t pad_tile(int64_t cells) { return (cells + kTile - 1) / kTile * kTile; }
 // The kernels read points and layers as 4-byte words: a buffer that does not
@@ -204,57 +171,20 @@ inline bool word_aligned(const void* p) { return (reinterpret_cast<uintptr_t>(p)
 // number of SMs of the current device (cached)
 int sm_count();
 
-// Launch ray(stream) beside rest() (which launches on s) and join both before
-// the next launch on s: the ray work goes to the side stream between two
-// events.  While s is being captured into a graph the two run in order on s
-// (a capture never spans a second stream, and nothing edits a capture while
-// it runs; em_batch.cu rearranges its own finished graphs instead).
-template <class Ray, class Rest>
-cudaError_t launch_beside(cudaStream_t s, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, Ray ray,
-                          Rest rest) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  cudaError_t e = cudaStreamIsCapturing(s, &cs);
-  if (e != cudaSuccess) return e;
-  if (cs != cudaStreamCaptureStatusNone || !side) {
-    e = ray(s);
-    return e == cudaSuccess ? rest() : e;
-  }
-  e = cudaEventRecord(fork, s);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(side, fork, 0);
-  if (e != cudaSuccess) return e;
-  e = ray(side);
-  // the join is made whatever happened since the fork
-  cudaError_t je = cudaEventRecord(join, side);
-  if (e == cudaSuccess) e = rest();
-  if (je == cudaSuccess) je = cudaStreamWaitEvent(s, join, 0);
-  return e == cudaSuccess ? je : e;
-}
-
-// The kernels a captured sequence is rearranged by (em_batch.cu).
-const void* coarse_kernel();
-const void* alloc_kernel();
-const void* clear_kernel();
-bool is_fuse_kernel(const void* f);
-
 // ---- launchers (each returns cudaGetLastError() of its launches)
 // ext: some map of the batch uses the exclusion area or the upper-bound layer
-cudaError_t launch_bin(const BatchDev* b, int64_t n_points, int64_t n_cells, bool ext, cudaStream_t s);
-cudaError_t launch_drift(const BatchDev* b, int64_t n_points, int64_t n_cells, bool ext, cudaStream_t s);
-// the coarse threshold grids, then the march (group: samples per chunk and lanes per marched chunk)
-cudaError_t launch_ray(const BatchDev* b, int64_t n_points, int64_t n_cells, int group, bool ext, cudaStream_t s);
-cudaError_t launch_alloc(const BatchDev* b, int64_t n_cells, cudaStream_t s);
-cudaError_t launch_scatter(const BatchDev* b, int64_t n_points, bool ext, cudaStream_t s);
-cudaError_t launch_fuse(const BatchDev* b, int64_t n_cells, int threads, cudaStream_t s);
-cudaError_t launch_clear(const BatchDev* b, int64_t n_cells, cudaStream_t s);
-// The whole update but the drift compensation and the stencils (count, coarse
-// grids, tile ranges, scatter, ray march, fusion, removal, overlap clearance)
-// in one cooperative launch with grid barriers; barrier waits are bounded by
+cudaError_t launch_pre(const BatchDev* b, int64_t n_points, bool ext, cudaStream_t s);
+cudaError_t launch_cells(const BatchDev* b, int64_t n_cells, cudaStream_t s);
+// ray: some map marches rays (group: samples per chunk and lanes per marched chunk)
+cudaError_t launch_points(const BatchDev* b, int64_t n_points, int group, bool ray, bool ext, cudaStream_t s);
+cudaError_t launch_write(const BatchDev* b, int64_t n_cells, cudaStream_t s);
+// The whole update but the drift compensation and the stencils (points per
+// cell, thresholds, points, write) in one cooperative launch with grid barriers; barrier waits are bounded by
 // wait_ms.  cudaErrorNotSupported when the device cannot run it.
 cudaError_t launch_persist(const BatchDev* b, int group, bool ext, int wait_ms, cudaStream_t s);
 // The bounded wait of the persistent kernel on a word that nothing sets: one
 // block, budget wait_us; *timed_out (device memory) becomes 1 when it runs out.
 cudaError_t launch_wait_selftest(const unsigned long long* word, int* timed_out, int wait_us, cudaStream_t s);
-cudaError_t launch_overlap(const BatchDev* b, int64_t n_cells, cudaStream_t s);
 cudaError_t launch_normals(const BatchDev* b, int64_t n_cells, cudaStream_t s);
 cudaError_t launch_smooth(const BatchDev* b, int64_t n_cells, cudaStream_t s);
 cudaError_t launch_inpaint(const BatchDev* b, int64_t n_cells, cudaStream_t s);

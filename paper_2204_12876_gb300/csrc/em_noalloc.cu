@@ -4,14 +4,13 @@
 // that forbids allocation after start-up (an allocation can block on the
 // driver for milliseconds), or a host framework whose own caching allocator
 // has already claimed the device memory.  For them this entry point runs the
-// same kernels as em_update (binning, counting sort by cell, gate + fusion, ray
-// march, removal) on map layers the caller owns, and keeps every piece of
+// same kernels as em_update (binning, gate + fusion, ray march, removal) on map layers the caller owns, and keeps every piece of
 // scratch memory in one file-scope __device__ array of fixed size.  The call's
 // descriptor goes to the device as a kernel parameter (no host buffer, no
 // copy), and its only other preparation is a memset of the scratch.
 //
 // Limits: at most kMaxCells cells per map and kMaxPoints points per update
-// (about 6.1 MiB of scratch, held by every GPU that loads the library until the
+// (about 2.9 MiB of scratch, held by every GPU that loads the library until the
 // process exits).  Every call shares the array and it keeps the last call's
 // contents; the call clears what must start at zero.  Calls whose GPU work
 // overlaps (e.g. on two streams) race on the array.
@@ -45,26 +44,32 @@ struct Desc {
 };
 static_assert(sizeof(Desc) <= 4096, "the descriptor travels as a kernel parameter");
 
-// scratch layout; the part that must start at zero (ctl, marks, tile counts) is contiguous
-constexpr size_t kMaxTiles = ((size_t)kMaxCells + kTile - 1) / kTile;
+// Scratch layout.  The part that must start at zero (control blocks, marks, tile
+// flags and the accumulators of this call's cells) is contiguous, so one memset
+// as long as the map is clears it.
 constexpr size_t kOffDesc = 0;
 constexpr size_t kOffCtl = kOffDesc + up256(sizeof(Desc));
 constexpr size_t kOffBCtl = kOffCtl + up256(sizeof(MapCtl));
-constexpr size_t kOffMark = kOffBCtl + up256(sizeof(BatchCtl));
-constexpr size_t kOffTCnt = kOffMark + up256(((size_t)kMaxCells + 31) / 32 * sizeof(uint32_t));
-constexpr size_t kOffTBase = kOffTCnt + up256((kMaxTiles + 1) * sizeof(int32_t));
-constexpr size_t kOffTCur = kOffTBase + up256((kMaxTiles + 1) * sizeof(int32_t));
-constexpr size_t kOffTMap = kOffTCur + up256((kMaxTiles + 1) * sizeof(int32_t));
-constexpr size_t kOffHeavy = kOffTMap + up256(kMaxTiles * sizeof(int32_t));
-constexpr size_t kOffLight = kOffHeavy + up256(kMaxTiles * sizeof(FuseItem));
-constexpr size_t kOffThr = kOffLight + up256(kMaxTiles * sizeof(FuseItem));
+constexpr size_t kOffZero = kOffBCtl + up256(sizeof(BatchCtl));  // the map's part of the zeroed scratch
+struct Layout {
+  size_t mark, touched, rej, cnt, acc, thr, cthr, end;
+};
+// coarse: blocks of the coarse grid
+constexpr Layout layout(size_t cells, size_t coarse) {
+  Layout o{};
+  o.mark = kOffZero;
+  o.touched = o.mark + up256((cells + 31) / 32 * sizeof(uint32_t));
+  o.rej = o.touched + up256((cells + kTile - 1) / kTile);
+  o.cnt = o.rej + up256(cells * sizeof(uint32_t));
+  o.acc = o.cnt + up256(cells * sizeof(uint32_t));
+  o.thr = o.acc + up256(cells * sizeof(CellAcc));  // end of the zeroed part
+  o.cthr = o.thr + up256(cells * sizeof(float));
+  o.end = o.cthr + up256(coarse * sizeof(float));
+  return o;
+}
 // coarse blocks of a map of at most kMaxCells cells: (W/8 + 1)(H/8 + 1) <= kMaxCells/64 + (W + H)/8 + 1
 constexpr size_t kMaxCoarse = (size_t)kMaxCells / 64 + ((size_t)kMaxCells + 1) / 8 + 2;
-constexpr size_t kOffCThr = kOffThr + up256((size_t)kMaxCells * sizeof(float));
-constexpr size_t kOffRz = kOffCThr + up256(kMaxCoarse * sizeof(float));
-constexpr size_t kOffRv = kOffRz + up256((size_t)kMaxPoints * sizeof(float));
-constexpr size_t kOffRc = kOffRv + up256((size_t)kMaxPoints * sizeof(float));
-constexpr size_t kScratchBytes = kOffRc + up256((size_t)kMaxPoints * sizeof(uint16_t));
+constexpr size_t kScratchBytes = layout(kMaxCells, kMaxCoarse).end;
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
@@ -165,13 +170,15 @@ extern "C" int em_update_noalloc(const em_params* params, int64_t shift_x, int64
   m->nx = const_cast<float*>(nx);
   m->ny = const_cast<float*>(ny);
   m->nz = const_cast<float*>(nz);
-  m->mark = reinterpret_cast<uint32_t*>(base + kOffMark);
-  m->thr = reinterpret_cast<float*>(base + kOffThr);
-  if (params->ray_step > 0.f) {
-    m->cthr = reinterpret_cast<float*>(base + kOffCThr);
-    m->CW = coarse_dim(W);
-    m->CH = coarse_dim(H);
-  }
+  set_item_grid(*m, W, H, params->ray_step > 0.f, params->drift_flatness > 0.f);
+  const Layout lay = layout((size_t)ncell, (size_t)m->CW * m->CH);
+  m->mark = reinterpret_cast<uint32_t*>(base + lay.mark);
+  m->touched = base + lay.touched;
+  m->rej = reinterpret_cast<uint32_t*>(base + lay.rej);
+  if (params->wall_num_thresh > 0) m->cnt = reinterpret_cast<uint32_t*>(base + lay.cnt);
+  m->acc = reinterpret_cast<CellAcc*>(base + lay.acc);
+  m->thr = reinterpret_cast<float*>(base + lay.thr);
+  m->cthr = reinterpret_cast<float*>(base + lay.cthr);
   m->ctl = reinterpret_cast<MapCtl*>(base + kOffCtl);
   m->cell_begin = 0;
   m->z_ref = clouds[0].pose[11];
@@ -212,40 +219,23 @@ extern "C" int em_update_noalloc(const em_params* params, int64_t shift_x, int64
   b->n_points = total;
   b->maps = reinterpret_cast<const MapDev*>(base + kOffDesc + offsetof(Desc, m));
   b->clouds = reinterpret_cast<const CloudDev*>(base + kOffDesc + offsetof(Desc, c));
-  b->rz = reinterpret_cast<float*>(base + kOffRz);
-  b->rv = reinterpret_cast<float*>(base + kOffRv);
-  b->rc = reinterpret_cast<uint16_t*>(base + kOffRc);
-  b->tile_cnt = reinterpret_cast<int32_t*>(base + kOffTCnt);
-  b->tile_base = reinterpret_cast<int32_t*>(base + kOffTBase);
-  b->tile_cur = reinterpret_cast<int32_t*>(base + kOffTCur);
-  b->tile_map = reinterpret_cast<int32_t*>(base + kOffTMap);
-  b->heavy = reinterpret_cast<FuseItem*>(base + kOffHeavy);
-  b->light = reinterpret_cast<FuseItem*>(base + kOffLight);
   b->n_cells = pad_tile(ncell);
-  b->n_coarse = (int64_t)m->CW * m->CH;
+  b->n_items = (int64_t)m->IW * m->IH;
   b->ctl = reinterpret_cast<BatchCtl*>(base + kOffBCtl);
-  b->heavy_thresh = 4096;
-  b->split_slots = 0;  // no tile is split: heavy tiles are fused whole
-  b->fuse_threads = 256;
 
   const BatchDev* bd = reinterpret_cast<const BatchDev*>(base + kOffDesc + offsetof(Desc, b));
   k_put_desc<<<1, 128, 0, s>>>(desc);
   rc = na_status(cudaGetLastError(), "k_put_desc");
   if (rc) return rc;
-  // counters, marks and per-tile counts start at zero
-  rc = na_status(cudaMemsetAsync(base + kOffCtl, 0, kOffTBase - kOffCtl, s), "cudaMemsetAsync");
+  rc = na_status(cudaMemsetAsync(base + kOffCtl, 0, lay.thr - kOffCtl, s), "cudaMemsetAsync");
   if (rc) return rc;
   const int64_t cells = pad_tile(ncell);
   const bool ext = params->excl_d > 0.f;  // no upper-bound layer here
-  cudaError_t e = launch_bin(bd, total, cells, ext, s);
-  if (e == cudaSuccess && params->drift_flatness > 0.f) e = launch_drift(bd, total, cells, ext, s);
-  if (total > 0) {
-    if (e == cudaSuccess && params->ray_step > 0.f) e = launch_ray(bd, total, cells, 8, ext, s);
-    if (e == cudaSuccess) e = launch_alloc(bd, cells, s);
-    if (e == cudaSuccess) e = launch_scatter(bd, total, ext, s);
-    if (e == cudaSuccess) e = launch_fuse(bd, cells, 256, s);
-  }
-  if (e == cudaSuccess) e = launch_clear(bd, cells, s);
-  if (e == cudaSuccess && params->overlap_dz > 0.f) e = launch_overlap(bd, cells, s);
+  const bool ray = params->ray_step > 0.f, drift = params->drift_flatness > 0.f;
+  cudaError_t e = cudaSuccess;
+  if (drift || m->cnt) e = launch_pre(bd, total, ext, s);
+  if (e == cudaSuccess && (ray || drift)) e = launch_cells(bd, cells, s);
+  if (e == cudaSuccess) e = launch_points(bd, total, 8, ray, ext, s);
+  if (e == cudaSuccess) e = launch_write(bd, cells, s);
   return na_status(e, "em_update_noalloc launch");
 }

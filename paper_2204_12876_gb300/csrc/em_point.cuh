@@ -1,8 +1,9 @@
-// em_point.cuh -- per-point arithmetic shared by the binning and ray kernels.
+// em_point.cuh -- per-point arithmetic shared by the kernels over the points.
 //
-// Both kernels must find the same cell for a point (the ray march skips the
-// point's own cell), so the arithmetic is written with explicit rounding
-// intrinsics: no contraction choice of the compiler can make the two differ.
+// Every kernel must find the same cell for a point (the wall rule counts the
+// points the fusion gates, the ray march skips the point's own cell), so the
+// arithmetic is written with explicit rounding intrinsics: no contraction
+// choice of the compiler can make two of them differ.
 #pragma once
 
 #include "em_internal.cuh"
@@ -108,55 +109,6 @@ __device__ __forceinline__ float fixed_to_float(__int128 t) {
                             __fmul_rn((float)(uint32_t)(mid >> 32), 2.44140625e-4f)));
   }
   return neg ? -v : v;
-}
-
-// Per-thread statistics counters of one map.  They are flushed with one atomic
-// per block and counter when the whole block saw a single map (the usual
-// case), else per thread: many threads adding to one address serialise on a
-// single L2 slice.
-struct MapCounters {
-  int map = -1;
-  unsigned long long v[4] = {0, 0, 0, 0};
-};
-
-// shared memory of flush_counters (the caller's)
-struct FlushSmem {
-  int map;
-  unsigned long long sum[4];
-};
-
-__device__ __forceinline__ void flush_counters(const BatchDev& b, MapCounters& mc, const int* idx, int n,
-                                               FlushSmem& fs) {
-  if (threadIdx.x == 0) fs.map = mc.map;
-  if (threadIdx.x < 4) fs.sum[threadIdx.x] = 0;
-  __syncthreads();
-  const bool uniform = __syncthreads_and(mc.map == fs.map || mc.map < 0);
-  if (uniform) {
-    for (int k = 0; k < n; ++k) {
-      unsigned long long v = mc.v[k];
-      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if ((threadIdx.x & 31) == 0 && v) atomicAdd(&fs.sum[k], v);
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < n && fs.map >= 0 && fs.sum[threadIdx.x])
-      atomicAdd(&b.maps[fs.map].ctl->stats[idx[threadIdx.x]], fs.sum[threadIdx.x]);
-    __syncthreads();  // the shared sums are free again
-  } else if (mc.map >= 0) {
-    for (int k = 0; k < n; ++k)
-      if (mc.v[k]) atomicAdd(&b.maps[mc.map].ctl->stats[idx[k]], mc.v[k]);
-  }
-}
-
-__device__ __forceinline__ void add_counter(const BatchDev& b, MapCounters& mc, int map, const int* idx, int n,
-                                            const unsigned long long* inc) {
-  if (map != mc.map) {
-    if (mc.map >= 0)
-      for (int k = 0; k < n; ++k)
-        if (mc.v[k]) atomicAdd(&b.maps[mc.map].ctl->stats[idx[k]], mc.v[k]);
-    mc.map = map;
-    for (int k = 0; k < n; ++k) mc.v[k] = 0;
-  }
-  for (int k = 0; k < n; ++k) mc.v[k] += inc[k];
 }
 
 // Runs of equal keys in consecutive lanes (sensor order puts neighbouring

@@ -62,8 +62,7 @@ struct Flight {
   int64_t bytes = 0;
 };
 
-constexpr int64_t kRecordBytes = EM_SERVE_RECORD_BYTES;  // one grouped record per point
-static_assert(kRecordBytes == sizeof(float4), "record size");
+constexpr int64_t kRecordBytes = EM_SERVE_RECORD_BYTES;  // admission accounting per point
 
 }  // namespace
 

@@ -1,0 +1,50 @@
+// k_cell.cu -- the kernels over the cells (cell_pass.cuh), launched before and
+// after the points.
+//
+// Eq. 1 and Eq. 2 for all accepted points of a cell at once, in information form:
+//   Lambda = 1 / (sigma_m^2 + n_rej v_out) + sum_i 1/sigma_p,i^2
+//   h'     = h_ref + sum_i (z_i - h_ref) / sigma_p,i^2 / Lambda,   sigma_m^2' = 1 / Lambda
+// with h_ref = h for a valid cell (an empty cell has 1/sigma_m^2 = 0 and h_ref =
+// the map's reference height z_ref).  Applying Eq. 1/2 point after point gives
+// the same result in exact arithmetic.
+//
+// The two sums are exact: every float32 term is a fixed-point integer with 44
+// fractional bits (kept as h 2^27 + l) and the integers are added.  Integer
+// addition is associative, so the result is the same for every order of the
+// points and every split of the work, bit for bit (no float atomics).
+#include "cell_pass.cuh"
+
+namespace em {
+
+// Latency-bound on one map (9 us cold for 250 x 250 cells: two dependent loads
+// and the square roots), DRAM-bound on many (31 us for the 64-map batch's 6.8 M
+// cells).  It takes the place of a threshold pass in the point kernel and a
+// one-thread-per-block coarse kernel (12 us alone on one map).
+__global__ void __launch_bounds__(kCellThreads) k_cells(const BatchDev* __restrict__ bp) {
+  cells_pass(*bp, own_grid());
+}
+
+// DRAM-bound on many maps (427 MB in 135 us for the 64-map batch: 36 bytes of
+// sums and 12 of state per touched cell, read and written); 8-12 us cold on one.
+__global__ void __launch_bounds__(kCellThreads) k_write(const BatchDev* __restrict__ bp) {
+  write_pass(*bp, own_grid());
+}
+
+// n_cells bounds the items: an item has at most kItemW x kItemH cells, a map's
+// last row and column of items may be partial
+cudaError_t launch_cells(const BatchDev* b, int64_t n_cells, cudaStream_t s) {
+  constexpr int kThreads = 128;  // small maps reach more SMs
+  const int64_t blocks = n_cells / (kItemW * kItemH * (kThreads / 32)) + 1;
+  const int64_t cap = (int64_t)sm_count() * 16;
+  k_cells<<<(int)(blocks < cap ? blocks : cap), kThreads, 0, s>>>(b);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_write(const BatchDev* b, int64_t n_cells, cudaStream_t s) {
+  const int64_t tiles = n_cells / kTile;  // a block per tile
+  const int64_t cap = (int64_t)sm_count() * 8;
+  k_write<<<(int)(tiles < 1 ? 1 : tiles < cap ? tiles : cap), kCellThreads, 0, s>>>(b);
+  return cudaGetLastError();
+}
+
+}  // namespace em

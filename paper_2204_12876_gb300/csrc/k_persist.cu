@@ -4,12 +4,9 @@
 // to II-E of the paper) in one cooperative kernel whose blocks are all
 // resident, with a grid-wide barrier wherever a pass needs the one before:
 //
-//   count: transform + bin + per-tile counts, then the ray thresholds
-//   | tile ranges and the fusion's work lists (one block, sort_pass.cuh) and
-//   |   the coarse threshold grids (every other block)
-//   | scatter of the records, then the ray march (independent of each other)
-//   | fusion: blocks take tiles and pieces from the work queue
-//   | removal of marked cells (| overlap clearance)
+//   points per cell (maps with the wall rule), thresholds and coarse grids
+//   | points: gate, sums, ray march (blocks take runs from the work counter)
+//   | new state of every cell, removal of marked cells, overlap clearance
 //
 // The stencils (normals, smoothing, in-painting) follow as their own kernels.
 // The passes share one shared-memory buffer; each one ends with a block
@@ -20,20 +17,17 @@
 // counter back to zero.  Every wait is bounded by a clock64 budget: a wait
 // that runs out raises the abort flag, writes EM_ERR_TIMEOUT into the maps'
 // error words, and every block leaves at its next barrier.
-#include "sort_pass.cuh"
-#include "ray_pass.cuh"
-#include "fuse_pass.cuh"
+#include "cell_pass.cuh"
+#include "point_pass.cuh"
 
 namespace em {
 
 constexpr int kPersistThreads = 256;
-static_assert(kPersistThreads == kPointThreads && kPersistThreads == kRayThreads &&
-                  kPersistThreads == kClearThreads,
-              "the passes share one block size");
+static_assert(kPersistThreads == kPointThreads && kPersistThreads == kCellThreads, "the passes share one block size");
 
 constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
 // the passes run one after another and share one shared-memory buffer
-constexpr size_t kPersistSmem = cmax(cmax(sizeof(TileSmem), sizeof(RaySmem)), cmax(sizeof(PointSmem), sizeof(AllocSmem)));
+constexpr size_t kPersistSmem = cmax(sizeof(PointsSmem<true>), sizeof(PreSmem));
 
 // Wait until *word >= target, or until `abort` is raised, for at most budget
 // SM clock cycles; true when the word got there.
@@ -73,30 +67,17 @@ __global__ void __launch_bounds__(kPersistThreads, 4) k_persist(const BatchDev* 
   const BatchDev& b = *bp;
   const int nb = gridDim.x, bid = blockIdx.x;
   const Grid all{bid, nb};
-  const bool ray = (b.passes & kPassRay) != 0;
-  count_pass<kExt>(b, all, *reinterpret_cast<PointSmem*>(sm));
-  bool ok = grid_barrier(b, nb, budget, s_ok);
-  if (ok) {
-    if (bid == 0) alloc_pass<kPersistThreads>(b, *reinterpret_cast<AllocSmem*>(sm));
-    else if (ray) coarse_pass(b, Grid{bid - 1, nb - 1});
+  bool ok = true;
+  if (b.passes & (kPassPre | kPassCells)) {
+    if (b.passes & kPassPre) pre_pass<kExt>(b, all, *reinterpret_cast<PreSmem*>(sm));
+    if (b.passes & kPassCells) cells_pass(b, all);
     ok = grid_barrier(b, nb, budget, s_ok);
   }
   if (ok) {
-    scatter_pass<kExt>(b, all, *reinterpret_cast<PointSmem*>(sm));
-    if (ray) ray_pass<G, kExt>(b, all, *reinterpret_cast<RaySmem*>(sm));
+    points_pass<G, true, kExt>(b, all, *reinterpret_cast<PointsSmem<true>*>(sm));
     ok = grid_barrier(b, nb, budget, s_ok);
   }
-  if (ok) {
-    fuse_pass<kPersistThreads>(b, *reinterpret_cast<TileSmem*>(sm));
-    ok = grid_barrier(b, nb, budget, s_ok);
-  }
-  if (ok) {
-    clear_pass(b, all);
-    if (b.passes & kPassOverlap) {
-      ok = grid_barrier(b, nb, budget, s_ok);
-      if (ok) overlap_pass(b, all);
-    }
-  }
+  if (ok) write_pass(b, all);
   // the last block to leave makes the barrier state ready for the next launch
   __syncthreads();
   if (threadIdx.x == 0) {

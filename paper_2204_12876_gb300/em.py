@@ -25,9 +25,9 @@ LAYER_NORMAL_X, LAYER_NORMAL_Y, LAYER_NORMAL_Z = 8, 16, 32
 LAYER_SMOOTH, LAYER_INPAINT, LAYER_VALID, LAYER_VARIANCE_NOW, LAYER_UPPER = 64, 128, 256, 512, 1024
 PROF_SLOTS = ("count", "ray", "alloc", "scatter", "fuse", "clear", "normals", "smooth", "inpaint", "drift",
               "overlap", "persist")
-KERNEL_NAMES = {"count": "k_count", "ray": "k_ray", "alloc": "k_alloc", "scatter": "k_scatter", "fuse": "k_fuse",
-                "clear": "k_clear", "normals": "k_normals", "smooth": "k_smooth", "inpaint": "k_inpaint",
-                "drift": "k_drift", "overlap": "k_overlap", "persist": "k_persist"}
+KERNEL_NAMES = {"count": "k_cells", "ray": "k_points", "alloc": "(none)", "scatter": "k_pre", "fuse": "k_write",
+                "clear": "(none)", "normals": "k_normals", "smooth": "k_smooth", "inpaint": "k_inpaint",
+                "drift": "(none)", "overlap": "(none)", "persist": "k_persist"}
 LAYER_NAMES = {LAYER_ELEVATION: "h", LAYER_VARIANCE: "var", LAYER_TIME: "t_last", LAYER_NORMAL_X: "nx",
                LAYER_NORMAL_Y: "ny", LAYER_NORMAL_Z: "nz", LAYER_SMOOTH: "smooth", LAYER_INPAINT: "inpaint",
                LAYER_VALID: "valid", LAYER_VARIANCE_NOW: "var_now", LAYER_UPPER: "upper"}

@@ -1,0 +1,109 @@
+"""The points' way into their cells (k_points, k_write): runs of equal cells in
+consecutive lanes, batches of 32 points across clouds and maps, map sizes
+around the kernels' tiles, and weights that vanish in fixed point.
+
+Expected values are the per-cell inverse-variance means in float64 (Eq. 1/2
+over an empty map, Section II-C), with the repository's tolerances for the
+float32 path: heights 1e-5 m, variances 1e-4 relative."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+R = 0.04
+POSE = np.array([1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1, 0.0], np.float32)
+
+
+@pytest.fixture(scope="module")
+def em():
+    from paper_2204_12876_gb300 import build
+    build.build()
+    from paper_2204_12876_gb300 import em as mod
+    return mod
+
+
+def runs_cloud(rng, W, H, n):
+    """n points in runs of 1, 2, 31, 32, 33 and 70 points of one cell, well inside their cells."""
+    cells = []
+    lengths = [1, 2, 31, 32, 33, 70, 5]
+    while len(cells) < n:
+        cells += [(int(rng.integers(W)), int(rng.integers(H)))] * lengths[len(cells) % len(lengths)]
+    c = np.array(cells[:n])
+    xy = (c + 0.5 + rng.uniform(-0.3, 0.3, (n, 2)) - np.array([W, H]) / 2) * R
+    p = np.concatenate([xy, rng.uniform(-0.8, -0.3, (n, 1))], axis=1).astype(np.float32)
+    return p, c
+
+
+def expected(parts, W, H, a0, a2):
+    """Per-cell (h, var) of points over an empty map, float64."""
+    sw, swz = np.zeros((H, W)), np.zeros((H, W))
+    for p, c in parts:
+        p = p.astype(np.float64)
+        w = 1.0 / (a0 + a2 * (p * p).sum(axis=1)) ** 2
+        np.add.at(sw, (c[:, 1], c[:, 0]), w)
+        np.add.at(swz, (c[:, 1], c[:, 0]), w * p[:, 2])
+    with np.errstate(invalid="ignore", divide="ignore"):
+        return swz / sw, 1.0 / sw
+
+
+def check(state, parts, W, H, a0=0.005, a2=0.002):
+    h, var = expected(parts, W, H, a0, a2)
+    hit = np.isfinite(h)
+    assert np.array_equal(np.isfinite(state["var"]), hit)
+    assert np.all(np.abs(state["h"][hit] - h[hit]) <= 1e-5)
+    assert np.all(np.abs(state["var"][hit] / var[hit] - 1.0) <= 1e-4)
+
+
+@pytest.mark.parametrize("W, H, n", [(1, 1, 1), (1, 1, 100), (31, 33, 31), (32, 32, 33), (33, 31, 1023),
+                                     (1025, 1, 2049), (64, 48, 20001)])
+@pytest.mark.parametrize("ray", [False, True])
+def test_runs_and_map_sizes(em, W, H, n, ray):
+    rng = np.random.default_rng(W * 7919 + n)
+    m = em.Map(em.Params(width=W, height=H, resolution=R, noise_a0=0.005, noise_a2=0.002,
+                         ray_step=R if ray else 0.0))
+    p, c = runs_cloud(rng, W, H, n)
+    m.update(torch.from_numpy(p).cuda(), POSE)
+    check(m.state(), [(p, c)], W, H)
+    st = m.stats()
+    assert st["points_valid"] == st["points_in_map"] == st["points_accepted"] == n and st["points_rejected"] == 0
+    assert st["cells_updated"] == len(np.unique(c[:, 1] * W + c[:, 0])) and st["updates"] == 1
+    m.close()
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+def test_batches_of_points_across_clouds_and_maps(em, persistent):
+    """Clouds of 1 to 97 points: most 32-point batches hold several clouds, many several maps."""
+    rng = np.random.default_rng(3)
+    sizes = [(20, 13), (1, 1), (40, 40), (7, 90)]
+    maps = [em.Map(em.Params(width=W, height=H, resolution=R, noise_a0=0.005, noise_a2=0.002, ray_step=R))
+            for W, H in sizes]
+    pairs, parts = [], [[] for _ in sizes]
+    for n in (1, 5, 31, 97, 64, 3, 17):
+        for j, (W, H) in enumerate(sizes):
+            p, c = runs_cloud(rng, W, H, n)
+            parts[j].append((p, c))
+            pairs.append((maps[j], torch.from_numpy(p).cuda(), POSE))
+    batch = em.Batch(max_maps=4, max_clouds=len(pairs), max_points=4096, max_cells=1600, persistent=persistent)
+    batch.update(pairs)
+    for j, (W, H) in enumerate(sizes):
+        maps[j].sync()
+        check(maps[j].state(), parts[j], W, H)
+        assert maps[j].stats()["points_accepted"] == sum(len(p) for p, _ in parts[j])
+    batch.close()
+
+
+def test_weights_below_fixed_point(em):
+    """A point whose weight is below 2^-44 still counts as accepted: a valid cell
+    keeps its height, its variance (to rounding) and gets the update's index."""
+    m = em.Map(em.Params(width=2, height=1, resolution=R, noise_a0=1e8))
+    h = np.array([[0.25, np.nan]], np.float32)
+    var = np.array([[0.01, np.inf]], np.float32)
+    m.set_state(h=h, var=var, t_last=np.zeros((1, 2), np.float32), t_now=4)
+    p = np.array([[-0.02, 0.0, 1.0]] * 40, np.float32)
+    m.update(torch.from_numpy(p).cuda(), POSE)
+    s = m.state()
+    assert s["h"][0, 0] == np.float32(0.25) and abs(s["var"][0, 0] / 0.01 - 1) < 1e-6
+    assert s["t_last"][0, 0] == 5 and s["t_last"][0, 1] == 0
+    assert m.stats()["points_accepted"] == 40 and m.stats()["cells_updated"] == 1
+    m.close()
