@@ -249,7 +249,7 @@ int em_profile_read(em_map* map, double* ms, int64_t* launches);
  * sequence of kernels over all of them -- the per-point and per-cell work of
  * every map shares each launch, so small updates no longer pay a launch
  * sequence each.  The arithmetic per map is exactly em_update's.
- * A batch object owns a ring of device descriptors and -- with EM_BATCH_GRAPH -- one captured CUDA graph
+ * A batch object owns a ring of device descriptors and -- with EM_BATCH_GRAPH -- one CUDA graph
  * per descriptor slot, replayed with a single cudaGraphLaunch per batch (grids
  * are sized from the capacities; actual sizes are read from the descriptor). */
 typedef struct em_batch em_batch;

@@ -317,6 +317,18 @@ uint32_t map_flags(const em_map* m) { return m->p.flags; }
 int32_t map_cells(const em_map* m) { return m->p.width * m->p.height; }
 const em_params& map_params(const em_map* m) { return m->p; }
 
+UpdateKind params_kind(const em_params& p, int32_t ray_group) {
+  UpdateKind k{};
+  k.ray_group = ray_group;
+  k.ray = p.ray_step > 0.f;
+  k.drift = p.drift_flatness > 0.f;
+  k.wall = p.wall_num_thresh > 0;
+  k.ext = p.excl_d > 0.f || (p.flags & EM_F_UPPER);
+  k.stencils = p.flags & (EM_F_NORMALS | EM_F_SMOOTH | EM_F_MEDIAN | EM_F_GAUSS | EM_F_INPAINT);
+  return k;
+}
+UpdateKind map_kind(const em_map* m, int32_t ray_group) { return params_kind(m->p, ray_group); }
+
 MapDev map_begin_update(em_map* m, int64_t points) {
   m->t_now += 1;
   m->points_in += points;
@@ -486,20 +498,9 @@ static int update_impl(em_map* m, const em_cloud* clouds, int32_t n_clouds, cuda
     return slot;
   }
   const int64_t ncell = pad_tile((int64_t)m->p.width * m->p.height);
-  const bool ext = m->p.excl_d > 0.f || (m->p.flags & EM_F_UPPER);  // kernels with the extended features
-  const bool ray = m->p.ray_step > 0.f, drift = m->p.drift_flatness > 0.f;
-  if (drift || m->p.wall_num_thresh > 0)
-    EM_TRY(timed(m, EM_PROF_SCATTER, s, [&] { return launch_pre(bd, total, ext, s); }), "k_pre");
-  if (ray || drift) EM_TRY(timed(m, EM_PROF_COUNT, s, [&] { return launch_cells(bd, ncell, s); }), "k_cells");
-  if (total > 0)
-    EM_TRY(timed(m, EM_PROF_RAY, s, [&] { return launch_points(bd, total, m->ray_group, ray, ext, s); }), "k_points");
-  EM_TRY(timed(m, EM_PROF_FUSE, s, [&] { return launch_write(bd, ncell, s); }), "k_write");
-  if (m->p.flags & EM_F_NORMALS)
-    EM_TRY(timed(m, EM_PROF_NORMALS, s, [&] { return launch_normals(bd, ncell, s); }), "k_normals");
-  if (m->p.flags & (EM_F_SMOOTH | EM_F_MEDIAN | EM_F_GAUSS))
-    EM_TRY(timed(m, EM_PROF_SMOOTH, s, [&] { return launch_smooth(bd, ncell, s); }), "k_smooth");
-  if (m->p.flags & EM_F_INPAINT)
-    EM_TRY(timed(m, EM_PROF_INPAINT, s, [&] { return launch_inpaint(bd, ncell, s); }), "k_inpaint");
+  const Sequence q = update_sequence(map_kind(m, m->ray_group), total, ncell);
+  for (int i = 0; i < q.n; ++i)
+    EM_TRY(timed(m, q.k[i].slot, s, [&] { return run(q.k[i], bd, s); }), q.k[i].name);
   EM_TRY(cudaEventRecord(m->desc_ev[slot], s), "cudaEventRecord");
   m->last_stream = s;
   m->last_n = total;

@@ -4,8 +4,8 @@
 // device descriptor), so a batch is the same launch sequence as one em_update
 // with more maps in the descriptor: per-point kernels span all clouds of all
 // maps, per-cell kernels walk the tiles of all maps' cells.  With EM_BATCH_GRAPH the
-// sequence is captured once per descriptor slot (grids sized from the batch
-// capacities) and replayed by one cudaGraphLaunch.
+// sequence becomes a graph once per descriptor slot (grids sized from the batch
+// capacities), replayed by one cudaGraphLaunch.
 #include <cuda_runtime.h>
 #include <string.h>
 
@@ -36,20 +36,6 @@ bool tuning_ok(const em_tuning& t) {
          t.big_thresh >= 32 && t.big_thresh <= 1023;
 }
 
-// what a captured graph depends on besides the slot
-struct GraphKey {
-  int32_t ray_group;
-  bool ray;
-  bool drift;
-  bool wall;
-  bool ext;  // some map uses the exclusion area or the upper-bound layer
-  uint32_t stencils;
-  bool operator==(const GraphKey& o) const {
-    return ray_group == o.ray_group && ray == o.ray && drift == o.drift && wall == o.wall && ext == o.ext &&
-           stencils == o.stencils;
-  }
-};
-
 }  // namespace
 
 struct em_batch {
@@ -58,15 +44,15 @@ struct em_batch {
   int64_t max_points = 0;
   uint32_t flags = 0;
   BatchCtl* bctl = nullptr;
+  long long wait_budget = 0;  // SM clock cycles of EM_PERSIST_WAIT_MS
   size_t desc_bytes = 0;
   unsigned char* desc_host = nullptr;
   unsigned char* desc_dev = nullptr;
   cudaEvent_t ev[kSlots] = {};
   int slot = 0;
   em_tuning tune{8, 512, 256};
-  cudaStream_t capture_stream = nullptr;
   cudaGraphExec_t graph[kSlots] = {};
-  GraphKey graph_key[kSlots] = {};
+  UpdateKind graph_kind[kSlots] = {};
   // host scratch for grouping
   std::vector<int> first_of, order, map_of;
   std::vector<em_map*> uniq;
@@ -80,18 +66,6 @@ struct em_batch {
 };
 
 namespace {
-
-// Events around one launch when the batch is profiling (prof may be null).
-template <class F>
-cudaError_t timed(em_batch* prof, int slot, cudaStream_t s, F fn) {
-  if (!prof || !prof->prof) return fn();
-  cudaEventRecord(prof->pev[2 * slot], s);
-  cudaError_t e = fn();
-  cudaEventRecord(prof->pev[2 * slot + 1], s);
-  prof->pused[slot] = true;
-  prof->prof_pending = true;
-  return e;
-}
 
 int prof_collect(em_batch* b) {
   if (!b->prof_pending) return EM_OK;
@@ -108,35 +82,19 @@ int prof_collect(em_batch* b) {
   return EM_OK;
 }
 
-// The kernel sequence of one update over the descriptor at `bd`.
-cudaError_t launch_sequence(em_batch* b, const BatchDev* bd, int64_t grid_points, int64_t grid_cells,
-                            const GraphKey& k, cudaStream_t s, em_batch* prof = nullptr) {
+// The update's kernels on a stream, with events around each when the batch is profiling.
+cudaError_t launch_sequence(em_batch* b, const Sequence& q, const BatchDev* bd, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
-  // EM_BATCH_PERSISTENT: the update's passes in one launch (k_persist.cu), when
-  // the device can run it and no map needs the drift compensation
-  bool persisted = false;
-  if ((b->flags & EM_BATCH_PERSISTENT) && !k.drift) {
-    e = timed(prof, EM_PROF_PERSIST, s, [&] { return launch_persist(bd, k.ray_group, k.ext, EM_PERSIST_WAIT_MS, s); });
-    persisted = e != cudaErrorNotSupported;
-    if (!persisted) {
-      cudaGetLastError();
-      e = cudaSuccess;
+  for (int i = 0; i < q.n && e == cudaSuccess; ++i) {
+    const int slot = q.k[i].slot;
+    if (b->prof) cudaEventRecord(b->pev[2 * slot], s);
+    e = run(q.k[i], bd, s);
+    if (b->prof) {
+      cudaEventRecord(b->pev[2 * slot + 1], s);
+      b->pused[slot] = true;
+      b->prof_pending = true;
     }
   }
-  if (!persisted) {
-    if (k.drift || k.wall) e = timed(prof, EM_PROF_SCATTER, s, [&] { return launch_pre(bd, grid_points, k.ext, s); });
-    if (e == cudaSuccess && (k.ray || k.drift))
-      e = timed(prof, EM_PROF_COUNT, s, [&] { return launch_cells(bd, grid_cells, s); });
-    if (e == cudaSuccess && grid_points > 0)
-      e = timed(prof, EM_PROF_RAY, s, [&] { return launch_points(bd, grid_points, k.ray_group, k.ray, k.ext, s); });
-    if (e == cudaSuccess) e = timed(prof, EM_PROF_FUSE, s, [&] { return launch_write(bd, grid_cells, s); });
-  }
-  if (e == cudaSuccess && (k.stencils & EM_F_NORMALS))
-    e = timed(prof, EM_PROF_NORMALS, s, [&] { return launch_normals(bd, grid_cells, s); });
-  if (e == cudaSuccess && (k.stencils & (EM_F_SMOOTH | EM_F_MEDIAN | EM_F_GAUSS)))
-    e = timed(prof, EM_PROF_SMOOTH, s, [&] { return launch_smooth(bd, grid_cells, s); });
-  if (e == cudaSuccess && (k.stencils & EM_F_INPAINT))
-    e = timed(prof, EM_PROF_INPAINT, s, [&] { return launch_inpaint(bd, grid_cells, s); });
   return e;
 }
 
@@ -146,7 +104,7 @@ struct Prepared {
   int64_t points = 0;
   int32_t n_maps = 0;
   int64_t cells = 0;  // padded size of the cell space
-  GraphKey key{};
+  UpdateKind kind{};
 };
 
 // Group the pairs by map, build the descriptor in slot `slot` and upload it.
@@ -192,7 +150,9 @@ int prepare(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t co
   MapDev* md = reinterpret_cast<MapDev*>(hb + sizeof(BatchDev));
   CloudDev* cd = reinterpret_cast<CloudDev*>(hb + sizeof(BatchDev) + (size_t)b->max_maps * sizeof(MapDev));
   memset(bd, 0, sizeof(BatchDev));
-  GraphKey key{tune.ray_group, false, false, false, false, 0u};
+  UpdateKind kind{};
+  kind.ray_group = tune.ray_group;
+  kind.persistent = (b->flags & EM_BATCH_PERSISTENT) != 0;
   int64_t cells = 0, items = 0;
   for (int u = 0; u < nm; ++u) {
     md[u] = map_begin_update(b->uniq[u], map_pts[u]);
@@ -200,11 +160,12 @@ int prepare(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t co
     cells += pad_tile(map_cells(b->uniq[u]));
     md[u].ibegin = items;
     items += (int64_t)md[u].IW * md[u].IH;
-    key.ray |= md[u].ray_step > 0.f;
-    key.drift |= md[u].drift_flat > 0.f;
-    key.wall |= md[u].cnt != nullptr;
-    key.ext |= md[u].excl_d > 0.f || md[u].upper != nullptr;
-    key.stencils |= map_flags(b->uniq[u]) & (EM_F_NORMALS | EM_F_SMOOTH | EM_F_MEDIAN | EM_F_GAUSS | EM_F_INPAINT);
+    const UpdateKind k = map_kind(b->uniq[u], tune.ray_group);
+    kind.ray |= k.ray;
+    kind.drift |= k.drift;
+    kind.wall |= k.wall;
+    kind.ext |= k.ext;
+    kind.stencils |= k.stencils;
   }
   // clouds ordered by map (stable), so each map's points are contiguous
   int ci = 0;
@@ -239,8 +200,8 @@ int prepare(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t co
   bd->n_cells = cells;
   bd->n_items = items;
   bd->ctl = b->bctl;
-  bd->passes = (key.ray ? kPassRay : 0u) | (key.wall || key.drift ? kPassPre : 0u) |
-               (key.ray || key.drift ? kPassCells : 0u);
+  bd->passes = (kind.wall || kind.drift ? kPassPre : 0u) | (kind.ray || kind.drift ? kPassCells : 0u);
+  bd->wait_budget = b->wait_budget;
   // upload header + maps, and the clouds at their fixed offset
   cudaError_t e = cudaMemcpyAsync(db, hb, sizeof(BatchDev) + (size_t)nm * sizeof(MapDev), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
@@ -255,7 +216,7 @@ int prepare(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t co
   out->points = total;
   out->n_maps = nm;
   out->cells = cells;
-  out->key = key;
+  out->kind = kind;
   return EM_OK;
 }
 
@@ -265,31 +226,20 @@ void finish(em_batch* b, const Prepared& p, cudaStream_t s) {
 }
 
 int run_graph(em_batch* b, const Prepared& p, cudaStream_t s) {
-  if (!b->graph[p.slot] || !(b->graph_key[p.slot] == p.key)) {
+  if (!b->graph[p.slot] || !(b->graph_kind[p.slot] == p.kind)) {
     if (b->graph[p.slot]) {
       cudaGraphExecDestroy(b->graph[p.slot]);
       b->graph[p.slot] = nullptr;
     }
     cudaGraph_t g = nullptr;
-    EB_TRY(cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
-    cudaError_t le = launch_sequence(b, p.bd, b->max_points, (int64_t)b->max_maps * pad_tile(b->max_cells), p.key,
-                                     b->capture_stream);
-    cudaError_t ce = cudaStreamEndCapture(b->capture_stream, &g);
-    if (le != cudaSuccess || ce != cudaSuccess) {
-      // Another thread can break a capture (a device-wide synchronize while it
-      // runs invalidates it).  The sequence then runs without a graph this
-      // time, and the next update of this kind tries the capture again.
-      if (g) cudaGraphDestroy(g);
-      cudaGetLastError();
-      EB_TRY(launch_sequence(b, p.bd, p.points, p.cells, p.key, s), "launch (capture failed)");
-      return EM_OK;
-    }
+    const Sequence q = update_sequence(p.kind, b->max_points, (int64_t)b->max_maps * pad_tile(b->max_cells));
+    EB_TRY(build_graph(q, p.bd, &g), "cudaGraphAddKernelNode");
     cudaGraphExec_t ex = nullptr;
     cudaError_t ie = cudaGraphInstantiate(&ex, g, 0);
     cudaGraphDestroy(g);
     EB_TRY(ie, "cudaGraphInstantiate");
     b->graph[p.slot] = ex;
-    b->graph_key[p.slot] = p.key;
+    b->graph_kind[p.slot] = p.kind;
   }
   EB_TRY(cudaGraphLaunch(b->graph[p.slot], s), "cudaGraphLaunch");
   return EM_OK;
@@ -308,7 +258,6 @@ void release(em_batch* b) {
     if (b->graph[i]) cudaGraphExecDestroy(b->graph[i]);
     if (b->ev[i]) cudaEventDestroy(b->ev[i]);
   }
-  if (b->capture_stream) cudaStreamDestroy(b->capture_stream);
   cudaFree(b->bctl);
   cudaFree(b->desc_dev);
   cudaFreeHost(b->desc_host);
@@ -370,7 +319,7 @@ int em_batch_create(int device, int32_t max_maps, int32_t max_clouds, int64_t ma
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->desc_dev, b->desc_bytes * kSlots);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->desc_host, b->desc_bytes * kSlots);
   for (int i = 0; i < kSlots && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&b->ev[i], cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->capture_stream, cudaStreamNonBlocking);
+  b->wait_budget = clock_budget(EM_PERSIST_WAIT_MS * 1000ll);
   if (e != cudaSuccess) {
     release(b);
     return map_record_error("em_batch_create", e);
@@ -402,7 +351,7 @@ int em_update_batch(em_batch* b, em_map* const* maps, const em_cloud* clouds, in
   if ((b->flags & EM_BATCH_GRAPH) && !b->prof) {
     rc = run_graph(b, p, s);
   } else {
-    cudaError_t e = launch_sequence(b, p.bd, p.points, p.cells, p.key, s, b);
+    cudaError_t e = launch_sequence(b, update_sequence(p.kind, p.points, p.cells), p.bd, s);
     rc = e == cudaSuccess ? EM_OK : map_record_error("batch launches", e);
   }
   finish(b, p, s);
@@ -492,7 +441,7 @@ int em_batch_autotune(em_batch* b, em_map* const* maps, const em_cloud* clouds, 
       int c = prepare(b, cmaps.data(), clouds, count, t, s, &p);
       if (c) return c;
       cudaEventRecord(e0, s);
-      cudaError_t le = launch_sequence(b, p.bd, p.points, p.cells, p.key, s);
+      cudaError_t le = launch_sequence(b, update_sequence(p.kind, p.points, p.cells), p.bd, s);
       cudaEventRecord(e1, s);
       finish(b, p, s);
       if (le != cudaSuccess) return map_record_error("autotune launches", le);

@@ -13,6 +13,9 @@ int map_device(const em_map* m);
 uint32_t map_flags(const em_map* m);
 int32_t map_cells(const em_map* m);
 const em_params& map_params(const em_map* m);
+// The passes an update of a map with these parameters needs.
+UpdateKind params_kind(const em_params& p, int32_t ray_group);
+UpdateKind map_kind(const em_map* m, int32_t ray_group);
 
 // Start one update of map m: advances its update index and returns its
 // device descriptor (pt_begin / pt_count are left to the caller).

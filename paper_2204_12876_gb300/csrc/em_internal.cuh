@@ -152,8 +152,9 @@ struct BatchDev {
   uint8_t* tr_status;
   BatchCtl* ctl;
   uint32_t passes;     // kPass* bits: optional passes some map of the batch needs
+  long long wait_budget;  // SM clock cycles a grid barrier of the persistent kernel may wait
 };
-enum : uint32_t { kPassRay = 1u, kPassPre = 2u, kPassCells = 4u };
+enum : uint32_t { kPassPre = 1u, kPassCells = 2u };
 
 // The coarse grid and the items of k_cells of a map of W x H cells.
 inline void set_item_grid(MapDev& d, int32_t W, int32_t H, bool ray, bool drift) {
@@ -171,23 +172,65 @@ inline bool word_aligned(const void* p) { return (reinterpret_cast<uintptr_t>(p)
 // number of SMs of the current device (cached)
 int sm_count();
 
-// ---- launchers (each returns cudaGetLastError() of its launches)
-// ext: some map of the batch uses the exclusion area or the upper-bound layer
-cudaError_t launch_pre(const BatchDev* b, int64_t n_points, bool ext, cudaStream_t s);
-cudaError_t launch_cells(const BatchDev* b, int64_t n_cells, cudaStream_t s);
-// ray: some map marches rays (group: samples per chunk and lanes per marched chunk)
-cudaError_t launch_points(const BatchDev* b, int64_t n_points, int group, bool ray, bool ext, cudaStream_t s);
-cudaError_t launch_write(const BatchDev* b, int64_t n_cells, cudaStream_t s);
+// ---- the kernels of an update
+// One launch: every kernel of an update takes the descriptor's device address
+// and nothing else, so a launch is plain data that can go to a stream or become
+// a graph node.
+struct Launch {
+  const void* fn;  // null: nothing to launch
+  unsigned grid, block;
+  size_t smem;
+  bool coop;
+  int slot;        // EM_PROF_* slot of its time
+  const char* name;
+};
+// What an update needs: the optional passes some map of it uses.
+struct UpdateKind {
+  int32_t ray_group;  // samples per chunk and lanes per marched chunk
+  bool ray;
+  bool drift;
+  bool wall;
+  bool ext;           // some map uses the exclusion area or the upper-bound layer
+  bool persistent;
+  uint32_t stencils;  // EM_F_* of the per-cell filters
+  bool operator==(const UpdateKind& o) const {
+    return ray_group == o.ray_group && ray == o.ray && drift == o.drift && wall == o.wall && ext == o.ext &&
+           persistent == o.persistent && stencils == o.stencils;
+  }
+};
+constexpr int kMaxLaunches = 8;
+struct Sequence {
+  int n = 0;
+  Launch k[kMaxLaunches];
+  void add(const Launch& l) {
+    if (l.fn) k[n++] = l;
+  }
+};
+// The launches of an update in stream order; grids for n_points points and
+// n_cells (padded) cells, which bound what the descriptor holds.
+Sequence update_sequence(const UpdateKind& k, int64_t n_points, int64_t n_cells);
+cudaError_t run(const Launch& l, const BatchDev* b, cudaStream_t s);
+// The sequence as a chain of kernel nodes.
+cudaError_t build_graph(const Sequence& q, const BatchDev* b, cudaGraph_t* out);
+
+Launch pre_launch(int64_t n_points, bool ext);
+Launch cells_launch(int64_t n_cells);
+Launch points_launch(int64_t n_points, int group, bool ray, bool ext);
+Launch write_launch(int64_t n_cells);
 // The whole update but the drift compensation and the stencils (points per
-// cell, thresholds, points, write) in one cooperative launch with grid barriers; barrier waits are bounded by
-// wait_ms.  cudaErrorNotSupported when the device cannot run it.
-cudaError_t launch_persist(const BatchDev* b, int group, bool ext, int wait_ms, cudaStream_t s);
+// cell, thresholds, points, write) in one cooperative launch with grid
+// barriers; barrier waits are bounded by the descriptor's wait_budget.  fn is
+// null when the device cannot run it.
+Launch persist_launch(int group, bool ext);
+long long clock_budget(long long us);  // SM clock cycles of that many microseconds
+Launch normals_launch(int64_t n_cells);
+Launch smooth_launch(int64_t n_cells);
+Launch inpaint_launch(int64_t n_cells);
+
+// ---- launchers of the other kernels (each returns cudaGetLastError())
 // The bounded wait of the persistent kernel on a word that nothing sets: one
 // block, budget wait_us; *timed_out (device memory) becomes 1 when it runs out.
 cudaError_t launch_wait_selftest(const unsigned long long* word, int* timed_out, int wait_us, cudaStream_t s);
-cudaError_t launch_normals(const BatchDev* b, int64_t n_cells, cudaStream_t s);
-cudaError_t launch_smooth(const BatchDev* b, int64_t n_cells, cudaStream_t s);
-cudaError_t launch_inpaint(const BatchDev* b, int64_t n_cells, cudaStream_t s);
 cudaError_t launch_shift_clear(const MapDev& m, int32_t dx, int32_t dy, cudaStream_t s);
 cudaError_t launch_layers_out(const MapDev& m, uint32_t mask, float* dst, cudaStream_t s);
 // Layer reads of up to kMaxReadJobs maps in one launch (the jobs are the kernel parameters).

@@ -230,12 +230,10 @@ extern "C" int em_update_noalloc(const em_params* params, int64_t shift_x, int64
   rc = na_status(cudaMemsetAsync(base + kOffCtl, 0, lay.thr - kOffCtl, s), "cudaMemsetAsync");
   if (rc) return rc;
   const int64_t cells = pad_tile(ncell);
-  const bool ext = params->excl_d > 0.f;  // no upper-bound layer here
-  const bool ray = params->ray_step > 0.f, drift = params->drift_flatness > 0.f;
+  UpdateKind kind = params_kind(*params, 8);
+  kind.stencils = 0;  // not the per-cell filters
+  const Sequence q = update_sequence(kind, total, cells);
   cudaError_t e = cudaSuccess;
-  if (drift || m->cnt) e = launch_pre(bd, total, ext, s);
-  if (e == cudaSuccess && (ray || drift)) e = launch_cells(bd, cells, s);
-  if (e == cudaSuccess) e = launch_points(bd, total, 8, ray, ext, s);
-  if (e == cudaSuccess) e = launch_write(bd, cells, s);
+  for (int i = 0; i < q.n && e == cudaSuccess; ++i) e = run(q.k[i], bd, s);
   return na_status(e, "em_update_noalloc launch");
 }

@@ -13,6 +13,7 @@
 // addition is associative, so the result is the same for every order of the
 // points and every split of the work, bit for bit (no float atomics).
 #include "cell_pass.cuh"
+#include "em.h"
 
 namespace em {
 
@@ -30,21 +31,19 @@ __global__ void __launch_bounds__(kCellThreads) k_write(const BatchDev* __restri
   write_pass(*bp, own_grid());
 }
 
-// n_cells bounds the items: an item has at most kItemW x kItemH cells, a map's
-// last row and column of items may be partial
-cudaError_t launch_cells(const BatchDev* b, int64_t n_cells, cudaStream_t s) {
+// n_cells bounds the items but for partial last rows and columns (the pass strides over the grid)
+Launch cells_launch(int64_t n_cells) {
   constexpr int kThreads = 128;  // small maps reach more SMs
   const int64_t blocks = n_cells / (kItemW * kItemH * (kThreads / 32)) + 1;
   const int64_t cap = (int64_t)sm_count() * 16;
-  k_cells<<<(int)(blocks < cap ? blocks : cap), kThreads, 0, s>>>(b);
-  return cudaGetLastError();
+  return {(const void*)&k_cells, (unsigned)(blocks < cap ? blocks : cap), kThreads, 0, false, EM_PROF_COUNT, "k_cells"};
 }
 
-cudaError_t launch_write(const BatchDev* b, int64_t n_cells, cudaStream_t s) {
+Launch write_launch(int64_t n_cells) {
   const int64_t tiles = n_cells / kTile;  // a block per tile
   const int64_t cap = (int64_t)sm_count() * 8;
-  k_write<<<(int)(tiles < 1 ? 1 : tiles < cap ? tiles : cap), kCellThreads, 0, s>>>(b);
-  return cudaGetLastError();
+  const unsigned grid = (unsigned)(tiles < 1 ? 1 : tiles < cap ? tiles : cap);
+  return {(const void*)&k_write, grid, kCellThreads, 0, false, EM_PROF_FUSE, "k_write"};
 }
 
 }  // namespace em

@@ -437,18 +437,12 @@ static int tile_grid(int64_t n_cells) {
   return (int)(tiles < 1 ? 1 : tiles < cap ? tiles : cap);
 }
 
-cudaError_t launch_normals(const BatchDev* b, int64_t n_cells, cudaStream_t s) {
-  k_normals<<<tile_grid(n_cells), kMapThreads, 0, s>>>(b);
-  return cudaGetLastError();
+static Launch stencil(const void* fn, int64_t n_cells, int slot, const char* name) {
+  return {fn, (unsigned)tile_grid(n_cells), kMapThreads, 0, false, slot, name};
 }
-cudaError_t launch_smooth(const BatchDev* b, int64_t n_cells, cudaStream_t s) {
-  k_smooth<<<tile_grid(n_cells), kMapThreads, 0, s>>>(b);
-  return cudaGetLastError();
-}
-cudaError_t launch_inpaint(const BatchDev* b, int64_t n_cells, cudaStream_t s) {
-  k_inpaint<<<tile_grid(n_cells), kMapThreads, 0, s>>>(b);
-  return cudaGetLastError();
-}
+Launch normals_launch(int64_t n_cells) { return stencil((const void*)&k_normals, n_cells, EM_PROF_NORMALS, "k_normals"); }
+Launch smooth_launch(int64_t n_cells) { return stencil((const void*)&k_smooth, n_cells, EM_PROF_SMOOTH, "k_smooth"); }
+Launch inpaint_launch(int64_t n_cells) { return stencil((const void*)&k_inpaint, n_cells, EM_PROF_INPAINT, "k_inpaint"); }
 
 cudaError_t launch_shift_clear(const MapDev& m, int32_t dx, int32_t dy, cudaStream_t s) {
   int32_t cx0 = 0, cx1 = 0, ry0 = 0, ry1 = 0;

@@ -18,6 +18,7 @@
 // that runs out raises the abort flag, writes EM_ERR_TIMEOUT into the maps'
 // error words, and every block leaves at its next barrier.
 #include "cell_pass.cuh"
+#include "em.h"
 #include "point_pass.cuh"
 
 namespace em {
@@ -61,10 +62,11 @@ __device__ __forceinline__ bool grid_barrier(const BatchDev& b, int nb, long lon
 }
 
 template <int G, bool kExt>
-__global__ void __launch_bounds__(kPersistThreads, 4) k_persist(const BatchDev* __restrict__ bp, long long budget) {
+__global__ void __launch_bounds__(kPersistThreads, 4) k_persist(const BatchDev* __restrict__ bp) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int s_ok;
   const BatchDev& b = *bp;
+  const long long budget = b.wait_budget;
   const int nb = gridDim.x, bid = blockIdx.x;
   const Grid all{bid, nb};
   bool ok = true;
@@ -95,65 +97,53 @@ __global__ void k_wait_selftest(const unsigned long long* word, int* timed_out, 
   if (threadIdx.x == 0) *timed_out = wait_at_least(word, 1ull, nullptr, budget) ? 0 : 1;
 }
 
-namespace {
-
-long long clock_budget(int ms_times_1000_us) {  // SM cycles of the given microseconds
+long long clock_budget(long long us) {
   int dev = 0, khz = 0;
   cudaGetDevice(&dev);
   if (cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess || khz <= 0) khz = 2000000;
-  return (long long)khz * ms_times_1000_us / 1000;
+  return (long long)khz * us / 1000;
 }
 
+namespace {
+
 template <int G, bool kExt>
-cudaError_t launch_persist_t(const BatchDev* b, long long budget, cudaStream_t s) {
+Launch persist_launch_t() {
   // per device, once: the shared-memory limit above the static 48 KB, and the
   // blocks that fit at once (the cooperative launch needs all of them resident)
-  static int per_sm[64][2] = {};
+  static int per_sm[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64) return cudaErrorNotSupported;
-  int& n = per_sm[dev][kExt ? 1 : 0];
+  if (dev < 0 || dev >= 64) return {};
+  const void* fn = (const void*)&k_persist<G, kExt>;
+  int& n = per_sm[dev];
   if (n == 0) {
-    cudaError_t e = cudaFuncSetAttribute(k_persist<G, kExt>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kPersistSmem);
-    if (e != cudaSuccess) return e;
     int v = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_persist<G, kExt>, kPersistThreads, kPersistSmem);
-    if (e != cudaSuccess) return e;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPersistSmem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, fn, kPersistThreads, kPersistSmem) != cudaSuccess) {
+      cudaGetLastError();
+      return {};
+    }
     n = v > 0 ? v : -1;
   }
-  if (n < 0) return cudaErrorNotSupported;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(n * sm_count()));
-  cfg.blockDim = dim3(kPersistThreads);
-  cfg.dynamicSmemBytes = kPersistSmem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_persist<G, kExt>, b, budget);
+  if (n < 0) return {};
+  return {fn, (unsigned)(n * sm_count()), kPersistThreads, kPersistSmem, true, EM_PROF_PERSIST, "k_persist"};
 }
 
 template <bool kExt>
-cudaError_t launch_persist_g(const BatchDev* b, int g, long long budget, cudaStream_t s) {
+Launch persist_launch_g(int g) {
   switch (g) {
-    case 1: return launch_persist_t<1, kExt>(b, budget, s);
-    case 2: return launch_persist_t<2, kExt>(b, budget, s);
-    case 4: return launch_persist_t<4, kExt>(b, budget, s);
-    case 16: return launch_persist_t<16, kExt>(b, budget, s);
-    case 32: return launch_persist_t<32, kExt>(b, budget, s);
-    default: return launch_persist_t<8, kExt>(b, budget, s);
+    case 1: return persist_launch_t<1, kExt>();
+    case 2: return persist_launch_t<2, kExt>();
+    case 4: return persist_launch_t<4, kExt>();
+    case 16: return persist_launch_t<16, kExt>();
+    case 32: return persist_launch_t<32, kExt>();
+    default: return persist_launch_t<8, kExt>();
   }
 }
 
 }  // namespace
 
-cudaError_t launch_persist(const BatchDev* b, int group, bool ext, int wait_ms, cudaStream_t s) {
-  const long long budget = clock_budget(wait_ms * 1000);
-  return ext ? launch_persist_g<true>(b, group, budget, s) : launch_persist_g<false>(b, group, budget, s);
-}
+Launch persist_launch(int group, bool ext) { return ext ? persist_launch_g<true>(group) : persist_launch_g<false>(group); }
 
 cudaError_t launch_wait_selftest(const unsigned long long* word, int* timed_out, int wait_us, cudaStream_t s) {
   k_wait_selftest<<<1, 32, 0, s>>>(word, timed_out, clock_budget(wait_us));

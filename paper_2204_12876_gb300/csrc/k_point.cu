@@ -31,6 +31,7 @@
 // when the lower of those two heights is not below the largest threshold of
 // the (at most 2 x 2) blocks they span, none of its samples can mark a cell
 // and it is skipped -- an exact test, not a heuristic.
+#include "em.h"
 #include "point_pass.cuh"
 
 namespace em {
@@ -66,38 +67,30 @@ static int point_grid(int64_t n, int per_sm) {
   return (int)(want < 1 ? 1 : want < cap ? want : cap);
 }
 
-cudaError_t launch_pre(const BatchDev* b, int64_t n_points, bool ext, cudaStream_t s) {
-  if (n_points <= 0) return cudaSuccess;
-  const int grid = point_grid(n_points, 16);
-  if (ext) k_pre<true><<<grid, kPointThreads, 0, s>>>(b);
-  else k_pre<false><<<grid, kPointThreads, 0, s>>>(b);
-  return cudaGetLastError();
+Launch pre_launch(int64_t n_points, bool ext) {
+  if (n_points <= 0) return {};
+  return {ext ? (const void*)&k_pre<true> : (const void*)&k_pre<false>, (unsigned)point_grid(n_points, 16),
+          kPointThreads, 0, false, EM_PROF_SCATTER, "k_pre"};
 }
 
 template <bool kExt>
-static void launch_points_g(const BatchDev* b, int g, int grid, cudaStream_t s) {
+static const void* points_kernel(int g) {
   switch (g) {
-    case 1: k_points<1, true, kExt><<<grid, kPointThreads, 0, s>>>(b); break;
-    case 2: k_points<2, true, kExt><<<grid, kPointThreads, 0, s>>>(b); break;
-    case 4: k_points<4, true, kExt><<<grid, kPointThreads, 0, s>>>(b); break;
-    case 16: k_points<16, true, kExt><<<grid, kPointThreads, 0, s>>>(b); break;
-    case 32: k_points<32, true, kExt><<<grid, kPointThreads, 0, s>>>(b); break;
-    default: k_points<8, true, kExt><<<grid, kPointThreads, 0, s>>>(b); break;
+    case 1: return (const void*)&k_points<1, true, kExt>;
+    case 2: return (const void*)&k_points<2, true, kExt>;
+    case 4: return (const void*)&k_points<4, true, kExt>;
+    case 16: return (const void*)&k_points<16, true, kExt>;
+    case 32: return (const void*)&k_points<32, true, kExt>;
+    default: return (const void*)&k_points<8, true, kExt>;
   }
 }
 
-cudaError_t launch_points(const BatchDev* b, int64_t n_points, int group, bool ray, bool ext, cudaStream_t s) {
-  if (n_points <= 0) return cudaSuccess;
-  const int grid = point_grid(n_points, 16);
-  if (!ray) {
-    if (ext) k_points<8, false, true><<<grid, kPointThreads, 0, s>>>(b);
-    else k_points<8, false, false><<<grid, kPointThreads, 0, s>>>(b);
-  } else if (ext) {
-    launch_points_g<true>(b, group, grid, s);
-  } else {
-    launch_points_g<false>(b, group, grid, s);
-  }
-  return cudaGetLastError();
+Launch points_launch(int64_t n_points, int group, bool ray, bool ext) {
+  if (n_points <= 0) return {};
+  const void* fn = ray ? (ext ? points_kernel<true>(group) : points_kernel<false>(group))
+                   : ext ? (const void*)&k_points<8, false, true>
+                         : (const void*)&k_points<8, false, false>;
+  return {fn, (unsigned)point_grid(n_points, 16), kPointThreads, 0, false, EM_PROF_RAY, "k_points"};
 }
 
 }  // namespace em
