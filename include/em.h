@@ -227,7 +227,8 @@ int em_get_trace(em_map* map, int32_t* ix, int32_t* iy, uint8_t* status, int64_t
  * Slots of em_profile_read, in this order: */
 enum {
   EM_PROF_COUNT = 0,   /* k_cells: drift compensation of the estimates, ray thresholds */
-  EM_PROF_RAY,         /* k_points: gate and sums of every point, visibility ray march */
+  EM_PROF_RAY,         /* k_points (and k_refresh between its parts): gate and sums of every point,
+                          visibility ray march */
   EM_PROF_ALLOC,       /* (no kernel) */
   EM_PROF_SCATTER,     /* k_pre: points per cell for the wall rule, drift sums */
   EM_PROF_FUSE,        /* k_write: new state of every cell, removal, overlap clearance */

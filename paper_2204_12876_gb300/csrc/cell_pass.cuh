@@ -2,6 +2,7 @@
 //
 //   cells_pass  before the points: estimates moved by the drift, ray thresholds
 //               of the pre-update map and their largest per coarse block
+//   refresh_pass  between parts of the points: marked cells out of both
 //   write_pass  after them: every cell's new state from its sums, removal of
 //               marked cells, overlap clearance
 //
@@ -15,13 +16,34 @@ namespace em {
 
 constexpr int kCellThreads = 256;
 
-// One warp per item of kItemW x kItemH logical cells: a lane's column of 8
-// cells gives 24 independent loads, rows are coalesced in both layouts, and the
-// item's four coarse blocks are maxima over 8 lanes.  The thresholds go to
-// logical order, so the march indexes them without the ring wrap.
-static_assert(kItemH == kCoarse && kItemW == 32 && kItemW % kCoarse == 0, "items hold whole coarse blocks");
-__device__ __forceinline__ void cells_pass(const BatchDev& b, Grid gr) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+// Do the points of a large update come in a sensor's order?  kOrderSamples
+// batches of 32 consecutive points, spread over the clouds, one warp's loads for
+// one block each; a batch counts as scattered when more than half of its
+// neighbouring points lie farther apart than half the nearer one's distance.
+__device__ __forceinline__ void sample_order(const BatchDev& b, Grid gr) {
+  if (b.n_points < kSplitPoints) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t n_batches = b.n_points / 32;  // whole ones
+  int scattered = 0;
+  for (int k = gr.bid; k < kOrderSamples; k += gr.nb) {
+    const int64_t g = n_batches * k / kOrderSamples * 32 + lane;
+    const CloudDev& c = b.clouds[find_cloud(b.clouds, b.n_clouds, g)];
+    float px, py, pz;
+    load_point(c, g - c.begin, px, py, pz);
+    const float qx = __shfl_down_sync(kFull, px, 1), qy = __shfl_down_sync(kFull, py, 1),
+                qz = __shfl_down_sync(kFull, pz, 1);
+    const float dx = qx - px, dy = qy - py, dz = qz - pz;
+    const float near = fminf(px * px + py * py + pz * pz, qx * qx + qy * qy + qz * qz);
+    const bool far = lane < 31 && dx * dx + dy * dy + dz * dz > 0.25f * near;  // false for NaN
+    scattered += __popc(__ballot_sync(kFull, far)) > 16;
+  }
+  if (lane == 0 && scattered) atomicAdd(&b.ctl->scattered, scattered);
+}
+
+// One warp per item: body(map, item column, item row), called by whole warps.
+template <class F>
+__device__ __forceinline__ void for_each_item(const BatchDev& b, Grid gr, F body) {
+  const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   for (int64_t g = (int64_t)gr.bid * warps + warp; g < b.n_items; g += (int64_t)gr.nb * warps) {
     int lo = 0, hi = b.n_maps - 1;  // the last map whose items start at or before g
     while (lo < hi) {
@@ -30,7 +52,34 @@ __device__ __forceinline__ void cells_pass(const BatchDev& b, Grid gr) {
     }
     const MapDev& m = b.maps[lo];
     const int32_t q = (int32_t)(g - m.ibegin);
-    const int32_t ty = q / m.IW, tx = q - ty * m.IW;
+    const int32_t ty = q / m.IW;
+    body(m, q - ty * m.IW, ty);
+  }
+}
+
+// The item's coarse blocks from the lanes' column maxima, and the rim entries
+// beside blocks at the map's edge.
+__device__ __forceinline__ void put_coarse(const MapDev& m, int32_t tx, int32_t ty, float mx) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < kCoarse; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
+  const int32_t cx = tx * (kItemW / kCoarse) + lane / kCoarse;
+  if (lane % kCoarse != 0 || cx >= m.CW) return;
+  float* const c = m.cthr + ty * m.CS + cx;
+  const int l = cx == 0 ? -1 : 0, r = cx == m.CW - 1 ? 1 : 0, t = ty == 0 ? -1 : 0, d = ty == m.CH - 1 ? 1 : 0;
+  for (int y = t; y <= d; ++y)
+    for (int x = l; x <= r; ++x) c[y * m.CS + x] = x == 0 && y == 0 ? mx : __int_as_float(0xff800000);
+}
+
+// One warp per item of kItemW x kItemH logical cells: a lane's column of 8
+// cells gives 24 independent loads, rows are coalesced in both layouts, and the
+// item's four coarse blocks are maxima over 8 lanes.  The thresholds go to
+// logical order, so the march indexes them without the ring wrap.
+static_assert(kItemH == kCoarse && kItemW == 32 && kItemW % kCoarse == 0, "items hold whole coarse blocks");
+__device__ __forceinline__ void cells_pass(const BatchDev& b, Grid gr) {
+  if (threadIdx.x < 32) sample_order(b, gr);
+  for_each_item(b, gr, [&](const MapDev& m, int32_t tx, int32_t ty) {
+    const int lane = threadIdx.x & 31;
     const int32_t W = m.W, lx = tx * kItemW + lane, y0 = ty * kItemH;
     const int32_t rows = lx < W ? min(kItemH, m.H - y0) : 0;
     int32_t px = lx + m.ox;
@@ -53,7 +102,7 @@ __device__ __forceinline__ void cells_pass(const BatchDev& b, Grid gr) {
       // every thread derives the same mean)
       const unsigned long long n = m.ctl->drift_n;
       const float mean = n ? __fdiv_rn(fixed_to_float(fix128(m.ctl->drift_h, m.ctl->drift_l)), (float)n) : 0.f;
-      if (q == 0 && lane == 0) {  // once per map
+      if (tx == 0 && ty == 0 && lane == 0) {  // once per map
         atomicAdd(&m.ctl->stats[kStDriftPoints], n);
         m.ctl->drift_last = mean;
       }
@@ -65,7 +114,7 @@ __device__ __forceinline__ void cells_pass(const BatchDev& b, Grid gr) {
         }
       }
     }
-    if (!ray) continue;
+    if (!ray) return;
     // Eq. 3: h - sqrt(var_eff); an empty cell is never penetrated (-inf).  With
     // the upper-bound layer it holds the cell's bound instead, so a ray sample
     // below the bound takes the march's candidate path and lowers it (Section II-H)
@@ -79,11 +128,43 @@ __device__ __forceinline__ void cells_pass(const BatchDev& b, Grid gr) {
       m.thr[(y0 + r) * W + lx] = t;
       mx = fmaxf(mx, t);  // a NaN never marks: skipped
     }
+    put_coarse(m, tx, ty, mx);
+  });
+}
+
+// Between two parts of the points: a marked cell stays marked, so its threshold
+// becomes -inf; an empty cell's is its bound as lowered so far; and the coarse
+// blocks' maxima are taken again.
+__device__ __forceinline__ void refresh_pass(const BatchDev& b, Grid gr) {
+  if (!in_parts(b)) return;
+  for_each_item(b, gr, [&](const MapDev& m, int32_t tx, int32_t ty) {
+    if (m.ray_step <= 0.f) return;
+    const int lane = threadIdx.x & 31;
+    const int32_t W = m.W, lx = tx * kItemW + lane, y0 = ty * kItemH;
+    const int32_t rows = lx < W ? min(kItemH, m.H - y0) : 0;
+    int32_t px = lx + m.ox;
+    px -= px >= W ? W : 0;
+    float t[kItemH];
+    uint32_t mark[kItemH];
 #pragma unroll
-    for (int o = 1; o < kCoarse; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
-    const int32_t cx = tx * (kItemW / kCoarse) + lane / kCoarse;
-    if (lane % kCoarse == 0 && cx < m.CW) m.cthr[ty * m.CW + cx] = mx;
-  }
+    for (int r = 0; r < kItemH; ++r) {  // all loads first
+      int32_t py = y0 + r + m.oy;
+      py -= py >= m.H ? m.H : 0;
+      const int32_t p = py * W + px;
+      t[r] = r < rows ? m.thr[(y0 + r) * W + lx] : __int_as_float(0xff800000);
+      mark[r] = r < rows ? (m.mark[p >> 5] >> (p & 31)) & 1u : 0u;
+      if (m.upper && r < rows && !isfinite(m.var[p])) t[r] = m.upper[p];
+    }
+    float mx = __int_as_float(0xff800000);
+#pragma unroll
+    for (int r = 0; r < kItemH; ++r) {
+      if (r >= rows) continue;
+      if (mark[r]) t[r] = __int_as_float(0xff800000);
+      if (mark[r] || m.upper) m.thr[(y0 + r) * W + lx] = t[r];
+      mx = fmaxf(mx, t[r]);
+    }
+    put_coarse(m, tx, ty, mx);
+  });
 }
 
 // New state of a cell from its complete sums; acc: some point was accepted, rej:
@@ -128,7 +209,10 @@ __device__ __forceinline__ void clear_acc(CellAcc* p) {
 constexpr int kWriteRounds = kTile / kCellThreads;
 __device__ __forceinline__ void write_pass(const BatchDev& b, Grid gr) {
   const int lane = threadIdx.x & 31;
-  if (gr.bid == 0 && threadIdx.x == 0) b.ctl->next = 0;
+  if (gr.bid == 0 && threadIdx.x == 0) {
+    for (int i = 0; i < kParts; ++i) b.ctl->next[i] = 0;
+    b.ctl->scattered = 0;
+  }
   for_each_tile(b, gr, [&](const MapDev& m, int, int32_t p0, int32_t count) {
     const int32_t tile = p0 / kTile;
     if (p0 == 0 && threadIdx.x == 0) {  // once per map

@@ -127,9 +127,10 @@ MapDev make_mapdev(const em_map* m) {
   memset(&d, 0, sizeof(d));
   d.h = m->h; d.var = m->var; d.t_last = m->t_last;
   d.nx = m->nx; d.ny = m->ny; d.nz = m->nz; d.smooth = m->smooth; d.inpaint = m->inpaint; d.upper = m->upper;
-  d.mark = m->mark; d.thr = m->thr; d.cthr = m->cthr;
+  d.mark = m->mark; d.thr = m->thr;
   d.acc = m->acc; d.rej = m->rej; d.cnt = m->cnt; d.touched = m->touched;
   set_item_grid(d, m->p.width, m->p.height, m->p.ray_step > 0.f, m->p.drift_flatness > 0.f);
+  if (m->cthr) d.cthr = m->cthr + coarse_first(m->p.width);
   d.ctl = m->ctl;
   d.cell_begin = 0;
   d.W = m->p.width; d.H = m->p.height; d.ox = m->ox; d.oy = m->oy;
@@ -299,7 +300,7 @@ int prof_collect(em_map* m) {
 template <class F>
 cudaError_t timed(em_map* m, int slot, cudaStream_t s, F fn) {
   if (!m->prof) return fn();
-  cudaEventRecord(m->prof_ev[2 * slot], s);
+  if (!m->prof_used[slot]) cudaEventRecord(m->prof_ev[2 * slot], s);  // a slot spans its launches
   cudaError_t e = fn();
   cudaEventRecord(m->prof_ev[2 * slot + 1], s);
   m->prof_used[slot] = true;
@@ -433,7 +434,8 @@ int em_create(const em_params* params, int device, em_map** out) {
   const size_t ntile = (size_t)(pad_tile((int64_t)nc) / kTile);
   EM_ALLOC(m->mark, (nc + 31) / 32)
   if (params->ray_step > 0.f) {
-    EM_ALLOC(m->thr, nc) EM_ALLOC(m->cthr, (size_t)coarse_dim(params->width) * coarse_dim(params->height))
+    const size_t nb = (size_t)coarse_size(params->width, params->height);
+    EM_ALLOC(m->thr, nc) EM_ALLOC(m->cthr, nb)
   }
   EM_ALLOC(m->acc, nc) EM_ALLOC(m->rej, nc) EM_ALLOC(m->touched, ntile)
   if (params->wall_num_thresh > 0) { EM_ALLOC(m->cnt, nc) }

@@ -41,6 +41,10 @@ constexpr int kTile = 1024;  // cells per tile of the cell space
 constexpr int kCoarseShift = 3;
 constexpr int kCoarse = 1 << kCoarseShift;
 inline int32_t coarse_dim(int32_t cells) { return (cells + kCoarse - 1) >> kCoarseShift; }
+// the grid in memory, with its rim: rows of coarse_stride(W) blocks; block (0, 0) is entry coarse_first(W)
+inline int32_t coarse_stride(int32_t W) { return coarse_dim(W) + 2; }
+inline int64_t coarse_size(int32_t W, int32_t H) { return (int64_t)coarse_stride(W) * (coarse_dim(H) + 2); }
+inline int32_t coarse_first(int32_t W) { return coarse_stride(W) + 1; }
 
 
 // per-map counters (device), in em_stats order
@@ -63,12 +67,12 @@ struct MapCtl {
 
 // per-batch device control block (zero between updates)
 struct BatchCtl {
-  int32_t next;              // work counter of k_points: runs of at most kRayRun 32-point batches
+  int32_t next[3];           // per part, work counter of k_points: runs of at most kRayRun 32-point batches
+  int32_t scattered;         // of the sampled batches of a large update, those whose points lie far apart (k_cells)
   // grid barrier of the persistent kernel (k_persist.cu): blocks done, the abort
   // flag of a barrier wait that ran out, and block tickets
   int32_t bar_done;
   int32_t bar_abort;
-  int32_t pad;
   unsigned long long bar_ticket;
 };
 
@@ -81,6 +85,13 @@ struct __align__(32) CellAcc {
   unsigned long long wh, wl, th, tl;
 };
 constexpr unsigned long long kAccTouched = 1ull << 63;
+
+// Large updates whose points come in no order go through them in parts
+// (point_pass.cuh): at least kSplitPoints points, and more than half of
+// kOrderSamples sampled batches scattered.
+constexpr int kParts = 3;
+constexpr uint32_t kSplitPoints = 1u << 20;
+constexpr int kOrderSamples = 64;
 
 constexpr int kItemW = 32, kItemH = 8;  // k_cells: logical cells per warp item
 
@@ -105,7 +116,9 @@ struct MapDev {
   float* upper;     // upper bound of the ground height (Section II-H), +inf where none; may be null
   uint32_t* mark;   // visibility marks, one bit per physical cell, zero between updates
   float* thr;       // per LOGICAL cell [iy][ix]: h - sqrt(var_eff) of the pre-update map, -inf if empty
-  float* cthr;      // per coarse block [by][bx] (CW x CH of them): the largest thr of its cells
+                    // (with the upper-bound layer an empty cell's bound); k_refresh: -inf where marked
+  float* cthr;      // per coarse block [by][bx] (CW x CH of them, rows CS apart, a rim of -inf blocks
+                    // around them): the largest thr of its cells
   MapCtl* ctl;
   CellAcc* acc;     // per physical cell
   uint32_t* rej;    // rejected points per physical cell, zero between updates
@@ -113,7 +126,7 @@ struct MapDev {
   uint8_t* touched; // per tile of kTile cells: some point of this update fell into it
   int64_t ibegin;   // this map's first item in the batch's item space (maps with the ray march or drift)
   int32_t IW, IH;   // items per row and column; 0 x 0 without the ray march and the drift compensation
-  int32_t CW, CH;   // coarse blocks per row and column; 0 x 0 without the ray march
+  int32_t CW, CH, CS;  // coarse blocks per row and column (0 x 0 without the ray march), row stride
   int64_t cell_begin;  // this map's first cell in the batch cell space (multiple of kTile)
   int32_t W, H, ox, oy;
   float x0, y0, res, inv_res;  // inv_res = 1 / res rounded to float
@@ -160,6 +173,7 @@ enum : uint32_t { kPassPre = 1u, kPassCells = 2u };
 inline void set_item_grid(MapDev& d, int32_t W, int32_t H, bool ray, bool drift) {
   d.CW = ray ? coarse_dim(W) : 0;
   d.CH = ray ? coarse_dim(H) : 0;
+  d.CS = ray ? coarse_stride(W) : 0;
   d.IW = ray || drift ? (W + kItemW - 1) / kItemW : 0;
   d.IH = ray || drift ? (H + kItemH - 1) / kItemH : 0;
 }
@@ -174,8 +188,8 @@ int sm_count();
 
 // ---- the kernels of an update
 // One launch: every kernel of an update takes the descriptor's device address
-// and nothing else, so a launch is plain data that can go to a stream or become
-// a graph node.
+// (k_points also the part), so a launch is plain data that can go to a stream or
+// become a graph node.
 struct Launch {
   const void* fn;  // null: nothing to launch
   unsigned grid, block;
@@ -183,6 +197,7 @@ struct Launch {
   bool coop;
   int slot;        // EM_PROF_* slot of its time
   const char* name;
+  int part;        // k_points: the part of the points
 };
 // What an update needs: the optional passes some map of it uses.
 struct UpdateKind {
@@ -198,7 +213,7 @@ struct UpdateKind {
            persistent == o.persistent && stencils == o.stencils;
   }
 };
-constexpr int kMaxLaunches = 8;
+constexpr int kMaxLaunches = 16;
 struct Sequence {
   int n = 0;
   Launch k[kMaxLaunches];
@@ -215,7 +230,8 @@ cudaError_t build_graph(const Sequence& q, const BatchDev* b, cudaGraph_t* out);
 
 Launch pre_launch(int64_t n_points, bool ext);
 Launch cells_launch(int64_t n_cells);
-Launch points_launch(int64_t n_points, int group, bool ray, bool ext);
+Launch refresh_launch(int64_t n_cells);
+Launch points_launch(int64_t n_points, int group, bool ray, bool ext, int part);
 Launch write_launch(int64_t n_cells);
 // The whole update but the drift compensation and the stencils (points per
 // cell, thresholds, points, write) in one cooperative launch with grid
@@ -296,6 +312,11 @@ __device__ __forceinline__ int find_cloud(const CloudDev* cl, int n_clouds, int6
 __device__ __forceinline__ int find_cloud(const CloudDev* cl, int n_clouds, int64_t g, int hint) {
   if ((unsigned)hint < (unsigned)n_clouds && cl[hint].begin <= g && g < cl[hint].begin + cl[hint].n) return hint;
   return find_cloud(cl, n_clouds, g);
+}
+
+// Whether this update's points go in parts (k_cells has run).
+__device__ __forceinline__ bool in_parts(const BatchDev& b) {
+  return b.n_points >= kSplitPoints && b.ctl->scattered > kOrderSamples / 2;
 }
 
 // index of the map whose cell range holds batch cell g (maps sorted by cell_begin)

@@ -67,8 +67,9 @@ constexpr Layout layout(size_t cells, size_t coarse) {
   o.end = o.cthr + up256(coarse * sizeof(float));
   return o;
 }
-// coarse blocks of a map of at most kMaxCells cells: (W/8 + 1)(H/8 + 1) <= kMaxCells/64 + (W + H)/8 + 1
-constexpr size_t kMaxCoarse = (size_t)kMaxCells / 64 + ((size_t)kMaxCells + 1) / 8 + 2;
+// coarse entries of a map of at most kMaxCells cells: (W/8 + 3)(H/8 + 3) <= kMaxCells/64 + 3 (W + H)/8 + 9,
+// and W + H <= kMaxCells + 1
+constexpr size_t kMaxCoarse = (size_t)kMaxCells / 64 + 3 * ((size_t)kMaxCells + 1) / 8 + 10;
 constexpr size_t kScratchBytes = layout(kMaxCells, kMaxCoarse).end;
 
 constexpr int kMaxDevices = 64;
@@ -171,14 +172,14 @@ extern "C" int em_update_noalloc(const em_params* params, int64_t shift_x, int64
   m->ny = const_cast<float*>(ny);
   m->nz = const_cast<float*>(nz);
   set_item_grid(*m, W, H, params->ray_step > 0.f, params->drift_flatness > 0.f);
-  const Layout lay = layout((size_t)ncell, (size_t)m->CW * m->CH);
+  const Layout lay = layout((size_t)ncell, m->CW ? (size_t)coarse_size(W, H) : 0);
   m->mark = reinterpret_cast<uint32_t*>(base + lay.mark);
   m->touched = base + lay.touched;
   m->rej = reinterpret_cast<uint32_t*>(base + lay.rej);
   if (params->wall_num_thresh > 0) m->cnt = reinterpret_cast<uint32_t*>(base + lay.cnt);
   m->acc = reinterpret_cast<CellAcc*>(base + lay.acc);
   m->thr = reinterpret_cast<float*>(base + lay.thr);
-  m->cthr = reinterpret_cast<float*>(base + lay.cthr);
+  m->cthr = reinterpret_cast<float*>(base + lay.cthr) + coarse_first(W);
   m->ctl = reinterpret_cast<MapCtl*>(base + kOffCtl);
   m->cell_begin = 0;
   m->z_ref = clouds[0].pose[11];

@@ -31,12 +31,21 @@ __global__ void __launch_bounds__(kCellThreads) k_write(const BatchDev* __restri
   write_pass(*bp, own_grid());
 }
 
+// Skips (one load a block) when the points went in one part.
+__global__ void __launch_bounds__(kCellThreads) k_refresh(const BatchDev* __restrict__ bp) {
+  refresh_pass(*bp, own_grid());
+}
+
 // n_cells bounds the items but for partial last rows and columns (the pass strides over the grid)
-Launch cells_launch(int64_t n_cells) {
+static Launch item_launch(const void* fn, int64_t n_cells, int slot, const char* name) {
   constexpr int kThreads = 128;  // small maps reach more SMs
   const int64_t blocks = n_cells / (kItemW * kItemH * (kThreads / 32)) + 1;
   const int64_t cap = (int64_t)sm_count() * 16;
-  return {(const void*)&k_cells, (unsigned)(blocks < cap ? blocks : cap), kThreads, 0, false, EM_PROF_COUNT, "k_cells"};
+  return {fn, (unsigned)(blocks < cap ? blocks : cap), kThreads, 0, false, slot, name, 0};
+}
+Launch cells_launch(int64_t n_cells) { return item_launch((const void*)&k_cells, n_cells, EM_PROF_COUNT, "k_cells"); }
+Launch refresh_launch(int64_t n_cells) {
+  return item_launch((const void*)&k_refresh, n_cells, EM_PROF_RAY, "k_refresh");
 }
 
 Launch write_launch(int64_t n_cells) {

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kPersistThreads, 4) k_persist(const BatchDev* 
     ok = grid_barrier(b, nb, budget, s_ok);
   }
   if (ok) {
-    points_pass<G, true, kExt>(b, all, *reinterpret_cast<PointsSmem<true>*>(sm));
+    points_pass<G, true, kExt>(b, all, -1, *reinterpret_cast<PointsSmem<true>*>(sm));
     ok = grid_barrier(b, nb, budget, s_ok);
   }
   if (ok) write_pass(b, all);

@@ -31,6 +31,17 @@
 // when the lower of those two heights is not below the largest threshold of
 // the (at most 2 x 2) blocks they span, none of its samples can mark a cell
 // and it is skipped -- an exact test, not a heuristic.
+//
+// What bounds it: issue and latency (one depth frame of 4 x 76,800 points: 23.5 M
+// warp instructions before the tests went to block coordinates on a rimmed grid
+// and the marks to a queue, 20 M then; 66 -> 58 us per update), on scattered
+// points the gathers of thresholds from L2 (1.4 G sectors for the 64-map batch,
+// which the parts with refreshed thresholds cut to about a third).  256 threads
+// and 64 registers, four blocks per SM: one resident wave that takes runs of
+// batches from a counter.  Measured and not kept: one test for the beam of a warp's
+// 32 rays before the rays' own (no fewer instructions: rays of an image row
+// have 4 to 8 chunks); thresholds or block maxima updated in place by the march
+// (mark_sample).
 #include "em.h"
 #include "point_pass.cuh"
 
@@ -43,9 +54,9 @@ __global__ void __launch_bounds__(kPointThreads) k_pre(const BatchDev* __restric
 }
 
 template <int G, bool kRay, bool kExt>
-__global__ void __launch_bounds__(kPointThreads, 4) k_points(const BatchDev* __restrict__ bp) {
+__global__ void __launch_bounds__(kPointThreads, 4) k_points(const BatchDev* __restrict__ bp, int part) {
   __shared__ PointsSmem<kRay> S;
-  points_pass<G, kRay, kExt>(*bp, own_grid(), S);
+  points_pass<G, kRay, kExt>(*bp, own_grid(), part, S);
 }
 
 int sm_count() {
@@ -85,12 +96,12 @@ static const void* points_kernel(int g) {
   }
 }
 
-Launch points_launch(int64_t n_points, int group, bool ray, bool ext) {
+Launch points_launch(int64_t n_points, int group, bool ray, bool ext, int part) {
   if (n_points <= 0) return {};
   const void* fn = ray ? (ext ? points_kernel<true>(group) : points_kernel<false>(group))
                    : ext ? (const void*)&k_points<8, false, true>
                          : (const void*)&k_points<8, false, false>;
-  return {fn, (unsigned)point_grid(n_points, 16), kPointThreads, 0, false, EM_PROF_RAY, "k_points"};
+  return {fn, (unsigned)point_grid(n_points, 4), kPointThreads, 0, false, EM_PROF_RAY, "k_points", part};
 }
 
 }  // namespace em

@@ -15,7 +15,11 @@ Sequence update_sequence(const UpdateKind& k, int64_t n_points, int64_t n_cells)
   } else {
     if (k.wall || k.drift) q.add(pre_launch(n_points, k.ext));
     if (k.ray || k.drift) q.add(cells_launch(n_cells));
-    q.add(points_launch(n_points, k.ray_group, k.ray, k.ext));
+    const int parts = k.ray && n_points >= (int64_t)kSplitPoints ? kParts : 1;
+    for (int i = 0; i < parts; ++i) {
+      if (i > 0) q.add(refresh_launch(n_cells));
+      q.add(points_launch(n_points, k.ray_group, k.ray, k.ext, i));
+    }
     q.add(write_launch(n_cells));
   }
   if (k.stencils & EM_F_NORMALS) q.add(normals_launch(n_cells));
@@ -25,7 +29,7 @@ Sequence update_sequence(const UpdateKind& k, int64_t n_points, int64_t n_cells)
 }
 
 cudaError_t run(const Launch& l, const BatchDev* b, cudaStream_t s) {
-  void* args[] = {(void*)&b};
+  void* args[] = {(void*)&b, (void*)&l.part};  // (a kernel takes as many as it has parameters)
   return l.coop ? cudaLaunchCooperativeKernel(l.fn, dim3(l.grid), dim3(l.block), args, l.smem, s)
                 : cudaLaunchKernel(l.fn, dim3(l.grid), dim3(l.block), args, l.smem, s);
 }
@@ -39,7 +43,7 @@ cudaError_t build_graph(const Sequence& q, const BatchDev* b, cudaGraph_t* out) 
   cudaGraphNode_t prev = nullptr;
   for (int i = 0; i < q.n && e == cudaSuccess; ++i) {
     const Launch& l = q.k[i];
-    void* args[] = {(void*)&b};
+    void* args[] = {(void*)&b, (void*)&l.part};
     cudaKernelNodeParams p = {};
     p.func = const_cast<void*>(l.fn);
     p.gridDim = dim3(l.grid);

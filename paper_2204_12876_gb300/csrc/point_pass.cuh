@@ -18,6 +18,15 @@ constexpr int kPointThreads = 256;
 constexpr int kPointWarps = kPointThreads / 32;
 constexpr int kRayRun = 8;  // 32-point batches per take from the work counter, at most
 
+// Large updates whose points come in no order go through them in parts, the
+// first ones small: between them k_refresh takes the marked cells out of the
+// thresholds and the coarse grid, so the later parts skip what the earlier ones
+// have decided (64-map batch, 14 M points: 4.15 -> 2.35 ms).  Points in a
+// sensor's order go in one part: their march is cheap, and parts break its
+// locality (32-robot round 601 -> 689 us).  Part i holds the places
+// part_first(i) .. part_first(i + 1) - 1 of every 32 batches.
+__device__ __forceinline__ uint32_t part_first(int i) { return i <= 0 ? 0u : i == 1 ? 2u : i == 2 ? 8u : 32u; }
+
 // Block-contiguous partition of the point space into chunks of whole warps.
 __device__ __forceinline__ void block_range(int64_t n, Grid gr, int64_t& beg, int64_t& end) {
   int64_t per = (n + gr.nb - 1) / gr.nb;
@@ -145,8 +154,8 @@ struct AccStage {
 // the accumulators: runs of equal cells in consecutive lanes are first reduced
 // by a segmented scan of the exact sums.  Every lane takes part; returns the
 // lane's status (meaningful where inm).
-__device__ __forceinline__ uint8_t add_points(const MapDev& m, int map, bool inm, uint32_t p, float z, float d,
-                                              AccStage& A) {
+__device__ __forceinline__ uint8_t add_points(const MapDev& m, int map, bool one_map, bool inm, uint32_t p, float z,
+                                              float d, AccStage& A) {
   const int lane = threadIdx.x & 31;
   Fix fw{0, 0u}, ft{0, 0u};
   uint8_t st = kPtOutside;
@@ -174,11 +183,16 @@ __device__ __forceinline__ uint8_t add_points(const MapDev& m, int map, bool inm
   // needs; within a run of at most 32 lanes the 27-bit low parts and the counts
   // (accepted | rejected << 16) fit 32 bits
   uint32_t nn = st == kPtFused ? 1u : st == kPtRejected ? (1u << 16) : 0u;
-  const unsigned long long tag = inm ? (unsigned long long)(uint32_t)map << 32 | p : ~0ull;
-  int head, len;
-  key_runs(tag, head, len);
-  const unsigned long long next = __shfl_down_sync(kFull, tag, 1);
-  const bool tail = inm && (lane == 31 || next != tag);
+  const uint32_t tag = inm ? p : 0xffffffffu;
+  const uint32_t prev = __shfl_up_sync(kFull, tag, 1);  // (every lane takes part in the shuffles)
+  bool first = lane == 0 || prev != tag;
+  if (!one_map) {
+    const int before = __shfl_up_sync(kFull, map, 1);
+    first = first || before != map;
+  }
+  const unsigned heads = __ballot_sync(kFull, first);
+  const int head = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+  const bool tail = inm && (lane == 31 || (heads >> (lane + 1)) & 1u);
   const int maxrun = (int)__reduce_max_sync(kFull, inm ? (unsigned)(lane - head + 1) : 1u);
   long long wh = fw.h, th = ft.h;
   uint32_t wl = fw.l, tl = ft.l;
@@ -249,10 +263,10 @@ __device__ __forceinline__ bool slab(float o, float v, float d, float a0, float 
 }
 
 // Per-ray set-up, made by one lane and read by the lanes that test and march
-// the ray's chunks.  Sample k lies at q = a + k b in cell units (x, y) and at
-// z = az + k bz, i.e. the track o + (k step / d) (R p_s) measured from the map
-// corner in cells.  Samples per ray are capped at 2^24 - 1, so the float
-// sample index is exact.
+// the ray's chunks.  Sample k lies at q = a + k b in coarse-block units (x, y:
+// an eighth of the position in cells, an exact scaling) and at z = az + k bz,
+// i.e. the track o + (k step / d) (R p_s) measured from the map corner.
+// Samples per ray are capped at 2^24 - 1, so the float sample index is exact.
 constexpr int32_t kMaxRayK = (1 << 24) - 1;
 
 struct RaySetup {
@@ -262,21 +276,27 @@ struct RaySetup {
   int32_t cn;           // samples per chunk
 };
 
-// floor(t) of a cell coordinate by one add rounded down: t + 1.5 2^23 lands
-// where the float spacing is 1, so its bits hold floor(t) + 0x4B400000 (|t| <
-// 2^22; anything farther out gives an index outside [0, 2^22) and fails the
-// map's box test)
-__device__ __forceinline__ int32_t cell_floor(float t) {
-  return __float_as_int(__fadd_rd(t, 12582912.0f)) - 0x4B400000;
-}
+// floor(8 t) -- the cell -- and floor(t) -- the block -- of a position in block
+// units by one add rounded down: t + 1.5 2^20 lands where the float spacing is
+// 1/8 (t + 1.5 2^23: 1), so its bits hold the floor plus a constant.  Exact for
+// cells below 2^22; the bits grow with t everywhere, so anything farther out
+// fails the map's box test.
+__device__ __forceinline__ int32_t cell_of(float t) { return __float_as_int(__fadd_rd(t, 1572864.0f)) - 0x49C00000; }
+__device__ __forceinline__ int32_t block_of(float t) { return __float_as_int(__fadd_rd(t, 12582912.0f)) - 0x4B400000; }
+static_assert(kCoarse == 8, "cell_of");
 
 // Shared memory of the points pass.  Per warp one buffer serves in turn the
 // points on their way in, the runs on their way out and the queue of chunks.
-constexpr int kRayQ = 256;  // queued chunks per warp (a ring)
+constexpr int kRayQ = 256;   // queued chunks per warp (a ring)
+constexpr int kMarkQ = 160;  // samples below their threshold: 31 waiting and 4 x 32 of a round
+struct ChunkQueue {
+  int2 chunk[kRayQ];      // {ray | samples << 8, first sample}
+  uint32_t mark[kMarkQ];  // sample | ray << 24
+};
 union WarpBuf {
   float4 stage[24];
   AccStage acc;
-  int2 q[kRayQ];  // {ray | samples << 8, first sample}
+  ChunkQueue q;
 };
 // The warps' rays, one array per field (lanes reading the fields of different
 // rays hit different banks).
@@ -312,6 +332,43 @@ __device__ __forceinline__ void put_ray(RaySmem& S, int t, const RaySetup& r) {
   S.ix[t] = r.ix; S.iy[t] = r.iy; S.k_lo[t] = r.k_lo; S.n[t] = r.n; S.map[t] = r.map; S.cn[t] = r.cn;
 }
 
+// One lane: sample k of ray sr of the warp lies below its cell's threshold.
+// Nothing the march reads for its tests is written here: a line that the SMs of
+// both dies read while others write it costs far more than the looks it saves
+// (thresholds or block flags updated in place took the 64-map batch from 4.0 to
+// 6.3 ms and one depth frame from 59 to 112 us).
+template <bool kExt>
+__device__ __forceinline__ void mark_sample(const BatchDev& b, const RaySmem& S, int sr, uint32_t k) {
+  const MapDev& m = b.maps[S.map[sr]];
+  const float kf = (float)k;
+  // the sample again, by the march's rounded arithmetic
+  const int32_t cx = cell_of(__fmaf_rn(kf, S.bx[sr], S.ax[sr])), cy = cell_of(__fmaf_rn(kf, S.by[sr], S.ay[sr]));
+  const int32_t p = phys_index(m, cx, cy);
+  if (kExt && !isfinite(m.var[p])) {
+    // an empty cell (its threshold is the upper bound): the sample lowers the
+    // bound (Section II-H); float minimum through the ordered bits
+    const int z = __float_as_int(__fmaf_rn(kf, S.bz[sr], S.az[sr]));
+    if (z >= 0) atomicMin(reinterpret_cast<int*>(m.upper + p), z);
+    else atomicMax(reinterpret_cast<unsigned int*>(m.upper + p), (unsigned)z);
+    return;
+  }
+  // many rays graze the same surface cells: nothing to do when the bit is already
+  // set (bits are only ever set during this kernel, so a stale read can only
+  // cost a redundant atomic, never a lost mark)
+  uint32_t* const word = m.mark + (p >> 5);
+  const uint32_t bit = 1u << (p & 31);
+  if (*word & bit) return;
+  if (m.alpha_n > 0.f) {  // Eq. 4
+    float n0 = m.nx[p], n1 = m.ny[p], n2 = m.nz[p];
+    if (!(isfinite(n0) && isfinite(n1) && isfinite(n2))) { n0 = 0.f; n1 = 0.f; n2 = 1.f; }
+    const float rd = S.d[sr];
+    const float rx = __fdiv_rn(S.vx[sr], rd), ry = __fdiv_rn(S.vy[sr], rd), rz = __fdiv_rn(S.vz[sr], rd);
+    const float dot = fabsf(__fmaf_rn(rx, n0, __fmaf_rn(ry, n1, __fmul_rn(rz, n2))));
+    if (!(dot > m.alpha_n)) return;
+  }
+  atomicOr(word, bit);
+}
+
 // Each warp takes 32 consecutive points, adds them to their cells, and marches
 // their rays: every lane sets up one ray (the k range inside the map box and
 // before the point, its chunk length) and tests its ray's chunks one after
@@ -319,7 +376,7 @@ __device__ __forceinline__ void put_ray(RaySmem& S, int t, const RaySetup& r) {
 // 4 x 32 / G at a time, G lanes per chunk and one sample per lane and round
 // (4 gathers in flight).
 template <int G, bool kRay, bool kExt>
-__device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, PointsSmem<kRay>& SM) {
+__device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, int part, PointsSmem<kRay>& SM) {
   constexpr int kU = G >= 4 ? 4 : G;         // samples per lane and march round, all of one chunk
   constexpr int kLPC = G / kU;               // lanes per chunk in the march
   constexpr int kFQ = 32 / kLPC;             // chunks per march round (at most 32)
@@ -333,15 +390,29 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, PointsSm
   // Runs are as long as leaves every warp of the grid two of them, at most
   // kRayRun batches.
   const uint32_t n_points = (uint32_t)b.n_points;  // below 2^31
-  const uint32_t n_batches = (n_points + 31) / 32, warps = (uint32_t)gr.nb * kPointWarps;
+  // the part's batches: `len` of every 32, those at places first .. of the
+  // bit-reversed order, so that every part samples the whole clouds (part -1, or
+  // points that go in one part: all of them, in order)
+  uint32_t first = 0, len = 32;
+  if (kRay && part >= 0 && in_parts(b)) {
+    first = part_first(part);
+    len = part_first(part + 1) - first;
+  } else if (part > 0) {
+    return;
+  }
+  const uint32_t warps = (uint32_t)gr.nb * kPointWarps;
+  uint32_t n_batches = (n_points + 31) / 32;
+  if (len < 32) n_batches = (n_batches + 31) / 32 * len;
   const uint32_t run_len = max(1u, min((uint32_t)kRayRun, n_batches / (2 * warps)));
   const uint32_t n_runs = (n_batches + run_len - 1) / run_len;
   int cmap = -1;  // the map the warp counts for, and this lane's counter
   unsigned long long count = 0;
   int hint = -1;  // the cloud of the warp's previous batch
   uint32_t run = (uint32_t)gr.bid * kPointWarps + warp;
-  uint32_t batch = run * run_len;
+  uint32_t index = run * run_len;
   while (run < n_runs) {
+    const uint32_t batch = len < 32 ? index / len * 32 + (__brev(first + index % len) >> 27) : index;
+    if (batch * 32 < n_points) {
     // ---- the points: transform, gate, sums
     float px, py, pz;
     const int ci = load_warp_points(b, (int64_t)batch * 32, n_points, SM.w[warp].stage, px, py, pz, hint);
@@ -353,15 +424,15 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, PointsSm
     const PointGeom pg = point_geom<kExt>(m, c, px, py, pz);
     const bool inm = live && pg.in_range && in_map(m, pg.ix, pg.iy);
     const uint32_t cell = inm ? (uint32_t)phys_index(m, pg.ix, pg.iy) : 0u;
-    const uint8_t st = add_points(m, map, inm, cell, pg.z, pg.d, SM.w[warp].acc);
+    const int map0 = __shfl_sync(kFull, map, 0);
+    const bool one_map = __all_sync(kFull, map == map0);
+    const uint8_t st = add_points(m, map, one_map, inm, cell, pg.z, pg.d, SM.w[warp].acc);
     if (b.tr_status && live) {
       b.tr_ix[g] = pg.finite ? pg.ix : INT32_MIN;
       b.tr_iy[g] = pg.finite ? pg.iy : INT32_MIN;
       b.tr_status[g] = !pg.finite ? kPtNonFinite : !pg.in_range ? kPtRange : st;
     }
     const bool ok = live && pg.in_range;
-    const int map0 = __shfl_sync(kFull, map, 0);
-    const bool one_map = __all_sync(kFull, !live || map == map0);  // lane 0 is live
     if (one_map) {
       if (map0 != cmap) {
         add_counts(b, cmap, count);
@@ -386,7 +457,7 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, PointsSm
     }
     if constexpr (kRay) {
     RaySmem& S = SM.ray;
-    int2* q = SM.w[warp].q;
+    ChunkQueue& Q = SM.w[warp].q;
     const int wb = warp * 32;  // the warp's rays in S
     // ---- set-up: one ray per lane
     RaySetup r;
@@ -413,10 +484,13 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, PointsSm
         for (int it = 0; it < 64 && k_last < kMaxRayK && __fmul_rn((float)(k_last + 1), step) < pg.d; ++it) ++k_last;
         if (k_last < k_hi) k_hi = k_last;
         const float cstep = __fdiv_rn(step, pg.d);  // f_k = k * step / d
-        r.ax = __fmul_rn(__fsub_rn(c.t[0], m.x0), m.inv_res);
-        r.ay = __fmul_rn(__fsub_rn(c.t[1], m.y0), m.inv_res);
-        r.bx = __fmul_rn(__fmul_rn(cstep, pg.vx), m.inv_res);
-        r.by = __fmul_rn(__fmul_rn(cstep, pg.vy), m.inv_res);
+        // in cells, then in blocks (an exact scaling: every sample's cell is that of the unscaled track)
+        const float bx = __fmul_rn(__fmul_rn(cstep, pg.vx), m.inv_res);
+        const float by = __fmul_rn(__fmul_rn(cstep, pg.vy), m.inv_res);
+        r.ax = __fmul_rn(__fmul_rn(__fsub_rn(c.t[0], m.x0), m.inv_res), 1.f / kCoarse);
+        r.ay = __fmul_rn(__fmul_rn(__fsub_rn(c.t[1], m.y0), m.inv_res), 1.f / kCoarse);
+        r.bx = __fmul_rn(bx, 1.f / kCoarse);
+        r.by = __fmul_rn(by, 1.f / kCoarse);
         r.az = c.t[2];
         r.bz = __fmul_rn(cstep, pg.vz);
         r.vx = pg.vx; r.vy = pg.vy; r.vz = pg.vz;
@@ -428,14 +502,13 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, PointsSm
         // a chunk and the next chunk's first sample span about kCoarse cells per axis at
         // most, so they touch at most 2 x 2 blocks (a rounding case that touches more is
         // marched untested)
-        const float span = fmaxf(fmaxf(fabsf(r.bx), fabsf(r.by)), 1e-6f);
+        const float span = fmaxf(fmaxf(fabsf(bx), fabsf(by)), 1e-6f);
         r.cn = (int32_t)fminf((float)G, fmaxf(1.f, floorf(__fdividef((float)kCoarse, span))));
       }
     }
     // samples of the march, per map
     if (one_map) {
-      unsigned long long t = (unsigned long long)r.n;
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+      const unsigned t = __reduce_add_sync(kFull, (unsigned)r.n);  // 32 (2^24 - 1) at most
       if (lane == kPsSamples) count += t;
     } else if (r.n > 0) {
       atomicAdd(&m.ctl->stats[kStRaySamples], (unsigned long long)r.n);
@@ -451,17 +524,19 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, PointsSm
     // least a quarter of the rounds.
     const int32_t nch = r.n > 0 ? (r.n + r.cn - 1) / r.cn : 0;
     const int32_t nq = (nch + kCU - 1) / kCU;
-    int32_t qinc = nq;  // inclusive scan of the quads over the lanes
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int32_t t = __shfl_up_sync(0xffffffffu, qinc, o);
-      if (lane >= o) qinc += t;
-    }
-    const int32_t qtot = __shfl_sync(0xffffffffu, qinc, 31);
-    const int32_t qmax = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)nq);
+    const int32_t qmax = (int32_t)__reduce_max_sync(kFull, (unsigned)nq);
+    const int32_t qtot = (int32_t)__reduce_add_sync(kFull, (unsigned)nq);
     const bool flat = 4 * ((qtot + 31) >> 5) <= 3 * qmax;  // warp-uniform
     const int32_t rounds = flat ? (qtot + 31) >> 5 : qmax;
-    int qh = 0, qn = 0;  // queue head and length (warp-uniform)
+    int32_t qinc = nq;  // inclusive scan of the quads over the lanes
+    if (flat) {
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int32_t t = __shfl_up_sync(kFull, qinc, o);
+        if (lane >= o) qinc += t;
+      }
+    }
+    int qh = 0, qn = 0, mn = 0;  // chunk queue: head and length; mark queue: length (warp-uniform)
     for (int32_t it = 0; it < rounds; ++it) {
       // this lane's quad: ray `src`, chunks c0 .. c0 + kCU - 1
       int src = lane;
@@ -472,63 +547,50 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, PointsSm
         int o = 0;  // lanes whose quads all come before quad j: the owner of quad j
 #pragma unroll
         for (int s = 16; s > 0; s >>= 1) {
-          const int32_t v = __shfl_sync(0xffffffffu, qinc, o + s - 1);
+          const int32_t v = __shfl_sync(kFull, qinc, o + s - 1);
           if (v <= j) o += s;
         }
         act = j < qtot;
         src = o < 32 ? o : 31;
-        c0 = (j - __shfl_sync(0xffffffffu, qinc - nq, src)) * kCU;
+        c0 = (j - __shfl_sync(kFull, qinc - nq, src)) * kCU;
       }
       const int sr = wb + src;
-      const int32_t k_lo = S.k_lo[sr], n = S.n[sr], cn = S.cn[sr];
+      const int32_t cn = S.cn[sr], kq = S.k_lo[sr] + c0 * cn;  // the quad's first sample
+      const int32_t left = act ? S.n[sr] - c0 * cn : 0;        // samples from there on
       const float ax = S.ax[sr], bx = S.bx[sr], ay = S.ay[sr], by = S.by[sr], az = S.az[sr], bz = S.bz[sr];
+      // The round's chunks and their end samples: chunk u is tested over its own
+      // samples and the next chunk's first one (a superset, so the test stays
+      // exact), so neighbouring chunks share an end and its block.  Blocks
+      // outside the map are those of the grid's rim, which holds -inf.  All loads
+      // of the round come first (no branches between them), then the tests.
       const MapDev& m = b.maps[S.map[sr]];
-      const float* __restrict__ ct = m.cthr;
-      const int32_t W = m.W, H = m.H, CW = m.CW;
-      // The round's chunks c0 .. c0 + kCU - 1 and their end samples: chunk u is
-      // tested over its own samples and the next chunk's first one (a superset,
-      // so the test stays exact), so neighbouring chunks share an end and its
-      // block.  All loads of the round come first (predicated, no branches
-      // between them), then the tests.
-      const int32_t klast = k_lo + n - 1;
-      int32_t xc[kCU + 1], yc[kCU + 1], bxs[kCU + 1], bys[kCU + 1];
+      const float* ct = m.cthr;
+      const int32_t CW = m.CW, CH = m.CH, CS = m.CS;
+      int32_t xb[kCU + 1], yb[kCU + 1];
       float zc[kCU + 1], ve[kCU + 1];
 #pragma unroll
       for (int u = 0; u <= kCU; ++u) {
-        const float kf = (float)min(k_lo + (c0 + u) * cn, klast);
-        xc[u] = cell_floor(__fmaf_rn(kf, bx, ax));
-        yc[u] = cell_floor(__fmaf_rn(kf, by, ay));
+        const float kf = (float)(kq + min(u * cn, max(left - 1, 0)));
+        xb[u] = min(max(block_of(__fmaf_rn(kf, bx, ax)), -1), CW);
+        yb[u] = min(max(block_of(__fmaf_rn(kf, by, ay)), -1), CH);
         zc[u] = __fmaf_rn(kf, bz, az);
-        bxs[u] = min(max(xc[u], 0), W - 1) >> kCoarseShift;
-        bys[u] = min(max(yc[u], 0), H - 1) >> kCoarseShift;
-        ve[u] = act ? __ldg(ct + bys[u] * CW + bxs[u]) : __int_as_float(0xff800000);
+        ve[u] = left > 0 ? ct[yb[u] * CS + xb[u]] : __int_as_float(0xff800000);
       }
-      bool keep[kCU];
-      int32_t k0[kCU], cnt[kCU];
 #pragma unroll
       for (int u = 0; u < kCU; ++u) {
-        const int32_t c = c0 + u;
-        k0[u] = k_lo + c * cn;
-        cnt[u] = min(cn, n - c * cn);
-        const int32_t xl = min(xc[u], xc[u + 1]), xh = max(xc[u], xc[u + 1]);
-        const int32_t yl = min(yc[u], yc[u + 1]), yh = max(yc[u], yc[u + 1]);
-        // some sample of the chunk may be inside the map
-        const bool inside = act && c * cn < n && xh >= 0 && xl < W && yh >= 0 && yl < H;
-        // more than 2 x 2 blocks (not for the chunk lengths above): march it untested
-        const bool wide = abs(bxs[u + 1] - bxs[u]) > 1 || abs(bys[u + 1] - bys[u]) > 1;
+        const int32_t dx = xb[u + 1] - xb[u], dy = yb[u + 1] - yb[u];
         // the two other corners of the 2 x 2 box, when the chunk crosses a block row and column
-        const bool cross = inside && !wide && bxs[u] != bxs[u + 1] && bys[u] != bys[u + 1];
-        const float o1 = cross ? __ldg(ct + bys[u] * CW + bxs[u + 1]) : __int_as_float(0xff800000);
-        const float o2 = cross ? __ldg(ct + bys[u + 1] * CW + bxs[u]) : __int_as_float(0xff800000);
-        const float mx = fmaxf(fmaxf(ve[u], ve[u + 1]), fmaxf(o1, o2));
-        keep[u] = inside && (wide || fminf(zc[u], zc[u + 1]) < mx);
-      }
-      // ---- queue the chunks that may mark a cell
-#pragma unroll
-      for (int u = 0; u < kCU; ++u) {
-        const unsigned km = __ballot_sync(0xffffffffu, keep[u]);
-        if (keep[u])
-          q[(qh + qn + __popc(km & ((1u << lane) - 1u))) & (kQ - 1)] = make_int2(src | (cnt[u] << 8), k0[u]);
+        float mx = fmaxf(ve[u], ve[u + 1]);
+        if (left > 0 && dx != 0 && dy != 0) mx = fmaxf(mx, fmaxf(ct[yb[u] * CS + xb[u + 1]], ct[yb[u + 1] * CS + xb[u]]));
+        // more than 2 x 2 blocks (not for the chunk lengths above): march it untested
+        const bool wide = (unsigned)(dx + 1) > 2u || (unsigned)(dy + 1) > 2u;
+        const int32_t cnt = min(cn, left - u * cn);
+        const bool keep = cnt > 0 && (wide || fminf(zc[u], zc[u + 1]) < mx);
+        // ---- queue the chunks that may mark a cell
+        const unsigned km = __ballot_sync(kFull, keep);
+        if (keep)
+          Q.chunk[(qh + qn + __popc(km & ((1u << lane) - 1u))) & (kQ - 1)] =
+              make_int2(src | (cnt << 8), kq + u * cn);
         qn += __popc(km);
       }
       __syncwarp();
@@ -536,65 +598,49 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, PointsSm
       const bool last = it + 1 >= rounds;
       while (qn >= kFQ || (last && qn > 0)) {
         // lane: chunk qi, samples sj, sj + kLPC, ...; every threshold first (kU gathers
-        // in flight), then the marks
+        // in flight), then the samples below theirs go to the mark queue: a few lanes
+        // in a hundred, so marking them where they are found would run a long branch
+        // for one or two lanes at a time
         const int qi = lane / kLPC, sj = lane % kLPC;
-        const int2 e = q[(qh + qi) & (kQ - 1)];
-        const int32_t ne = e.x >> 8;
-        const int sr = wb + (e.x & 31);
-        const int32_t rmap = S.map[sr];
-        const bool live = qi < qn && (unsigned)rmap < (unsigned)b.n_maps;
-        const MapDev& mm = b.maps[live ? rmap : 0];
-        const int32_t Wm = mm.W, Hm = mm.H, ox = mm.ox, oy = mm.oy;
-        const float* __restrict__ tm = mm.thr;
-        uint32_t* __restrict__ mk = mm.mark;
-        const float ax = S.ax[sr], bx = S.bx[sr], ay = S.ay[sr], by = S.by[sr], az = S.az[sr], bz = S.bz[sr];
-        const int32_t rix = S.ix[sr], riy = S.iy[sr];
+        const int2 e = Q.chunk[(qh + qi) & (kQ - 1)];
+        const int32_t ne = qi < qn ? e.x >> 8 : 0;
+        const int mr = qi < qn ? e.x & 31 : 0, sm = wb + mr;
+        const MapDev& mm = b.maps[S.map[sm]];
+        const int32_t Wm = mm.W, Hm = mm.H;
+        const float* tm = mm.thr;
+        const float mx0 = S.ax[sm], mbx = S.bx[sm], my0 = S.ay[sm], mby = S.by[sm], mz0 = S.az[sm], mbz = S.bz[sm];
+        const int32_t rix = S.ix[sm], riy = S.iy[sm];
+        const float kf0 = (float)(e.y + sj);
         float zz[kU], th[kU];
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
-          const int32_t j = sj + u * kLPC;
-          const float kf = (float)(e.y + j);
-          const int32_t cx = cell_floor(__fmaf_rn(kf, bx, ax));
-          const int32_t cy = cell_floor(__fmaf_rn(kf, by, ay));
-          const bool ok = live && j < ne && (uint32_t)cx < (uint32_t)Wm && (uint32_t)cy < (uint32_t)Hm &&
+          const float kf = kf0 + (float)(u * kLPC);
+          const int32_t cx = cell_of(__fmaf_rn(kf, mbx, mx0));
+          const int32_t cy = cell_of(__fmaf_rn(kf, mby, my0));
+          const bool in = sj + u * kLPC < ne && (uint32_t)cx < (uint32_t)Wm && (uint32_t)cy < (uint32_t)Hm &&
                           !(cx == rix && cy == riy);
-          zz[u] = __fmaf_rn(kf, bz, az);
-          th[u] = ok ? __ldg(tm + cy * Wm + cx) : __int_as_float(0xff800000);  // logical index; -inf: never below
+          zz[u] = __fmaf_rn(kf, mbz, mz0);
+          th[u] = in ? tm[cy * Wm + cx] : __int_as_float(0xff800000);  // logical index; -inf: never below
         }
+        bool any = false;
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          if (!(zz[u] < th[u])) continue;  // the common case, and every sample not taken
-          // the sample's cell again (the same rounded arithmetic as above: no
-          // register holds it through the gathers), then its physical index in
-          // the ring-buffer layout of the map layers
-          const float kf = (float)(e.y + sj + u * kLPC);
-          const int32_t cx = cell_floor(__fmaf_rn(kf, bx, ax));
-          const int32_t cy = cell_floor(__fmaf_rn(kf, by, ay));
-          int32_t px = cx + ox;
-          px -= (px >= Wm) ? Wm : 0;
-          int32_t py = cy + oy;
-          py -= (py >= Hm) ? Hm : 0;
-          const int32_t p = py * Wm + px;
-          if (kExt && !isfinite(mm.var[p])) {
-            // an empty cell (its threshold is the upper bound): the sample lowers
-            // the bound (Section II-H); float minimum through the ordered bits
-            if (__float_as_int(zz[u]) >= 0) atomicMin(reinterpret_cast<int*>(mm.upper + p), __float_as_int(zz[u]));
-            else atomicMax(reinterpret_cast<unsigned int*>(mm.upper + p), __float_as_uint(zz[u]));
-            continue;
+        for (int u = 0; u < kU; ++u) any |= zz[u] < th[u];
+        if (__any_sync(kFull, any)) {
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            const bool below = zz[u] < th[u];
+            const unsigned bm = __ballot_sync(kFull, below);
+            if (below)
+              Q.mark[mn + __popc(bm & ((1u << lane) - 1u))] = (uint32_t)(e.y + sj + u * kLPC) | (uint32_t)mr << 24;
+            mn += __popc(bm);
           }
-          if (mm.alpha_n > 0.f) {
-            float n0 = mm.nx[p], n1 = mm.ny[p], n2 = mm.nz[p];
-            if (!(isfinite(n0) && isfinite(n1) && isfinite(n2))) { n0 = 0.f; n1 = 0.f; n2 = 1.f; }
-            const float rd = S.d[sr];
-            const float rx = __fdiv_rn(S.vx[sr], rd), ry = __fdiv_rn(S.vy[sr], rd), rz = __fdiv_rn(S.vz[sr], rd);
-            const float dot = fabsf(__fmaf_rn(rx, n0, __fmaf_rn(ry, n1, __fmul_rn(rz, n2))));
-            if (!(dot > mm.alpha_n)) continue;
+          __syncwarp();
+          while (mn >= 32) {
+            mn -= 32;
+            const uint32_t v = Q.mark[mn + lane];
+            mark_sample<kExt>(b, S, wb + (int)(v >> 24), v & 0xffffffu);
           }
-          // many rays graze the same surface cells: skip the atomic when the bit is
-          // already set.  Bits are only ever set during this kernel, so a stale read
-          // can only cost a redundant atomic, never a lost mark.
-          const uint32_t bit = 1u << (p & 31);
-          if (!(mk[p >> 5] & bit)) atomicOr(&mk[p >> 5], bit);
+          __syncwarp();
         }
         const int took = min(qn, kFQ);
         qh = (qh + took) & (kQ - 1);
@@ -602,15 +648,20 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, PointsSm
         __syncwarp();
       }
     }
+    if (lane < mn) {
+      const uint32_t v = Q.mark[lane];
+      mark_sample<kExt>(b, S, wb + (int)(v >> 24), v & 0xffffffu);
+    }
     __syncwarp();
     }
+    }  // a batch of the clouds
     // the next batch of the run, or the next run
-    ++batch;
-    if (batch >= (run + 1) * run_len || batch >= n_batches) {
+    ++index;
+    if (index >= (run + 1) * run_len || index >= n_batches) {
       uint32_t t = 0;
-      if (lane == 0) t = (uint32_t)atomicAdd(&b.ctl->next, 1);
+      if (lane == 0) t = (uint32_t)atomicAdd(&b.ctl->next[max(part, 0)], 1);
       run = warps + __shfl_sync(kFull, t, 0);
-      batch = run * run_len;
+      index = run * run_len;
     }
   }
   // the warps' counts: one atomic per block and counter when the block saw one
