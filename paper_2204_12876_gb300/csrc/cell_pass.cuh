@@ -20,7 +20,8 @@ constexpr int kCellThreads = 256;
 // batches of 32 consecutive points, spread over the clouds, one warp's loads for
 // one block each; a batch counts as scattered when more than half of its
 // neighbouring points lie farther apart than half the nearer one's distance.
-__device__ __forceinline__ void sample_order(const BatchDev& b, Grid gr) {
+template <class V>
+__device__ __forceinline__ void sample_order(const V& b, Grid gr) {
   if (b.n_points < kSplitPoints) return;
   const int lane = threadIdx.x & 31;
   const int64_t n_batches = b.n_points / 32;  // whole ones
@@ -41,8 +42,8 @@ __device__ __forceinline__ void sample_order(const BatchDev& b, Grid gr) {
 }
 
 // One warp per item: body(map, item column, item row), called by whole warps.
-template <class F>
-__device__ __forceinline__ void for_each_item(const BatchDev& b, Grid gr, F body) {
+template <class V, class F>
+__device__ __forceinline__ void for_each_item(const V& b, Grid gr, F body) {
   const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   for (int64_t g = (int64_t)gr.bid * warps + warp; g < b.n_items; g += (int64_t)gr.nb * warps) {
     int lo = 0, hi = b.n_maps - 1;  // the last map whose items start at or before g
@@ -50,7 +51,7 @@ __device__ __forceinline__ void for_each_item(const BatchDev& b, Grid gr, F body
       const int mid = (lo + hi + 1) >> 1;
       if (b.maps[mid].ibegin <= g) lo = mid; else hi = mid - 1;
     }
-    const MapDev& m = b.maps[lo];
+    const MapDev& m = map_at(b, lo);
     const int32_t q = (int32_t)(g - m.ibegin);
     const int32_t ty = q / m.IW;
     body(m, q - ty * m.IW, ty);
@@ -76,7 +77,8 @@ __device__ __forceinline__ void put_coarse(const MapDev& m, int32_t tx, int32_t 
 // item's four coarse blocks are maxima over 8 lanes.  The thresholds go to
 // logical order, so the march indexes them without the ring wrap.
 static_assert(kItemH == kCoarse && kItemW == 32 && kItemW % kCoarse == 0, "items hold whole coarse blocks");
-__device__ __forceinline__ void cells_pass(const BatchDev& b, Grid gr) {
+template <class V>
+__device__ __forceinline__ void cells_pass(const V& b, Grid gr) {
   if (threadIdx.x < 32) sample_order(b, gr);
   for_each_item(b, gr, [&](const MapDev& m, int32_t tx, int32_t ty) {
     const int lane = threadIdx.x & 31;
@@ -135,7 +137,8 @@ __device__ __forceinline__ void cells_pass(const BatchDev& b, Grid gr) {
 // Between two parts of the points: a marked cell stays marked, so its threshold
 // becomes -inf; an empty cell's is its bound as lowered so far; and the coarse
 // blocks' maxima are taken again.
-__device__ __forceinline__ void refresh_pass(const BatchDev& b, Grid gr) {
+template <class V>
+__device__ __forceinline__ void refresh_pass(const V& b, Grid gr) {
   if (!in_parts(b)) return;
   for_each_item(b, gr, [&](const MapDev& m, int32_t tx, int32_t ty) {
     if (m.ray_step <= 0.f) return;
@@ -207,7 +210,8 @@ __device__ __forceinline__ void clear_acc(CellAcc* p) {
 // tile's flag go back to zero for the next update.  Tiles start on multiples of
 // kTile cells, so a tile owns whole mark words.
 constexpr int kWriteRounds = kTile / kCellThreads;
-__device__ __forceinline__ void write_pass(const BatchDev& b, Grid gr) {
+template <class V>
+__device__ __forceinline__ void write_pass(const V& b, Grid gr) {
   const int lane = threadIdx.x & 31;
   if (gr.bid == 0 && threadIdx.x == 0) {
     for (int i = 0; i < kParts; ++i) b.ctl->next[i] = 0;

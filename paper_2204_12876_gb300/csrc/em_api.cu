@@ -37,6 +37,7 @@ int cuda_status(cudaError_t e, const char* what) {
 constexpr int kSlots = 4;
 constexpr int kMaxClouds = 64;
 constexpr size_t kDescBytes = sizeof(BatchDev) + sizeof(MapDev) + kMaxClouds * sizeof(CloudDev) + 64;
+static_assert(kDescBytes >= sizeof(MapDesc), "the descriptor ring");
 
 template <class T>
 cudaError_t dev_alloc(T** p, size_t count, int64_t* total) {
@@ -231,18 +232,10 @@ bool pose_ok(const float* pose) {
   return true;
 }
 
-// Build and upload the descriptor of a one-map update; returns the device
-// address of its BatchDev.
-int upload_desc(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t total, cudaStream_t s,
-                const BatchDev** out) {
-  const int slot = m->slot;
-  m->slot = (m->slot + 1) % kSlots;
-  EM_TRY(cudaEventSynchronize(m->desc_ev[slot]), "cudaEventSynchronize");
-  unsigned char* hb = m->desc_host + (size_t)slot * kDescBytes;
-  unsigned char* db = m->desc_dev + (size_t)slot * kDescBytes;
-  BatchDev* b = reinterpret_cast<BatchDev*>(hb);
-  MapDev* md = reinterpret_cast<MapDev*>(hb + sizeof(BatchDev));
-  CloudDev* cd = reinterpret_cast<CloudDev*>(hb + sizeof(BatchDev) + sizeof(MapDev));
+// The descriptor of a one-map update into b, md and cd (pointers between them
+// are left to the caller).
+void fill_desc(const em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t total, BatchDev* b, MapDev* md,
+               CloudDev* cd) {
   memset(b, 0, sizeof(BatchDev));
   *md = make_mapdev(m);
   md->z_ref = n_clouds > 0 ? clouds[0].pose[11] : 0.f;  // the first cloud's sensor origin
@@ -266,14 +259,28 @@ int upload_desc(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t tot
   b->n_maps = 1;
   b->n_clouds = n_clouds;
   b->n_points = total;
-  b->maps = reinterpret_cast<const MapDev*>(db + sizeof(BatchDev));
-  b->clouds = reinterpret_cast<const CloudDev*>(db + sizeof(BatchDev) + sizeof(MapDev));
   b->tr_ix = m->tr_ix;
   b->tr_iy = m->tr_iy;
   b->tr_status = m->tr_status;
   b->n_cells = pad_tile((int64_t)m->p.width * m->p.height);
   b->n_items = (int64_t)md->IW * md->IH;
   b->ctl = m->bctl;
+}
+
+// Build and upload the descriptor of a one-map update (more clouds than a
+// MapDesc holds); its slot, and the device address of its BatchDev.
+int upload_desc(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t total, cudaStream_t s,
+                const BatchDev** out) {
+  const int slot = m->slot;
+  m->slot = (m->slot + 1) % kSlots;
+  EM_TRY(cudaEventSynchronize(m->desc_ev[slot]), "cudaEventSynchronize");
+  unsigned char* hb = m->desc_host + (size_t)slot * kDescBytes;
+  unsigned char* db = m->desc_dev + (size_t)slot * kDescBytes;
+  BatchDev* b = reinterpret_cast<BatchDev*>(hb);
+  fill_desc(m, clouds, n_clouds, total, b, reinterpret_cast<MapDev*>(hb + sizeof(BatchDev)),
+            reinterpret_cast<CloudDev*>(hb + sizeof(BatchDev) + sizeof(MapDev)));
+  b->maps = reinterpret_cast<const MapDev*>(db + sizeof(BatchDev));
+  b->clouds = reinterpret_cast<const CloudDev*>(db + sizeof(BatchDev) + sizeof(MapDev));
   const size_t bytes = sizeof(BatchDev) + sizeof(MapDev) + (size_t)n_clouds * sizeof(CloudDev);
   EM_TRY(cudaMemcpyAsync(db, hb, bytes, cudaMemcpyHostToDevice, s), "upload descriptor");
   *out = reinterpret_cast<const BatchDev*>(db);
@@ -493,17 +500,26 @@ static int update_impl(em_map* m, const em_cloud* clouds, int32_t n_clouds, cuda
   int rc = grow_workspace(m, total);
   if (rc) return rc;
   m->t_now += 1;
-  const BatchDev* bd = nullptr;
-  int slot = upload_desc(m, clouds, n_clouds, total, s, &bd);
-  if (slot < 0) {
-    m->t_now -= 1;
-    return slot;
-  }
   const int64_t ncell = pad_tile((int64_t)m->p.width * m->p.height);
-  const Sequence q = update_sequence(map_kind(m, m->ray_group), total, ncell);
+  UpdateKind kind = map_kind(m, m->ray_group);
+  kind.by_value = n_clouds <= kDescClouds && m->ray_group == kValueGroup;
+  MapDesc desc;
+  const BatchDev* bd = nullptr;
+  const void* arg = kind.by_value ? (const void*)&desc : (const void*)&bd;
+  int slot = -1;
+  if (kind.by_value) {
+    fill_desc(m, clouds, n_clouds, total, &desc.b, &desc.m, desc.c);
+  } else {
+    slot = upload_desc(m, clouds, n_clouds, total, s, &bd);
+    if (slot < 0) {
+      m->t_now -= 1;
+      return slot;
+    }
+  }
+  const Sequence q = update_sequence(kind, total, ncell);
   for (int i = 0; i < q.n; ++i)
-    EM_TRY(timed(m, q.k[i].slot, s, [&] { return run(q.k[i], bd, s); }), q.k[i].name);
-  EM_TRY(cudaEventRecord(m->desc_ev[slot], s), "cudaEventRecord");
+    EM_TRY(timed(m, q.k[i].slot, s, [&] { return run(q.k[i], arg, i == 0 || m->prof, s); }), q.k[i].name);
+  if (slot >= 0) EM_TRY(cudaEventRecord(m->desc_ev[slot], s), "cudaEventRecord");
   m->last_stream = s;
   m->last_n = total;
   m->points_in += total;

@@ -167,6 +167,30 @@ struct BatchDev {
   uint32_t passes;     // kPass* bits: optional passes some map of the batch needs
   long long wait_budget;  // SM clock cycles a grid barrier of the persistent kernel may wait
 };
+// The descriptor of an update of one map with few clouds travels as a kernel
+// parameter: nothing to upload before the first kernel, and the fields are read
+// from the constant bank instead of through two dependent global loads.
+constexpr int kDescClouds = 8;
+struct MapDesc {
+  BatchDev b;
+  MapDev m;
+  CloudDev c[kDescClouds];
+};
+static_assert(sizeof(MapDesc) <= 4096, "a kernel parameter");
+// What the passes see of either form.
+struct MapView : BatchDev {};
+__device__ __forceinline__ const BatchDev& view(const BatchDev* p) { return *p; }
+__device__ __forceinline__ MapView view(const MapDesc& d) {
+  MapView v;
+  static_cast<BatchDev&>(v) = d.b;
+  v.n_maps = 1;
+  v.maps = &d.m;
+  v.clouds = d.c;
+  return v;
+}
+__device__ __forceinline__ const MapDev& map_at(const BatchDev& b, int i) { return b.maps[i]; }
+__device__ __forceinline__ const MapDev& map_at(const MapView& b, int) { return b.maps[0]; }
+
 enum : uint32_t { kPassPre = 1u, kPassCells = 2u };
 
 // The coarse grid and the items of k_cells of a map of W x H cells.
@@ -187,9 +211,9 @@ inline bool word_aligned(const void* p) { return (reinterpret_cast<uintptr_t>(p)
 int sm_count();
 
 // ---- the kernels of an update
-// One launch: every kernel of an update takes the descriptor's device address
-// (k_points also the part), so a launch is plain data that can go to a stream or
-// become a graph node.
+// One launch: every kernel of an update takes the descriptor -- its device
+// address, or the descriptor itself (MapDesc) -- and k_points also the part, so a
+// launch is plain data that can go to a stream or become a graph node.
 struct Launch {
   const void* fn;  // null: nothing to launch
   unsigned grid, block;
@@ -207,10 +231,11 @@ struct UpdateKind {
   bool wall;
   bool ext;           // some map uses the exclusion area or the upper-bound layer
   bool persistent;
+  bool by_value;      // the kernels take a MapDesc
   uint32_t stencils;  // EM_F_* of the per-cell filters
   bool operator==(const UpdateKind& o) const {
     return ray_group == o.ray_group && ray == o.ray && drift == o.drift && wall == o.wall && ext == o.ext &&
-           persistent == o.persistent && stencils == o.stencils;
+           persistent == o.persistent && by_value == o.by_value && stencils == o.stencils;
   }
 };
 constexpr int kMaxLaunches = 16;
@@ -223,25 +248,28 @@ struct Sequence {
 };
 // The launches of an update in stream order; grids for n_points points and
 // n_cells (padded) cells, which bound what the descriptor holds.
+#define EM_KERNEL(k, by_value) ((by_value) ? (const void*)&k<MapDesc> : (const void*)&k<const BatchDev*>)
+constexpr int kValueGroup = 8;  // the one ray_group built for MapDesc
 Sequence update_sequence(const UpdateKind& k, int64_t n_points, int64_t n_cells);
-cudaError_t run(const Launch& l, const BatchDev* b, cudaStream_t s);
+// desc: the kernel's descriptor argument (a const BatchDev* or a MapDesc)
+cudaError_t run(const Launch& l, const void* desc, bool first, cudaStream_t s);
 // The sequence as a chain of kernel nodes.
 cudaError_t build_graph(const Sequence& q, const BatchDev* b, cudaGraph_t* out);
 
-Launch pre_launch(int64_t n_points, bool ext);
-Launch cells_launch(int64_t n_cells);
-Launch refresh_launch(int64_t n_cells);
-Launch points_launch(int64_t n_points, int group, bool ray, bool ext, int part);
-Launch write_launch(int64_t n_cells);
+Launch pre_launch(int64_t n_points, bool ext, bool by_value);
+Launch cells_launch(int64_t n_cells, bool by_value);
+Launch refresh_launch(int64_t n_cells, bool by_value);
+Launch points_launch(int64_t n_points, int group, bool ray, bool ext, int part, bool by_value);
+Launch write_launch(int64_t n_cells, bool by_value);
 // The whole update but the drift compensation and the stencils (points per
 // cell, thresholds, points, write) in one cooperative launch with grid
 // barriers; barrier waits are bounded by the descriptor's wait_budget.  fn is
 // null when the device cannot run it.
 Launch persist_launch(int group, bool ext);
 long long clock_budget(long long us);  // SM clock cycles of that many microseconds
-Launch normals_launch(int64_t n_cells);
-Launch smooth_launch(int64_t n_cells);
-Launch inpaint_launch(int64_t n_cells);
+Launch normals_launch(int64_t n_cells, bool by_value);
+Launch smooth_launch(int64_t n_cells, bool by_value);
+Launch inpaint_launch(int64_t n_cells, bool by_value);
 
 // ---- launchers of the other kernels (each returns cudaGetLastError())
 // The bounded wait of the persistent kernel on a word that nothing sets: one
@@ -266,6 +294,14 @@ cudaError_t launch_layers_in(const MapDev& m, uint32_t mask, const float* src, c
 cudaError_t launch_fill_map(const MapDev& m, cudaStream_t s);
 
 // ---- small device helpers shared by the kernels
+
+// Start of every kernel of an update: it may have been launched while the
+// kernel before it on the stream still ran (launch.cu), so it waits for that
+// one's end and memory, then lets the next one be launched in the same way.
+__device__ __forceinline__ void begin_after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+}
 
 __device__ __forceinline__ int32_t clamp_floor(float q) {
   float f = floorf(q);
@@ -338,13 +374,13 @@ __device__ __forceinline__ Grid own_grid() { return Grid{(int)blockIdx.x, (int)g
 
 // Iterate over the tiles of the cell space: for each tile the map it lies in
 // (block-uniform) and the tile's first physical cell.  body(m, map, p0, count).
-template <class F>
-__device__ __forceinline__ void for_each_tile(const struct BatchDev& b, Grid gr, F body) {
+template <class V, class F>
+__device__ __forceinline__ void for_each_tile(const V& b, Grid gr, F body) {
   const int64_t n_tiles = b.n_cells / kTile;
   for (int64_t t = gr.bid; t < n_tiles; t += gr.nb) {
     const int64_t g0 = t * kTile;
     const int mi = find_map_cell(b.maps, b.n_maps, g0);
-    const MapDev& m = b.maps[mi];
+    const MapDev& m = map_at(b, mi);
     const int64_t p0 = g0 - m.cell_begin;
     const int32_t ncell = m.W * m.H;
     if (p0 >= ncell) continue;  // padding at the end of a map
@@ -352,9 +388,4 @@ __device__ __forceinline__ void for_each_tile(const struct BatchDev& b, Grid gr,
     body(m, mi, (int32_t)p0, cnt);
   }
 }
-template <class F>
-__device__ __forceinline__ void for_each_tile(const struct BatchDev& b, F body) {
-  for_each_tile(b, own_grid(), body);
-}
-
 }  // namespace em

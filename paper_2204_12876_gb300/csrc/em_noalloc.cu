@@ -35,20 +35,12 @@ constexpr int kMaxCloudsNA = EM_NOALLOC_MAX_CLOUDS;
 
 constexpr size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// Everything one call's kernels read from the descriptor, passed by value to
-// k_put_desc (well below the 32 KB of a kernel's parameters).
-struct Desc {
-  BatchDev b;
-  MapDev m;
-  CloudDev c[kMaxCloudsNA];
-};
-static_assert(sizeof(Desc) <= 4096, "the descriptor travels as a kernel parameter");
+static_assert(kMaxCloudsNA <= kDescClouds, "the descriptor travels as a kernel parameter");
 
 // Scratch layout.  The part that must start at zero (control blocks, marks, tile
 // flags and the accumulators of this call's cells) is contiguous, so one memset
 // as long as the map is clears it.
-constexpr size_t kOffDesc = 0;
-constexpr size_t kOffCtl = kOffDesc + up256(sizeof(Desc));
+constexpr size_t kOffCtl = 0;
 constexpr size_t kOffBCtl = kOffCtl + up256(sizeof(MapCtl));
 constexpr size_t kOffZero = kOffBCtl + up256(sizeof(BatchCtl));  // the map's part of the zeroed scratch
 struct Layout {
@@ -81,15 +73,6 @@ unsigned char* g_addr[kMaxDevices] = {};
 // The scratch itself.  In host code this name is only a stand-in for the
 // device array: its device address comes from cudaGetSymbolAddress.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
-
-// The descriptor, from the kernel's parameters into the front of the scratch
-// (the kernels that follow on the stream read it there).
-static_assert(kOffDesc == 0 && sizeof(Desc) % 4 == 0, "word copy of the descriptor");
-__global__ void k_put_desc(const Desc d) {
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(&d);
-  uint32_t* dst = reinterpret_cast<uint32_t*>(g_noalloc_scratch + kOffDesc);
-  for (int i = threadIdx.x; i < (int)(sizeof(Desc) / 4); i += blockDim.x) dst[i] = src[i];
-}
 
 namespace {
 
@@ -159,8 +142,8 @@ extern "C" int em_update_noalloc(const em_params* params, int64_t shift_x, int64
   cudaStream_t s = (cudaStream_t)stream;
   const int32_t W = params->width, H = params->height, ncell = W * H;
 
-  // descriptor, built here and handed to k_put_desc by value
-  Desc desc;
+  // descriptor, built here and handed to every kernel by value
+  MapDesc desc;
   memset(&desc, 0, sizeof(desc));
   BatchDev* b = &desc.b;
   MapDev* m = &desc.m;
@@ -218,23 +201,18 @@ extern "C" int em_update_noalloc(const em_params* params, int64_t shift_x, int64
   b->n_maps = 1;
   b->n_clouds = n_clouds;
   b->n_points = total;
-  b->maps = reinterpret_cast<const MapDev*>(base + kOffDesc + offsetof(Desc, m));
-  b->clouds = reinterpret_cast<const CloudDev*>(base + kOffDesc + offsetof(Desc, c));
   b->n_cells = pad_tile(ncell);
   b->n_items = (int64_t)m->IW * m->IH;
   b->ctl = reinterpret_cast<BatchCtl*>(base + kOffBCtl);
 
-  const BatchDev* bd = reinterpret_cast<const BatchDev*>(base + kOffDesc + offsetof(Desc, b));
-  k_put_desc<<<1, 128, 0, s>>>(desc);
-  rc = na_status(cudaGetLastError(), "k_put_desc");
-  if (rc) return rc;
   rc = na_status(cudaMemsetAsync(base + kOffCtl, 0, lay.thr - kOffCtl, s), "cudaMemsetAsync");
   if (rc) return rc;
   const int64_t cells = pad_tile(ncell);
-  UpdateKind kind = params_kind(*params, 8);
+  UpdateKind kind = params_kind(*params, kValueGroup);
   kind.stencils = 0;  // not the per-cell filters
+  kind.by_value = true;
   const Sequence q = update_sequence(kind, total, cells);
   cudaError_t e = cudaSuccess;
-  for (int i = 0; i < q.n && e == cudaSuccess; ++i) e = run(q.k[i], bd, s);
+  for (int i = 0; i < q.n && e == cudaSuccess; ++i) e = run(q.k[i], &desc, i == 0, s);
   return na_status(e, "em_update_noalloc launch");
 }

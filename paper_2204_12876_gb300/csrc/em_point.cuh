@@ -137,7 +137,8 @@ __device__ __forceinline__ void load_point(const CloudDev& c, int64_t i, float& 
 // stride 4 -> one float4 per lane; stride 3 -> 24 float4 staged in shared memory.
 // `hint` is the cloud of the warp's previous chunk (-1: none); it becomes the
 // cloud of this chunk's first point.
-__device__ __forceinline__ int load_warp_points(const BatchDev& b, int64_t wbase, int64_t end, float4* stage,
+template <class V>
+__device__ __forceinline__ int load_warp_points(const V& b, int64_t wbase, int64_t end, float4* stage,
                                                 float& px, float& py, float& pz, int& hint) {
   const int lane = threadIdx.x & 31;
   const int64_t g = wbase + lane;

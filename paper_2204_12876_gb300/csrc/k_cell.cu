@@ -21,19 +21,25 @@ namespace em {
 // and the square roots), DRAM-bound on many (31 us for the 64-map batch's 6.8 M
 // cells).  It takes the place of a threshold pass in the point kernel and a
 // one-thread-per-block coarse kernel (12 us alone on one map).
-__global__ void __launch_bounds__(kCellThreads) k_cells(const BatchDev* __restrict__ bp) {
-  cells_pass(*bp, own_grid());
+template <class D>
+__global__ void __launch_bounds__(kCellThreads) k_cells(const __grid_constant__ D d) {
+  begin_after_previous();
+  cells_pass(view(d), own_grid());
 }
 
 // DRAM-bound on many maps (427 MB in 135 us for the 64-map batch: 36 bytes of
 // sums and 12 of state per touched cell, read and written); 8-12 us cold on one.
-__global__ void __launch_bounds__(kCellThreads) k_write(const BatchDev* __restrict__ bp) {
-  write_pass(*bp, own_grid());
+template <class D>
+__global__ void __launch_bounds__(kCellThreads) k_write(const __grid_constant__ D d) {
+  begin_after_previous();
+  write_pass(view(d), own_grid());
 }
 
 // Skips (one load a block) when the points went in one part.
-__global__ void __launch_bounds__(kCellThreads) k_refresh(const BatchDev* __restrict__ bp) {
-  refresh_pass(*bp, own_grid());
+template <class D>
+__global__ void __launch_bounds__(kCellThreads) k_refresh(const __grid_constant__ D d) {
+  begin_after_previous();
+  refresh_pass(view(d), own_grid());
 }
 
 // n_cells bounds the items but for partial last rows and columns (the pass strides over the grid)
@@ -43,16 +49,18 @@ static Launch item_launch(const void* fn, int64_t n_cells, int slot, const char*
   const int64_t cap = (int64_t)sm_count() * 16;
   return {fn, (unsigned)(blocks < cap ? blocks : cap), kThreads, 0, false, slot, name, 0};
 }
-Launch cells_launch(int64_t n_cells) { return item_launch((const void*)&k_cells, n_cells, EM_PROF_COUNT, "k_cells"); }
-Launch refresh_launch(int64_t n_cells) {
-  return item_launch((const void*)&k_refresh, n_cells, EM_PROF_RAY, "k_refresh");
+Launch cells_launch(int64_t n_cells, bool by_value) {
+  return item_launch(EM_KERNEL(k_cells, by_value), n_cells, EM_PROF_COUNT, "k_cells");
+}
+Launch refresh_launch(int64_t n_cells, bool by_value) {
+  return item_launch(EM_KERNEL(k_refresh, by_value), n_cells, EM_PROF_RAY, "k_refresh");
 }
 
-Launch write_launch(int64_t n_cells) {
+Launch write_launch(int64_t n_cells, bool by_value) {
   const int64_t tiles = n_cells / kTile;  // a block per tile
   const int64_t cap = (int64_t)sm_count() * 8;
   const unsigned grid = (unsigned)(tiles < 1 ? 1 : tiles < cap ? tiles : cap);
-  return {(const void*)&k_write, grid, kCellThreads, 0, false, EM_PROF_FUSE, "k_write"};
+  return {EM_KERNEL(k_write, by_value), grid, kCellThreads, 0, false, EM_PROF_FUSE, "k_write", 0};
 }
 
 }  // namespace em

@@ -30,11 +30,13 @@ __device__ __forceinline__ bool valid_at(const MapDev& m, int32_t p) { return is
 constexpr int kNmT = 32, kNmSpan = kNmT + 2;
 static_assert(kNmT * kNmT == 4 * kMapThreads, "k_normals: four cells per thread");
 
-__global__ void __launch_bounds__(kMapThreads) k_normals(const BatchDev* __restrict__ bp) {
+template <class D>
+__global__ void __launch_bounds__(kMapThreads) k_normals(const __grid_constant__ D d) {
   __shared__ float s_h[kNmSpan][kNmSpan + 1];
-  const BatchDev& b = *bp;
+  begin_after_previous();
+  const auto& b = view(d);
   for (int mi = 0; mi < b.n_maps; ++mi) {
-    const MapDev& m = b.maps[mi];
+    const MapDev& m = map_at(b, mi);
     if (!m.nx || !(m.flags & EM_F_NORMALS)) continue;  // a batch may mix maps with and without normals
     const int32_t ntx = (m.W + kNmT - 1) / kNmT, nty = (m.H + kNmT - 1) / kNmT;
     for (int32_t tile = blockIdx.x; tile < ntx * nty; tile += gridDim.x) {
@@ -104,11 +106,13 @@ __global__ void __launch_bounds__(kMapThreads) k_normals(const BatchDev* __restr
 constexpr int kSmT = 32, kSmRim = 2, kSmSpan = kSmT + 2 * kSmRim;
 static_assert(kSmT * kSmT == 4 * kMapThreads, "k_smooth: four cells per thread");
 
-__global__ void __launch_bounds__(kMapThreads) k_smooth(const BatchDev* __restrict__ bp) {
+template <class D>
+__global__ void __launch_bounds__(kMapThreads) k_smooth(const __grid_constant__ D d) {
   __shared__ float s_h[kSmSpan][kSmSpan + 1];
-  const BatchDev& b = *bp;
+  begin_after_previous();
+  const auto& b = view(d);
   for (int mi = 0; mi < b.n_maps; ++mi) {
-    const MapDev& m = b.maps[mi];
+    const MapDev& m = map_at(b, mi);
     if (!m.smooth) continue;
     const int mode = (m.flags & EM_F_MEDIAN) ? 1 : (m.flags & EM_F_GAUSS) ? 2 : 0;
     const int32_t ntx = (m.W + kSmT - 1) / kSmT, nty = (m.H + kSmT - 1) / kSmT;
@@ -251,15 +255,17 @@ __device__ float inpaint_cell(const MapDev& m, const uint64_t* rows, int i, int 
   return mn;
 }
 
-__global__ void __launch_bounds__(kMapThreads, 4) k_inpaint(const BatchDev* __restrict__ bp) {
+template <class D>
+__global__ void __launch_bounds__(kMapThreads, 4) k_inpaint(const __grid_constant__ D d) {
   __shared__ uint64_t s_rows[kIpSpan];
   __shared__ uint64_t s_cols[kIpSpan];      // the same bits by column
   __shared__ uint16_t s_queue[kIpT * kIpT];  // tile cells that need the search
   __shared__ int s_queued;
-  const BatchDev& b = *bp;
+  begin_after_previous();
+  const auto& b = view(d);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int mi = 0; mi < b.n_maps; ++mi) {
-    const MapDev& m = b.maps[mi];
+    const MapDev& m = map_at(b, mi);
     if (!m.inpaint) continue;
     const int32_t ntx = (m.W + kIpT - 1) / kIpT, nty = (m.H + kIpT - 1) / kIpT;
     for (int32_t tile = blockIdx.x; tile < ntx * nty; tile += gridDim.x) {
@@ -438,11 +444,17 @@ static int tile_grid(int64_t n_cells) {
 }
 
 static Launch stencil(const void* fn, int64_t n_cells, int slot, const char* name) {
-  return {fn, (unsigned)tile_grid(n_cells), kMapThreads, 0, false, slot, name};
+  return {fn, (unsigned)tile_grid(n_cells), kMapThreads, 0, false, slot, name, 0};
 }
-Launch normals_launch(int64_t n_cells) { return stencil((const void*)&k_normals, n_cells, EM_PROF_NORMALS, "k_normals"); }
-Launch smooth_launch(int64_t n_cells) { return stencil((const void*)&k_smooth, n_cells, EM_PROF_SMOOTH, "k_smooth"); }
-Launch inpaint_launch(int64_t n_cells) { return stencil((const void*)&k_inpaint, n_cells, EM_PROF_INPAINT, "k_inpaint"); }
+Launch normals_launch(int64_t n_cells, bool by_value) {
+  return stencil(EM_KERNEL(k_normals, by_value), n_cells, EM_PROF_NORMALS, "k_normals");
+}
+Launch smooth_launch(int64_t n_cells, bool by_value) {
+  return stencil(EM_KERNEL(k_smooth, by_value), n_cells, EM_PROF_SMOOTH, "k_smooth");
+}
+Launch inpaint_launch(int64_t n_cells, bool by_value) {
+  return stencil(EM_KERNEL(k_inpaint, by_value), n_cells, EM_PROF_INPAINT, "k_inpaint");
+}
 
 cudaError_t launch_shift_clear(const MapDev& m, int32_t dx, int32_t dy, cudaStream_t s) {
   int32_t cx0 = 0, cx1 = 0, ry0 = 0, ry1 = 0;

@@ -65,6 +65,7 @@ template <int G, bool kExt>
 __global__ void __launch_bounds__(kPersistThreads, 4) k_persist(const BatchDev* __restrict__ bp) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int s_ok;
+  begin_after_previous();
   const BatchDev& b = *bp;
   const long long budget = b.wait_budget;
   const int nb = gridDim.x, bid = blockIdx.x;
@@ -126,7 +127,7 @@ Launch persist_launch_t() {
     n = v > 0 ? v : -1;
   }
   if (n < 0) return {};
-  return {fn, (unsigned)(n * sm_count()), kPersistThreads, kPersistSmem, true, EM_PROF_PERSIST, "k_persist"};
+  return {fn, (unsigned)(n * sm_count()), kPersistThreads, kPersistSmem, true, EM_PROF_PERSIST, "k_persist", 0};
 }
 
 template <bool kExt>

@@ -47,16 +47,18 @@
 
 namespace em {
 
-template <bool kExt>
-__global__ void __launch_bounds__(kPointThreads) k_pre(const BatchDev* __restrict__ bp) {
+template <bool kExt, class D>
+__global__ void __launch_bounds__(kPointThreads) k_pre(const __grid_constant__ D d) {
   __shared__ PreSmem S;
-  pre_pass<kExt>(*bp, own_grid(), S);
+  begin_after_previous();
+  pre_pass<kExt>(view(d), own_grid(), S);
 }
 
-template <int G, bool kRay, bool kExt>
-__global__ void __launch_bounds__(kPointThreads, 4) k_points(const BatchDev* __restrict__ bp, int part) {
+template <int G, bool kRay, bool kExt, class D>
+__global__ void __launch_bounds__(kPointThreads, 4) k_points(const __grid_constant__ D d, int part) {
   __shared__ PointsSmem<kRay> S;
-  points_pass<G, kRay, kExt>(*bp, own_grid(), part, S);
+  begin_after_previous();
+  points_pass<G, kRay, kExt>(view(d), own_grid(), part, S);
 }
 
 int sm_count() {
@@ -78,29 +80,42 @@ static int point_grid(int64_t n, int per_sm) {
   return (int)(want < 1 ? 1 : want < cap ? want : cap);
 }
 
-Launch pre_launch(int64_t n_points, bool ext) {
+Launch pre_launch(int64_t n_points, bool ext, bool by_value) {
   if (n_points <= 0) return {};
-  return {ext ? (const void*)&k_pre<true> : (const void*)&k_pre<false>, (unsigned)point_grid(n_points, 16),
-          kPointThreads, 0, false, EM_PROF_SCATTER, "k_pre"};
+  const void* fn = by_value ? (ext ? (const void*)&k_pre<true, MapDesc> : (const void*)&k_pre<false, MapDesc>)
+                   : ext    ? (const void*)&k_pre<true, const BatchDev*>
+                            : (const void*)&k_pre<false, const BatchDev*>;
+  return {fn, (unsigned)point_grid(n_points, 16), kPointThreads, 0, false, EM_PROF_SCATTER, "k_pre", 0};
 }
 
 template <bool kExt>
 static const void* points_kernel(int g) {
   switch (g) {
-    case 1: return (const void*)&k_points<1, true, kExt>;
-    case 2: return (const void*)&k_points<2, true, kExt>;
-    case 4: return (const void*)&k_points<4, true, kExt>;
-    case 16: return (const void*)&k_points<16, true, kExt>;
-    case 32: return (const void*)&k_points<32, true, kExt>;
-    default: return (const void*)&k_points<8, true, kExt>;
+    case 1: return (const void*)&k_points<1, true, kExt, const BatchDev*>;
+    case 2: return (const void*)&k_points<2, true, kExt, const BatchDev*>;
+    case 4: return (const void*)&k_points<4, true, kExt, const BatchDev*>;
+    case 16: return (const void*)&k_points<16, true, kExt, const BatchDev*>;
+    case 32: return (const void*)&k_points<32, true, kExt, const BatchDev*>;
+    default: return (const void*)&k_points<8, true, kExt, const BatchDev*>;
   }
 }
+// The descriptor by value: kValueGroup samples per chunk only.
+template <bool kRay, bool kExt>
+static const void* points_kernel_value() {
+  return (const void*)&k_points<kValueGroup, kRay, kExt, MapDesc>;
+}
 
-Launch points_launch(int64_t n_points, int group, bool ray, bool ext, int part) {
+Launch points_launch(int64_t n_points, int group, bool ray, bool ext, int part, bool by_value) {
   if (n_points <= 0) return {};
-  const void* fn = ray ? (ext ? points_kernel<true>(group) : points_kernel<false>(group))
-                   : ext ? (const void*)&k_points<8, false, true>
-                         : (const void*)&k_points<8, false, false>;
+  const void* fn;
+  if (by_value)
+    fn = ray ? (ext ? points_kernel_value<true, true>() : points_kernel_value<true, false>())
+         : ext ? points_kernel_value<false, true>()
+               : points_kernel_value<false, false>();
+  else
+    fn = ray ? (ext ? points_kernel<true>(group) : points_kernel<false>(group))
+         : ext ? (const void*)&k_points<8, false, true, const BatchDev*>
+               : (const void*)&k_points<8, false, false, const BatchDev*>;
   return {fn, (unsigned)point_grid(n_points, 4), kPointThreads, 0, false, EM_PROF_RAY, "k_points", part};
 }
 

@@ -55,8 +55,8 @@ struct PreSmem {
 // drift compensation (Section II-D) the errors of the points in flat cells
 // that hold an estimate (previous normal n_z >= drift_flatness; a NaN normal is
 // not flat), summed exactly per map.
-template <bool kExt>
-__device__ __forceinline__ void pre_pass(const BatchDev& b, Grid gr, PreSmem& S) {
+template <bool kExt, class V>
+__device__ __forceinline__ void pre_pass(const V& b, Grid gr, PreSmem& S) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int64_t beg, end;
   block_range(b.n_points, gr, beg, end);
@@ -68,13 +68,13 @@ __device__ __forceinline__ void pre_pass(const BatchDev& b, Grid gr, PreSmem& S)
     const int c0 = find_cloud(b.clouds, b.n_clouds, wbase, hint);
     hint = c0;
     const CloudDev& cl0 = b.clouds[c0];
-    const MapDev& m0 = b.maps[cl0.map];
+    const MapDev& m0 = map_at(b, cl0.map);
     if (wbase + 32 <= cl0.begin + cl0.n && m0.drift_flat <= 0.f && !m0.cnt) continue;  // nothing for a whole warp
     float px, py, pz;
     const int ci = load_warp_points(b, wbase, end, S.stage[warp], px, py, pz, hint);
     const int64_t g = wbase + lane;
     const CloudDev& c = b.clouds[ci];
-    const MapDev& m = b.maps[c.map];
+    const MapDev& m = map_at(b, c.map);
     const PointGeom pg = point_geom<kExt>(m, c, px, py, pz);
     const bool inm = g < end && pg.in_range && in_map(m, pg.ix, pg.iy);
     const int32_t key = inm ? phys_index(m, pg.ix, pg.iy) : 0;
@@ -87,7 +87,7 @@ __device__ __forceinline__ void pre_pass(const BatchDev& b, Grid gr, PreSmem& S)
       const float var = m.var[key], nz = m.nz[key], hc = m.h[key];
       if (isfinite(var) && nz >= m.drift_flat) {
         if (c.map != dmap) {
-          if (dmap >= 0) drift_add(b.maps[dmap], dh, dl, dn);
+          if (dmap >= 0) drift_add(map_at(b, dmap), dh, dl, dn);
           dmap = c.map;
           dh = 0;
           dl = dn = 0;
@@ -131,10 +131,10 @@ __device__ __forceinline__ void pre_pass(const BatchDev& b, Grid gr, PreSmem& S)
         tl += S.l[w];
         tn += S.n[w];
       }
-      drift_add(b.maps[bm], th, tl, tn);
+      drift_add(map_at(b, bm), th, tl, tn);
     }
   } else if (dmap >= 0 && dn) {
-    drift_add(b.maps[dmap], dh, dl, dn);
+    drift_add(map_at(b, dmap), dh, dl, dn);
   }
   __syncthreads();  // the shared memory is free again
 }
@@ -241,9 +241,10 @@ __device__ __forceinline__ int stat_of(int k) {
          : k == kPsWall     ? kStWall
                             : kStRaySamples;
 }
-__device__ __forceinline__ void add_counts(const BatchDev& b, int map, unsigned long long v) {
+template <class V>
+__device__ __forceinline__ void add_counts(const V& b, int map, unsigned long long v) {
   const int lane = threadIdx.x & 31;
-  if (map >= 0 && lane < kPointStats && v) atomicAdd(&b.maps[map].ctl->stats[stat_of(lane)], v);
+  if (map >= 0 && lane < kPointStats && v) atomicAdd(&map_at(b, map).ctl->stats[stat_of(lane)], v);
 }
 
 // ---- the rays
@@ -337,9 +338,9 @@ __device__ __forceinline__ void put_ray(RaySmem& S, int t, const RaySetup& r) {
 // both dies read while others write it costs far more than the looks it saves
 // (thresholds or block flags updated in place took the 64-map batch from 4.0 to
 // 6.3 ms and one depth frame from 59 to 112 us).
-template <bool kExt>
-__device__ __forceinline__ void mark_sample(const BatchDev& b, const RaySmem& S, int sr, uint32_t k) {
-  const MapDev& m = b.maps[S.map[sr]];
+template <bool kExt, class V>
+__device__ __forceinline__ void mark_sample(const V& b, const RaySmem& S, int sr, uint32_t k) {
+  const MapDev& m = map_at(b, S.map[sr]);
   const float kf = (float)k;
   // the sample again, by the march's rounded arithmetic
   const int32_t cx = cell_of(__fmaf_rn(kf, S.bx[sr], S.ax[sr])), cy = cell_of(__fmaf_rn(kf, S.by[sr], S.ay[sr]));
@@ -375,8 +376,8 @@ __device__ __forceinline__ void mark_sample(const BatchDev& b, const RaySmem& S,
 // another; the warp queues the chunks that may mark a cell and marches them
 // 4 x 32 / G at a time, G lanes per chunk and one sample per lane and round
 // (4 gathers in flight).
-template <int G, bool kRay, bool kExt>
-__device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, int part, PointsSmem<kRay>& SM) {
+template <int G, bool kRay, bool kExt, class V>
+__device__ __forceinline__ void points_pass(const V& b, Grid gr, int part, PointsSmem<kRay>& SM) {
   constexpr int kU = G >= 4 ? 4 : G;         // samples per lane and march round, all of one chunk
   constexpr int kLPC = G / kU;               // lanes per chunk in the march
   constexpr int kFQ = 32 / kLPC;             // chunks per march round (at most 32)
@@ -420,7 +421,7 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, int part
     const bool live = g < n_points;
     const CloudDev& c = b.clouds[ci];
     const int32_t map = c.map;
-    const MapDev& m = b.maps[map];
+    const MapDev& m = map_at(b, map);
     const PointGeom pg = point_geom<kExt>(m, c, px, py, pz);
     const bool inm = live && pg.in_range && in_map(m, pg.ix, pg.iy);
     const uint32_t cell = inm ? (uint32_t)phys_index(m, pg.ix, pg.iy) : 0u;
@@ -563,7 +564,7 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, int part
       // exact), so neighbouring chunks share an end and its block.  Blocks
       // outside the map are those of the grid's rim, which holds -inf.  All loads
       // of the round come first (no branches between them), then the tests.
-      const MapDev& m = b.maps[S.map[sr]];
+      const MapDev& m = map_at(b, S.map[sr]);
       const float* ct = m.cthr;
       const int32_t CW = m.CW, CH = m.CH, CS = m.CS;
       int32_t xb[kCU + 1], yb[kCU + 1];
@@ -605,7 +606,7 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, int part
         const int2 e = Q.chunk[(qh + qi) & (kQ - 1)];
         const int32_t ne = qi < qn ? e.x >> 8 : 0;
         const int mr = qi < qn ? e.x & 31 : 0, sm = wb + mr;
-        const MapDev& mm = b.maps[S.map[sm]];
+        const MapDev& mm = map_at(b, S.map[sm]);
         const int32_t Wm = mm.W, Hm = mm.H;
         const float* tm = mm.thr;
         const float mx0 = S.ax[sm], mbx = S.bx[sm], my0 = S.ay[sm], mby = S.by[sm], mz0 = S.az[sm], mbz = S.bz[sm];
@@ -677,7 +678,7 @@ __device__ __forceinline__ void points_pass(const BatchDev& b, Grid gr, int part
   }
   __syncthreads();
   if (threadIdx.x < kPointStats && F.map >= 0 && F.sum[threadIdx.x])
-    atomicAdd(&b.maps[F.map].ctl->stats[stat_of(threadIdx.x)], F.sum[threadIdx.x]);
+    atomicAdd(&map_at(b, F.map).ctl->stats[stat_of(threadIdx.x)], F.sum[threadIdx.x]);
   __syncthreads();  // the shared memory is free again
 }
 
