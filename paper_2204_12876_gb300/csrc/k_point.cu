@@ -74,8 +74,9 @@ int sm_count() {
   return cached[dev];
 }
 
-static int point_grid(int64_t n, int per_sm) {
-  const int64_t want = (n + kPointThreads - 1) / kPointThreads;  // one 32-point batch per warp
+// Blocks for n points, `span` of them per warp at least.
+static int point_grid(int64_t n, int span, int per_sm) {
+  const int64_t want = (n + span * kPointWarps - 1) / (span * kPointWarps);
   const int64_t cap = (int64_t)sm_count() * per_sm;
   return (int)(want < 1 ? 1 : want < cap ? want : cap);
 }
@@ -85,7 +86,7 @@ Launch pre_launch(int64_t n_points, bool ext, bool by_value) {
   const void* fn = by_value ? (ext ? (const void*)&k_pre<true, MapDesc> : (const void*)&k_pre<false, MapDesc>)
                    : ext    ? (const void*)&k_pre<true, const BatchDev*>
                             : (const void*)&k_pre<false, const BatchDev*>;
-  return {fn, (unsigned)point_grid(n_points, 16), kPointThreads, 0, false, EM_PROF_SCATTER, "k_pre", 0};
+  return {fn, (unsigned)point_grid(n_points, 32, 16), kPointThreads, 0, false, EM_PROF_SCATTER, "k_pre", 0};
 }
 
 template <bool kExt>
@@ -116,7 +117,7 @@ Launch points_launch(int64_t n_points, int group, bool ray, bool ext, int part, 
     fn = ray ? (ext ? points_kernel<true>(group) : points_kernel<false>(group))
          : ext ? (const void*)&k_points<8, false, true, const BatchDev*>
                : (const void*)&k_points<8, false, false, const BatchDev*>;
-  return {fn, (unsigned)point_grid(n_points, 4), kPointThreads, 0, false, EM_PROF_RAY, "k_points", part};
+  return {fn, (unsigned)point_grid(n_points, kMinSpan, 4), kPointThreads, 0, false, EM_PROF_RAY, "k_points", part};
 }
 
 }  // namespace em

@@ -16,7 +16,8 @@ namespace em {
 
 constexpr int kPointThreads = 256;
 constexpr int kPointWarps = kPointThreads / 32;
-constexpr int kRayRun = 8;  // 32-point batches per take from the work counter, at most
+constexpr int kRayRun = 8;  // batches per take from the work counter, at most
+constexpr uint32_t kMinSpan = 8;
 
 // Large updates whose points come in no order go through them in parts, the
 // first ones small: between them k_refresh takes the marked cells out of the
@@ -358,9 +359,15 @@ __device__ __forceinline__ void mark_sample(const V& b, const RaySmem& S, int sr
   // cost a redundant atomic, never a lost mark)
   uint32_t* const word = m.mark + (p >> 5);
   const uint32_t bit = 1u << (p & 31);
+  const bool guard = m.alpha_n > 0.f;
+  float n0 = 0.f, n1 = 0.f, n2 = 1.f;
+  if (guard) {  // (read with the mark, not after it)
+    n0 = m.nx[p];
+    n1 = m.ny[p];
+    n2 = m.nz[p];
+  }
   if (*word & bit) return;
-  if (m.alpha_n > 0.f) {  // Eq. 4
-    float n0 = m.nx[p], n1 = m.ny[p], n2 = m.nz[p];
+  if (guard) {  // Eq. 4
     if (!(isfinite(n0) && isfinite(n1) && isfinite(n2))) { n0 = 0.f; n1 = 0.f; n2 = 1.f; }
     const float rd = S.d[sr];
     const float rx = __fdiv_rn(S.vx[sr], rd), ry = __fdiv_rn(S.vy[sr], rd), rz = __fdiv_rn(S.vz[sr], rd);
@@ -401,8 +408,15 @@ __device__ __forceinline__ void points_pass(const V& b, Grid gr, int part, Point
   } else if (part > 0) {
     return;
   }
+  // A batch is 32 points, or 16 or 8 while that leaves every warp at most one: a
+  // small update is as slow as its slowest warp, and the tests and the march of
+  // fewer rays are spread over the same 32 lanes (43,018 points of two dome
+  // LiDARs: 64 -> 57 us an update).  Two batches per warp gave those 54 us, but
+  // 76,800 points of a camera 33 for 28; batches of 4 gain nothing more.
   const uint32_t warps = (uint32_t)gr.nb * kPointWarps;
-  uint32_t n_batches = (n_points + 31) / 32;
+  uint32_t span = 32;
+  while (span > kMinSpan && (n_points + span / 2 - 1) / (span / 2) <= warps) span /= 2;
+  uint32_t n_batches = (n_points + span - 1) / span;
   if (len < 32) n_batches = (n_batches + 31) / 32 * len;
   const uint32_t run_len = max(1u, min((uint32_t)kRayRun, n_batches / (2 * warps)));
   const uint32_t n_runs = (n_batches + run_len - 1) / run_len;
@@ -413,12 +427,13 @@ __device__ __forceinline__ void points_pass(const V& b, Grid gr, int part, Point
   uint32_t index = run * run_len;
   while (run < n_runs) {
     const uint32_t batch = len < 32 ? index / len * 32 + (__brev(first + index % len) >> 27) : index;
-    if (batch * 32 < n_points) {
+    const uint32_t p0 = batch * span;
+    if (p0 < n_points) {
     // ---- the points: transform, gate, sums
     float px, py, pz;
-    const int ci = load_warp_points(b, (int64_t)batch * 32, n_points, SM.w[warp].stage, px, py, pz, hint);
-    const uint32_t g = batch * 32 + lane;
-    const bool live = g < n_points;
+    const uint32_t p1 = min(p0 + span, n_points), g = p0 + lane;
+    const int ci = load_warp_points(b, p0, p1, SM.w[warp].stage, px, py, pz, hint);
+    const bool live = g < p1;
     const CloudDev& c = b.clouds[ci];
     const int32_t map = c.map;
     const MapDev& m = map_at(b, map);
