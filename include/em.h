@@ -233,9 +233,9 @@ enum {
   EM_PROF_SCATTER,     /* k_pre: points per cell for the wall rule, drift sums */
   EM_PROF_FUSE,        /* k_write: new state of every cell, removal, overlap clearance */
   EM_PROF_CLEAR,       /* (no kernel) */
-  EM_PROF_NORMALS,
-  EM_PROF_SMOOTH,
-  EM_PROF_INPAINT,
+  EM_PROF_NORMALS,     /* k_stencils: normals, smoothing, in-painting */
+  EM_PROF_SMOOTH,      /* (no kernel) */
+  EM_PROF_INPAINT,     /* (no kernel) */
   EM_PROF_DRIFT,       /* (no kernel) */
   EM_PROF_OVERLAP,     /* (no kernel) */
   EM_PROF_PERSIST,     /* k_persist: the passes of a batched update in one launch (EM_BATCH_PERSISTENT) */

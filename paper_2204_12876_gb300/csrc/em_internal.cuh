@@ -26,7 +26,7 @@
 //              against the pre-update thresholds       (Section II-E)
 //   k_write    per cell: Eq. 1/2 in information form from the sums; removal of
 //              penetrated cells not written recently   (Section II-C, II-E, II-F)
-//   k_normals / k_smooth / k_inpaint                   (Section II-A, II-I)
+//   k_stencils normals, smoothing, in-painting         (Section II-A, II-I)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -267,9 +267,7 @@ Launch write_launch(int64_t n_cells, bool by_value);
 // null when the device cannot run it.
 Launch persist_launch(int group, bool ext);
 long long clock_budget(long long us);  // SM clock cycles of that many microseconds
-Launch normals_launch(int64_t n_cells, bool by_value);
-Launch smooth_launch(int64_t n_cells, bool by_value);
-Launch inpaint_launch(int64_t n_cells, bool by_value);
+Launch stencils_launch(int64_t n_cells, bool by_value);
 
 // ---- launchers of the other kernels (each returns cudaGetLastError())
 // The bounded wait of the persistent kernel on a word that nothing sets: one

@@ -22,9 +22,7 @@ Sequence update_sequence(const UpdateKind& k, int64_t n_points, int64_t n_cells)
     }
     q.add(write_launch(n_cells, k.by_value));
   }
-  if (k.stencils & EM_F_NORMALS) q.add(normals_launch(n_cells, k.by_value));
-  if (k.stencils & (EM_F_SMOOTH | EM_F_MEDIAN | EM_F_GAUSS)) q.add(smooth_launch(n_cells, k.by_value));
-  if (k.stencils & EM_F_INPAINT) q.add(inpaint_launch(n_cells, k.by_value));
+  if (k.stencils) q.add(stencils_launch(n_cells, k.by_value));
   return q;
 }
 

@@ -26,7 +26,7 @@ LAYER_SMOOTH, LAYER_INPAINT, LAYER_VALID, LAYER_VARIANCE_NOW, LAYER_UPPER = 64, 
 PROF_SLOTS = ("count", "ray", "alloc", "scatter", "fuse", "clear", "normals", "smooth", "inpaint", "drift",
               "overlap", "persist")
 KERNEL_NAMES = {"count": "k_cells", "ray": "k_points", "alloc": "(none)", "scatter": "k_pre", "fuse": "k_write",
-                "clear": "(none)", "normals": "k_normals", "smooth": "k_smooth", "inpaint": "k_inpaint",
+                "clear": "(none)", "normals": "k_stencils", "smooth": "(none)", "inpaint": "(none)",
                 "drift": "(none)", "overlap": "(none)", "persist": "k_persist"}
 LAYER_NAMES = {LAYER_ELEVATION: "h", LAYER_VARIANCE: "var", LAYER_TIME: "t_last", LAYER_NORMAL_X: "nx",
                LAYER_NORMAL_Y: "ny", LAYER_NORMAL_Z: "nz", LAYER_SMOOTH: "smooth", LAYER_INPAINT: "inpaint",
