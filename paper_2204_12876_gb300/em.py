@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from dataclasses import dataclass, fields
 
 import numpy as np
@@ -153,25 +154,40 @@ class Params:
         return _Params(**{f.name: getattr(self, f.name) for f in fields(self)})
 
 
+_t = None  # torch, imported on first use (the module loads without it)
+
+
+def _torch():
+    global _t
+    if _t is None:
+        import torch
+        _t = torch
+    return _t
+
+
 def _stream_handle(stream) -> int | None:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        t = _torch()
+        raw = getattr(t._C, "_cuda_getCurrentRawStream", None)  # the same handle without a Stream object
+        return raw(t.cuda.current_device()) if raw else t.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
 
 
-def _torch():
-    import torch  # imported on first use (the module loads without it)
-    return torch
-
-
 _F12 = ctypes.c_float * 12
+_NF32 = np.dtype(np.float32)
+
+
+def _pose_bytes(pose) -> bytes:
+    """A pose's 12 float32 values, row-major."""
+    if type(pose) is np.ndarray and pose.dtype == _NF32 and pose.size == 12:
+        return pose.tobytes()
+    return np.ascontiguousarray(pose, dtype=np.float32).reshape(12).tobytes()
 
 
 def _pose(pose) -> ctypes.Array:
-    return _F12.from_buffer_copy(np.ascontiguousarray(pose, dtype=np.float32).reshape(12))
+    return _F12.from_buffer_copy(_pose_bytes(pose))
 
 
 def _cloud_struct(pts, pose, host: bool, any_device: bool = False) -> _Cloud:
@@ -217,11 +233,12 @@ class Map:
 
     def update(self, points, pose, stream=None):
         """Fuse one device cloud: points is a float32 CUDA tensor (n, 3|4)."""
-        if points.dtype.__str__() != "torch.float32" or not points.is_cuda or not points.is_contiguous():
+        if points.dtype is not _torch().float32 or not points.is_cuda or not points.is_contiguous():
             raise ValueError("points must be a contiguous float32 CUDA tensor of shape (n, 3) or (n, 4)")
         n, stride = points.shape
-        _check(lib.em_update(self._h, points.data_ptr(), n, stride, _pose(pose), _stream_handle(stream)),
-               "em_update")
+        rc = lib.em_update(self._h, points.data_ptr(), n, stride, _pose(pose), _stream_handle(stream))
+        if rc:
+            _check(rc, "em_update")
 
     def update_multi(self, clouds, stream=None):
         """One update from several device clouds [(tensor, pose), ...]."""
@@ -239,8 +256,8 @@ class Map:
 
     def get_layers(self, mask: int, out=None, stream=None):
         """Layers in ascending bit order.  out=None: host numpy (k, H, W); else a CUDA tensor."""
-        k = bin(mask).count("1")
-        H, W = self.shape
+        k = int(mask).bit_count()
+        H, W = self.params.height, self.params.width
         if out is None:
             host = np.empty((k, H, W), np.float32)
             _check(lib.em_get_layers(self._h, mask, host.ctypes.data, 1, _stream_handle(stream)), "em_get_layers")
@@ -457,6 +474,12 @@ class _Request(ctypes.Structure):
                 ("clouds_on_host", ctypes.c_int32)]
 
 
+# the same layouts for struct.pack_into (a pose as its 48 bytes)
+_REQUEST = struct.Struct("iiPIiPi4x")
+_CLOUD = struct.Struct("Pqi48s4x")
+assert _REQUEST.size == ctypes.sizeof(_Request) and _CLOUD.size == ctypes.sizeof(_Cloud)
+
+
 class _ServerStats(ctypes.Structure):
     _fields_ = [(n, ctypes.c_int64) for n in ("submitted", "completed", "rejected", "cancelled", "batches",
                                              "batched_requests", "max_batch_size", "bytes_in_use", "peak_bytes",
@@ -560,37 +583,39 @@ class Server:
         this update.  One call queues them all (they reach the same batch when they fit);
         ready as in submit.  Returns the tickets."""
         n = len(requests)
-        reqs = (_Request * n)()
-        keep = []
         f32 = _torch().float32
-        for q, (map_id, clouds, read) in enumerate(requests):
+        # requests, then clouds, in one buffer of the C layout
+        n_clouds = sum([len(clouds) for _, clouds, _ in requests])
+        buf = ctypes.create_string_buffer(n * _REQUEST.size + n_clouds * _CLOUD.size)
+        base = ctypes.addressof(buf)
+        at, cat = 0, n * _REQUEST.size
+        for map_id, clouds, read in requests:
             on_host = not clouds[0][0].is_cuda
-            cs = []
+            first = base + cat
             for p, pose in clouds:
+                shape = p.shape
                 if p.is_cuda == on_host or p.dtype is not f32 or not p.is_contiguous() or \
-                        p.dim() != 2 or p.shape[1] not in (3, 4) or (on_host and not p.is_pinned()):
+                        len(shape) != 2 or shape[1] not in (3, 4) or (on_host and not p.is_pinned()):
                     raise ValueError("points: contiguous float32 (n, 3|4) tensors, all CUDA or all pinned CPU")
-                cs.append(_Cloud(p.data_ptr(), p.shape[0], p.shape[1], _pose(pose)))
-            arr = (_Cloud * len(cs))(*cs)
-            keep.append((arr, clouds, read))
-            r = reqs[q]
-            r.map_id = int(map_id)
-            r.n_clouds = len(cs)
-            r.clouds = arr
-            r.clouds_on_host = 1 if on_host else 0
+                _CLOUD.pack_into(buf, cat, p.data_ptr(), shape[0], shape[1], _pose_bytes(pose))
+                cat += _CLOUD.size
+            mask, to_host, dst = 0, 0, 0
             if read is not None:
                 mask, out = read
                 if out.dtype is not f32 or not out.is_contiguous():
                     raise ValueError("read-back buffer must be a contiguous float32 tensor")
-                r.read_mask = int(mask)
-                r.read_to_host = 0 if out.is_cuda else 1
-                r.read_dst = out.data_ptr()
+                to_host, dst = 0 if out.is_cuda else 1, out.data_ptr()
+            _REQUEST.pack_into(buf, at, ctypes.c_int32(map_id).value, len(clouds), first, int(mask) & 0xffffffff,
+                               to_host, dst, 1 if on_host else 0)
+            at += _REQUEST.size
         tks = (ctypes.c_uint64 * n)()
-        _check(lib.em_server_submit_many(self._h, reqs, n, ready.cuda_event if ready is not None else None, tks),
+        _check(lib.em_server_submit_many(self._h, ctypes.cast(buf, ctypes.POINTER(_Request)), n,
+                                         ready.cuda_event if ready is not None else None, tks),
                "em_server_submit_many")
-        for q in range(n):
-            self._keep[tks[q]] = (keep[q], ready)
-        return list(tks)
+        tickets = list(tks)
+        for t, r in zip(tickets, requests):  # (the library copies the descriptors; the tensors must live)
+            self._keep[t] = (r, ready)
+        return tickets
 
     def wait_many(self, tickets, timeout_us: int = -1, results: bool = False):
         """Wait for all tickets in one call.  Returns their statuses (or result dicts)."""
@@ -598,8 +623,9 @@ class Server:
         tks = (ctypes.c_uint64 * n)(*tickets)
         res = (_Result * n)()
         _check(lib.em_server_wait_many(self._h, tks, n, int(timeout_us), res), "em_server_wait_many")
+        keep = self._keep
         for t in tickets:
-            self._keep.pop(t, None)
+            keep.pop(t, None)
         if results:
             return [{f: getattr(r, f) for f, _ in _Result._fields_} for r in res]
         return [r.status for r in res]
