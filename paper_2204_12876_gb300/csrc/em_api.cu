@@ -518,7 +518,7 @@ static int update_impl(em_map* m, const em_cloud* clouds, int32_t n_clouds, cuda
   }
   const Sequence q = update_sequence(kind, total, ncell);
   for (int i = 0; i < q.n; ++i)
-    EM_TRY(timed(m, q.k[i].slot, s, [&] { return run(q.k[i], arg, i == 0 || m->prof, s); }), q.k[i].name);
+    EM_TRY(timed(m, q.k[i].slot, s, [&] { return run(q.k[i], arg, s); }), q.k[i].name);
   if (slot >= 0) EM_TRY(cudaEventRecord(m->desc_ev[slot], s), "cudaEventRecord");
   m->last_stream = s;
   m->last_n = total;

@@ -88,7 +88,7 @@ cudaError_t launch_sequence(em_batch* b, const Sequence& q, const BatchDev* bd, 
   for (int i = 0; i < q.n && e == cudaSuccess; ++i) {
     const int slot = q.k[i].slot;
     if (b->prof && !b->pused[slot]) cudaEventRecord(b->pev[2 * slot], s);  // a slot spans its launches
-    e = run(q.k[i], &bd, i == 0 || b->prof, s);
+    e = run(q.k[i], &bd, s);
     if (b->prof) {
       cudaEventRecord(b->pev[2 * slot + 1], s);
       b->pused[slot] = true;

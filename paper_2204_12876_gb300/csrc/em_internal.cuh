@@ -252,7 +252,23 @@ struct Sequence {
 constexpr int kValueGroup = 8;  // the one ray_group built for MapDesc
 Sequence update_sequence(const UpdateKind& k, int64_t n_points, int64_t n_cells);
 // desc: the kernel's descriptor argument (a const BatchDev* or a MapDesc)
-cudaError_t run(const Launch& l, const void* desc, bool first, cudaStream_t s);
+cudaError_t run(const Launch& l, const void* desc, cudaStream_t s);
+
+// Launch a kernel that begins with begin_after_previous(): it may start while the
+// kernel before it on the stream ends.
+template <class... P, class... A>
+cudaError_t launch_after(void (*k)(P...), int grid, int block, cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
 // The sequence as a chain of kernel nodes.
 cudaError_t build_graph(const Sequence& q, const BatchDev* b, cudaGraph_t* out);
 

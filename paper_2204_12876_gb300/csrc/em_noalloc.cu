@@ -213,6 +213,6 @@ extern "C" int em_update_noalloc(const em_params* params, int64_t shift_x, int64
   kind.by_value = true;
   const Sequence q = update_sequence(kind, total, cells);
   cudaError_t e = cudaSuccess;
-  for (int i = 0; i < q.n && e == cudaSuccess; ++i) e = run(q.k[i], &desc, i == 0, s);
+  for (int i = 0; i < q.n && e == cudaSuccess; ++i) e = run(q.k[i], &desc, s);
   return na_status(e, "em_update_noalloc launch");
 }

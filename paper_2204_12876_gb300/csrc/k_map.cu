@@ -328,6 +328,7 @@ __device__ __forceinline__ void empty_cell(const MapDev& m, int32_t p) {
 
 // exposed logical columns [cx0, cx1) over all rows, and rows [ry0, ry1) over all columns
 __global__ void __launch_bounds__(kMapThreads) k_shift(MapDev m, int32_t cx0, int32_t cx1, int32_t ry0, int32_t ry1) {
+  begin_after_previous();
   const int32_t ncol = (cx1 - cx0) * m.H;
   const int32_t nrow = (ry1 - ry0) * m.W;
   for (int32_t i = blockIdx.x * kMapThreads + threadIdx.x; i < ncol + nrow; i += gridDim.x * kMapThreads) {
@@ -385,6 +386,7 @@ __device__ __forceinline__ void layers_out(const MapDev& m, uint32_t mask, float
 }
 
 __global__ void __launch_bounds__(kMapThreads) k_layers_out(MapDev m, uint32_t mask, float* __restrict__ dst) {
+  begin_after_previous();
   layers_out(m, mask, dst, blockIdx.x * kMapThreads + threadIdx.x, gridDim.x * kMapThreads);
 }
 
@@ -438,8 +440,7 @@ cudaError_t launch_shift_clear(const MapDev& m, int32_t dx, int32_t dy, cudaStre
   if (dy > 0) { ry0 = m.H - dy; ry1 = m.H; } else if (dy < 0) { ry0 = 0; ry1 = -dy; }
   const int64_t n = (int64_t)(cx1 - cx0) * m.H + (int64_t)(ry1 - ry0) * m.W;
   if (n == 0) return cudaSuccess;
-  k_shift<<<cell_grid(n), kMapThreads, 0, s>>>(m, cx0, cx1, ry0, ry1);
-  return cudaGetLastError();
+  return launch_after(k_shift, cell_grid(n), kMapThreads, s, m, cx0, cx1, ry0, ry1);
 }
 
 cudaError_t launch_fill_map(const MapDev& m, cudaStream_t s) {
@@ -448,8 +449,7 @@ cudaError_t launch_fill_map(const MapDev& m, cudaStream_t s) {
 }
 
 cudaError_t launch_layers_out(const MapDev& m, uint32_t mask, float* dst, cudaStream_t s) {
-  k_layers_out<<<cell_grid((int64_t)m.W * m.H), kMapThreads, 0, s>>>(m, mask, dst);
-  return cudaGetLastError();
+  return launch_after(k_layers_out, cell_grid((int64_t)m.W * m.H), kMapThreads, s, m, mask, dst);
 }
 
 cudaError_t launch_layers_out_multi(const ReadJobs& jobs, cudaStream_t s) {

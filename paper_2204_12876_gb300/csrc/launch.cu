@@ -26,14 +26,14 @@ Sequence update_sequence(const UpdateKind& k, int64_t n_points, int64_t n_cells)
   return q;
 }
 
-// Every launch of an update but the first may start while the one before it
+// Every launch of an update may start while the kernel before it on the stream
 // ends (programmatic stream serialisation; every kernel begins with the wait for
 // the previous one, so the work itself stays in order).  The gap between two
 // dependent kernels shrinks to the wait's wake-up: with the descriptor as a
 // parameter, which takes the upload out of the chain, one depth frame went from
 // 58.6 to 45.0 us, a 20,000-point cloud from 26.9 to 20.3, the seven kernels of
 // the dome LiDARs' update from 89 to 64.
-cudaError_t run(const Launch& l, const void* desc, bool first, cudaStream_t s) {
+cudaError_t run(const Launch& l, const void* desc, cudaStream_t s) {
   void* args[] = {const_cast<void*>(desc), (void*)&l.part};  // (a kernel takes as many as it has parameters)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(l.grid);
@@ -49,7 +49,7 @@ cudaError_t run(const Launch& l, const void* desc, bool first, cudaStream_t s) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
   }
   cfg.attrs = attr;
-  cfg.numAttrs = l.coop || !first ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelExC(&cfg, l.fn, args);
 }
 
