@@ -225,7 +225,7 @@ __device__ __forceinline__ void write_pass(const V& b, Grid gr) {
       m.ctl->drift_l = 0;
       m.ctl->drift_n = 0;
     }
-    const bool touched = m.touched[tile] != 0;
+    const bool touched = !m.touched || m.touched[tile] != 0;
     const bool overlap = m.ovl_dz > 0.f;
     CellAcc a[kWriteRounds];
     uint32_t rej[kWriteRounds], mark[kWriteRounds];
@@ -294,8 +294,10 @@ __device__ __forceinline__ void write_pass(const V& b, Grid gr) {
     const unsigned nu = __reduce_add_sync(kFull, updated), nc = __reduce_add_sync(kFull, cleared);
     if (lane == 0 && nu) atomicAdd(&m.ctl->stats[kStCellsUpdated], (unsigned long long)nu);
     if (lane == 0 && nc) atomicAdd(&m.ctl->stats[kStCleared], (unsigned long long)nc);
-    __syncthreads();  // every thread has read the tile's flag
-    if (threadIdx.x == 0 && touched) m.touched[tile] = 0;
+    if (m.touched) {
+      __syncthreads();  // every thread has read the tile's flag
+      if (threadIdx.x == 0 && touched) m.touched[tile] = 0;
+    }
   });
 }
 

@@ -444,7 +444,8 @@ int em_create(const em_params* params, int device, em_map** out) {
     const size_t nb = (size_t)coarse_size(params->width, params->height);
     EM_ALLOC(m->thr, nc) EM_ALLOC(m->cthr, nb)
   }
-  EM_ALLOC(m->acc, nc) EM_ALLOC(m->rej, nc) EM_ALLOC(m->touched, ntile)
+  EM_ALLOC(m->acc, nc) EM_ALLOC(m->rej, nc)
+  if ((int64_t)nc > kFlagCells) { EM_ALLOC(m->touched, ntile) }
   if (params->wall_num_thresh > 0) { EM_ALLOC(m->cnt, nc) }
   EM_ALLOC(m->ctl, 1) EM_ALLOC(m->bctl, 1)
   EM_ALLOC(m->desc_dev, kDescBytes * kSlots)
@@ -457,7 +458,7 @@ int em_create(const em_params* params, int device, em_map** out) {
   if (e == cudaSuccess) e = cudaMemset(m->acc, 0, nc * sizeof(CellAcc));
   if (e == cudaSuccess) e = cudaMemset(m->rej, 0, nc * sizeof(uint32_t));
   if (e == cudaSuccess && m->cnt) e = cudaMemset(m->cnt, 0, nc * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMemset(m->touched, 0, ntile);
+  if (e == cudaSuccess && m->touched) e = cudaMemset(m->touched, 0, ntile);
   if (e == cudaSuccess) e = cuda_status(launch_fill_map(make_mapdev(m), nullptr), "fill") ? cudaErrorUnknown : cudaSuccess;
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {

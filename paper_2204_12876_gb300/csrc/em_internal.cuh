@@ -93,6 +93,13 @@ constexpr int kParts = 3;
 constexpr uint32_t kSplitPoints = 1u << 20;
 constexpr int kOrderSamples = 64;
 
+// Maps beyond this many cells keep a flag per tile, so that a cloud on a corner of
+// a huge map does not cost a read of all its accumulators.  Smaller maps' flags
+// would be a few sectors that every warp of the update writes: without them a
+// raw depth image took 45 us instead of 49, four depth cameras 36.8 instead of
+// 38.5, and reading the accumulators of the untouched tiles costs less.
+constexpr int64_t kFlagCells = 1 << 20;
+
 constexpr int kItemW = 32, kItemH = 8;  // k_cells: logical cells per warp item
 
 // device-side error word value for a failed internal consistency check (EM_ERR_CUDA)
@@ -123,7 +130,8 @@ struct MapDev {
   CellAcc* acc;     // per physical cell
   uint32_t* rej;    // rejected points per physical cell, zero between updates
   uint32_t* cnt;    // wall rule: points per physical cell, zero between updates; null without the rule
-  uint8_t* touched; // per tile of kTile cells: some point of this update fell into it
+  uint8_t* touched; // per tile of kTile cells: some point of this update fell into it; null for maps of at
+                    // most kFlagCells cells, whose tiles all count as touched
   int64_t ibegin;   // this map's first item in the batch's item space (maps with the ray march or drift)
   int32_t IW, IH;   // items per row and column; 0 x 0 without the ray march and the drift compensation
   int32_t CW, CH, CS;  // coarse blocks per row and column (0 x 0 without the ray march), row stride

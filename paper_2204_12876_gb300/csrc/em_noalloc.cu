@@ -37,21 +37,20 @@ constexpr size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
 static_assert(kMaxCloudsNA <= kDescClouds, "the descriptor travels as a kernel parameter");
 
-// Scratch layout.  The part that must start at zero (control blocks, marks, tile
-// flags and the accumulators of this call's cells) is contiguous, so one memset
+// Scratch layout.  The part that must start at zero (control blocks, marks and
+// the accumulators of this call's cells) is contiguous, so one memset
 // as long as the map is clears it.
 constexpr size_t kOffCtl = 0;
 constexpr size_t kOffBCtl = kOffCtl + up256(sizeof(MapCtl));
 constexpr size_t kOffZero = kOffBCtl + up256(sizeof(BatchCtl));  // the map's part of the zeroed scratch
 struct Layout {
-  size_t mark, touched, rej, cnt, acc, thr, cthr, end;
+  size_t mark, rej, cnt, acc, thr, cthr, end;
 };
 // coarse: blocks of the coarse grid
 constexpr Layout layout(size_t cells, size_t coarse) {
   Layout o{};
   o.mark = kOffZero;
-  o.touched = o.mark + up256((cells + 31) / 32 * sizeof(uint32_t));
-  o.rej = o.touched + up256((cells + kTile - 1) / kTile);
+  o.rej = o.mark + up256((cells + 31) / 32 * sizeof(uint32_t));
   o.cnt = o.rej + up256(cells * sizeof(uint32_t));
   o.acc = o.cnt + up256(cells * sizeof(uint32_t));
   o.thr = o.acc + up256(cells * sizeof(CellAcc));  // end of the zeroed part
@@ -61,6 +60,7 @@ constexpr Layout layout(size_t cells, size_t coarse) {
 }
 // coarse entries of a map of at most kMaxCells cells: (W/8 + 3)(H/8 + 3) <= kMaxCells/64 + 3 (W + H)/8 + 9,
 // and W + H <= kMaxCells + 1
+static_assert(kMaxCells <= kFlagCells, "no tile flags");
 constexpr size_t kMaxCoarse = (size_t)kMaxCells / 64 + 3 * ((size_t)kMaxCells + 1) / 8 + 10;
 constexpr size_t kScratchBytes = layout(kMaxCells, kMaxCoarse).end;
 
@@ -157,7 +157,6 @@ extern "C" int em_update_noalloc(const em_params* params, int64_t shift_x, int64
   set_item_grid(*m, W, H, params->ray_step > 0.f, params->drift_flatness > 0.f);
   const Layout lay = layout((size_t)ncell, m->CW ? (size_t)coarse_size(W, H) : 0);
   m->mark = reinterpret_cast<uint32_t*>(base + lay.mark);
-  m->touched = base + lay.touched;
   m->rej = reinterpret_cast<uint32_t*>(base + lay.rej);
   if (params->wall_num_thresh > 0) m->cnt = reinterpret_cast<uint32_t*>(base + lay.cnt);
   m->acc = reinterpret_cast<CellAcc*>(base + lay.acc);

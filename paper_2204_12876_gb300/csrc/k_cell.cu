@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kCellThreads) k_refresh(const __grid_constant_
 
 // n_cells bounds the items but for partial last rows and columns (the pass strides over the grid)
 static Launch item_launch(const void* fn, int64_t n_cells, int slot, const char* name) {
-  constexpr int kThreads = 128;  // small maps reach more SMs
+  constexpr int kThreads = kCellThreads;
   const int64_t blocks = n_cells / (kItemW * kItemH * (kThreads / 32)) + 1;
   const int64_t cap = (int64_t)sm_count() * 16;
   return {fn, (unsigned)(blocks < cap ? blocks : cap), kThreads, 0, false, slot, name, 0};

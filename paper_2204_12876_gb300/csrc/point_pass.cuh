@@ -211,7 +211,7 @@ __device__ __forceinline__ uint8_t add_points(const MapDev& m, int map, bool one
   }
   // the run's last lane holds its sums
   if (tail) {
-    m.touched[p / kTile] = 1;  // every writer stores the same
+    if (m.touched) m.touched[p / kTile] = 1;  // every writer stores the same
     if (nn >> 16) atomicAdd(&m.rej[p], nn >> 16);
     if ((nn & 0xffffu) && (wh | (long long)wl) == 0) atomicOr(&m.acc[p].wl, kAccTouched);
   }
