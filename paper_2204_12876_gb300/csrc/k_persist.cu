@@ -5,7 +5,8 @@
 // resident, with a grid-wide barrier wherever a pass needs the one before:
 //
 //   points per cell (maps with the wall rule), thresholds and coarse grids
-//   | points: gate, sums, ray march (blocks take runs from the work counter)
+//   | points: gate, sums, ray march (blocks take runs from the work counter); for
+//   |   scattered points in parts, the thresholds refreshed between them
 //   | new state of every cell, removal of marked cells, overlap clearance
 //
 // The stencils (normals, smoothing, in-painting) follow as their own kernels.
@@ -76,8 +77,14 @@ __global__ void __launch_bounds__(kPersistThreads, 4) k_persist(const BatchDev* 
     if (b.passes & kPassCells) cells_pass(b, all);
     ok = grid_barrier(b, nb, budget, s_ok);
   }
-  if (ok) {
-    points_pass<G, true, kExt>(b, all, -1, *reinterpret_cast<PointsSmem<true>*>(sm));
+  const int parts = ok && in_parts(b) ? kParts : 1;  // (the same for every block)
+  for (int i = 0; ok && i < parts; ++i) {
+    if (i > 0) {
+      refresh_pass(b, all);
+      ok = grid_barrier(b, nb, budget, s_ok);
+      if (!ok) break;
+    }
+    points_pass<G, true, kExt>(b, all, i, *reinterpret_cast<PointsSmem<true>*>(sm));
     ok = grid_barrier(b, nb, budget, s_ok);
   }
   if (ok) write_pass(b, all);

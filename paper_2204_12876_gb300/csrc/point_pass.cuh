@@ -399,10 +399,10 @@ __device__ __forceinline__ void points_pass(const V& b, Grid gr, int part, Point
   // kRayRun batches.
   const uint32_t n_points = (uint32_t)b.n_points;  // below 2^31
   // the part's batches: `len` of every 32, those at places first .. of the
-  // bit-reversed order, so that every part samples the whole clouds (part -1, or
-  // points that go in one part: all of them, in order)
+  // bit-reversed order, so that every part samples the whole clouds (points
+  // that go in one part: all of them, in order)
   uint32_t first = 0, len = 32;
-  if (kRay && part >= 0 && in_parts(b)) {
+  if (kRay && in_parts(b)) {
     first = part_first(part);
     len = part_first(part + 1) - first;
   } else if (part > 0) {
@@ -675,7 +675,7 @@ __device__ __forceinline__ void points_pass(const V& b, Grid gr, int part, Point
     ++index;
     if (index >= (run + 1) * run_len || index >= n_batches) {
       uint32_t t = 0;
-      if (lane == 0) t = (uint32_t)atomicAdd(&b.ctl->next[max(part, 0)], 1);
+      if (lane == 0) t = (uint32_t)atomicAdd(&b.ctl->next[part], 1);
       run = warps + __shfl_sync(kFull, t, 0);
       index = run * run_len;
     }

@@ -107,3 +107,44 @@ def test_weights_below_fixed_point(em):
     assert s["t_last"][0, 0] == 5 and s["t_last"][0, 1] == 0
     assert m.stats()["points_accepted"] == 40 and m.stats()["cells_updated"] == 1
     m.close()
+
+
+def test_updates_under_stream_capture(em):
+    """The one-map forms take their descriptor as a kernel parameter, so an update
+    captured from a stream replays whole: each replay fuses the cloud again as
+    the update index it was captured with."""
+    rng = np.random.default_rng(5)
+    W, H, n = 40, 33, 5000
+    p, _ = runs_cloud(rng, W, H, n)
+    d = torch.from_numpy(p).cuda()
+    P = em.Params(width=W, height=H, resolution=R, noise_a0=0.005, noise_a2=0.002, ray_step=R)
+    states = []
+    for captured in (False, True):
+        m = em.Map(P)
+        m.reserve(n)
+        h, v = torch.full((H, W), float("nan"), device="cuda"), torch.full((H, W), float("inf"), device="cuda")
+        t = torch.zeros((H, W), dtype=torch.int32, device="cuda")
+        em.update_noalloc(P, h, v, t, [(d, POSE)], t_now=1)  # (its first call looks up the scratch)
+        out = torch.empty(3, H, W, device="cuda")
+        torch.cuda.synchronize()
+
+        def step():
+            m.update(d, POSE)
+            em.update_noalloc(P, h, v, t, [(d, POSE)], t_now=2)
+            m.get_layers(em.LAYER_ELEVATION | em.LAYER_VARIANCE | em.LAYER_TIME, out=out)
+
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                step()
+            for _ in range(2):
+                g.replay()
+        else:
+            for _ in range(2):
+                step()
+                m.set_state(t_now=0)  # the captured update keeps its index
+        torch.cuda.synchronize()
+        states.append([x.cpu().numpy() for x in (out, h, v, t)])
+        m.close()
+    for a, b in zip(*states):
+        assert np.array_equal(a, b, equal_nan=True)
