@@ -572,9 +572,9 @@ def run_batched(args, em, torch, dev, barrier, max_over_ranks, world):
     batch.close()
     return {"workload": "64 maps, side U{100..500} cells @ 0.04 m, 10k..400k points each, random point order; "
                         "fusion, outlier gate and visibility ray march (step 0.04 m)",
-            "form": "one kernel sequence over every map, replayed from a captured CUDA graph (the default form)",
+            "form": "one kernel sequence over every map, replayed from a CUDA graph (the default form)",
             "persistent": {"form": "EM_BATCH_PERSISTENT: the update's passes in one cooperative launch with grid "
-                                   "barriers (stencils as kernels of their own), replayed from a captured CUDA graph",
+                                   "barriers (stencils as kernels of their own), replayed from a CUDA graph",
                            "value": pts_step * K * world / xsec, "unit": "points/s", "ms_per_step": xsec / K * 1e3,
                            "kernels": {em.KERNEL_NAMES[k]: {"ms_per_launch": round(v[0] / v[1], 5)}
                                        for k, v in xprof.items() if v[1]}},

@@ -256,7 +256,7 @@ int em_profile_read(em_map* map, double* ms, int64_t* launches);
 typedef struct em_batch em_batch;
 
 /* EM_BATCH_PERSISTENT: one cooperative launch of all blocks that fit on the
- * device at once runs the passes of the update (transform, binning, grouping,
+ * device at once runs the passes of the update (transform, binning,
  * gate, fusion, ray march, removal) over every map, with grid-wide barriers
  * between them, instead of one kernel per pass (the normals, smoothing and
  * in-painting stencils stay kernels of their own).  Every barrier wait is

@@ -353,6 +353,19 @@ void map_undo_update(em_map* m, int64_t points) {
   m->points_in -= points;
 }
 
+int map_update_one(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t total, cudaStream_t s) {
+  m->t_now += 1;
+  m->points_in += total;
+  UpdateKind kind = map_kind(m, kValueGroup);
+  kind.by_value = true;
+  MapDesc desc;
+  fill_desc(m, clouds, n_clouds, total, &desc.b, &desc.m, desc.c);
+  const Sequence q = update_sequence(kind, total, desc.b.n_cells);
+  for (int i = 0; i < q.n; ++i) EM_TRY(run(q.k[i], &desc, s), q.k[i].name);
+  map_end_update(m, s, 0);
+  return EM_OK;
+}
+
 int map_copy_state(em_map* dst, const em_map* src, cudaStream_t s) {
   if (dst->p.width != src->p.width || dst->p.height != src->p.height) return EM_ERR_INVALID_ARG;
   const size_t nc = (size_t)src->p.width * src->p.height;

@@ -107,9 +107,9 @@ struct Prepared {
   UpdateKind kind{};
 };
 
-// Group the pairs by map, build the descriptor in slot `slot` and upload it.
-int prepare(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t count, const em_tuning& tune,
-            cudaStream_t s, Prepared* out) {
+// Check the pairs and group them by map (b->uniq, b->map_of; points per map).
+int group(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t count, std::vector<int64_t>* map_pts,
+          int64_t* points) {
   if (!maps || !clouds || count < 1) return EM_ERR_INVALID_ARG;
   if (count > b->max_clouds) return EM_ERR_CAPACITY;
   b->uniq.clear();
@@ -132,15 +132,21 @@ int prepare(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t co
     }
     b->map_of[i] = u;
   }
-  const int nm = (int)b->uniq.size();
-  std::vector<int64_t> map_pts(nm, 0);
+  map_pts->assign(b->uniq.size(), 0);
   int64_t total = 0;
   for (int i = 0; i < count; ++i) {
-    map_pts[b->map_of[i]] += clouds[i].n;
+    (*map_pts)[b->map_of[i]] += clouds[i].n;
     total += clouds[i].n;
   }
   if (total > b->max_points) return EM_ERR_CAPACITY;
+  *points = total;
+  return EM_OK;
+}
 
+// Build the descriptor of the grouped pairs in the next slot and upload it.
+int prepare(em_batch* b, const em_cloud* clouds, int32_t count, const std::vector<int64_t>& map_pts, int64_t total,
+            const em_tuning& tune, cudaStream_t s, Prepared* out) {
+  const int nm = (int)b->uniq.size();
   const int slot = b->slot;
   b->slot = (b->slot + 1) % kSlots;
   EB_TRY(cudaEventSynchronize(b->ev[slot]), "cudaEventSynchronize");
@@ -345,8 +351,18 @@ int em_update_batch(em_batch* b, em_map* const* maps, const em_cloud* clouds, in
     rc = prof_collect(b);
     if (rc) return rc;
   }
+  std::vector<int64_t> map_pts;
+  int64_t total = 0;
+  rc = group(b, maps, clouds, count, &map_pts, &total);
+  if (rc) return rc;
+  // One map (a lightly loaded server's batches): as em_update, with nothing to
+  // upload and grids of its own size instead of the capacity's; a served request
+  // at 2,000 updates/s took 67 us through the graph, em_update 49.
+  if (b->uniq.size() == 1 && count <= kDescClouds && b->tune.ray_group == kValueGroup && !b->prof &&
+      !(b->flags & EM_BATCH_PERSISTENT) && !(map_flags(b->uniq[0]) & EM_F_TRACE))
+    return map_update_one(b->uniq[0], clouds, count, total, s);
   Prepared p;
-  rc = prepare(b, maps, clouds, count, b->tune, s, &p);
+  rc = prepare(b, clouds, count, map_pts, total, b->tune, s, &p);
   if (rc) return rc;
   if ((b->flags & EM_BATCH_GRAPH) && !b->prof) {
     rc = run_graph(b, p, s);
@@ -438,7 +454,10 @@ int em_batch_autotune(em_batch* b, em_map* const* maps, const em_cloud* clouds, 
         if (c) return c;
       }
       Prepared p;
-      int c = prepare(b, cmaps.data(), clouds, count, t, s, &p);
+      std::vector<int64_t> map_pts;
+      int64_t total = 0;
+      int c = group(b, cmaps.data(), clouds, count, &map_pts, &total);
+      if (c == EM_OK) c = prepare(b, clouds, count, map_pts, total, t, s, &p);
       if (c) return c;
       cudaEventRecord(e0, s);
       cudaError_t le = launch_sequence(b, update_sequence(p.kind, p.points, p.cells), p.bd, s);

@@ -23,6 +23,10 @@ MapDev map_begin_update(em_map* m, int64_t points);
 void map_end_update(em_map* m, cudaStream_t s, int64_t points);
 void map_undo_update(em_map* m, int64_t points);
 
+// One update of map m from at most kDescClouds clouds (checked by the caller),
+// total points, as a batch of that map alone does it (no trace, no profiling).
+int map_update_one(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t total, cudaStream_t s);
+
 // Copy layers, ring offsets, shift and update index of src into dst (same size).
 int map_copy_state(em_map* dst, const em_map* src, cudaStream_t s);
 

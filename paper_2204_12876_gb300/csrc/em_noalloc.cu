@@ -4,8 +4,9 @@
 // that forbids allocation after start-up (an allocation can block on the
 // driver for milliseconds), or a host framework whose own caching allocator
 // has already claimed the device memory.  For them this entry point runs the
-// same kernels as em_update (binning, gate + fusion, ray march, removal) on map layers the caller owns, and keeps every piece of
-// scratch memory in one file-scope __device__ array of fixed size.  The call's
+// same kernels as em_update (binning, gate + fusion, ray march, removal) on map
+// layers the caller owns, and keeps every piece of scratch memory in one
+// file-scope __device__ array of fixed size.  The call's
 // descriptor goes to the device as a kernel parameter (no host buffer, no
 // copy), and its only other preparation is a memset of the scratch.
 //

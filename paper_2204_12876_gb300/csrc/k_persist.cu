@@ -1,8 +1,8 @@
 // k_persist.cu -- the batched form in one persistent launch: the passes of an
-// update over every map of a batch (transform, noise, binning, grouping by
-// tile, wall rule, gate, Eq. 1/2 fusion, ray march and removal; Section II-A
-// to II-E of the paper) in one cooperative kernel whose blocks are all
-// resident, with a grid-wide barrier wherever a pass needs the one before:
+// update over every map of a batch (transform, noise, binning, wall rule, gate,
+// Eq. 1/2 fusion, ray march and removal; Section II-A to II-E of the paper) in
+// one cooperative kernel whose blocks are all resident, with a grid-wide
+// barrier wherever a pass needs the one before:
 //
 //   points per cell (maps with the wall rule), thresholds and coarse grids
 //   | points: gate, sums, ray march (blocks take runs from the work counter); for

@@ -148,3 +148,28 @@ def test_updates_under_stream_capture(em):
         m.close()
     for a, b in zip(*states):
         assert np.array_equal(a, b, equal_nan=True)
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_batch_of_one_map_equals_update(em, graph):
+    """A batch that names one map (once, or with several clouds) runs as em_update
+    does: same state and counters as Map.update_multi, also beside batches of two."""
+    rng = np.random.default_rng(6)
+    W, H = 50, 41
+    make = lambda: em.Map(em.Params(width=W, height=H, resolution=R, noise_a0=0.005, noise_a2=0.002,  # noqa: E731
+                                    mahalanobis_k=2.5, outlier_variance=1e-4, ray_step=R))
+    clouds = [[torch.from_numpy(runs_cloud(rng, W, H, n)[0]).cuda() for n in ns] for ns in ((3000,), (700, 5, 900), (64,))]
+    ref, m, other = make(), make(), make()
+    batch = em.Batch(max_maps=2, max_clouds=8, max_points=8192, max_cells=W * H, graph=graph)
+    for k, cs in enumerate(clouds):
+        ref.update_multi([(c, POSE) for c in cs])
+        pairs = [(m, c, POSE) for c in cs]
+        batch.update(pairs + [(other, cs[0], POSE)] if k == 1 else pairs)
+    a, b = ref.state(), m.state()
+    for k in ("h", "var", "t_last"):
+        assert np.array_equal(a[k], b[k], equal_nan=True), k
+    assert ref.stats() == m.stats() and m.info()["t_now"] == 3
+    with pytest.raises(em.EMError) as e:  # the batch's capacities hold for one map too
+        batch.update([(m, torch.zeros(9000, 3, device="cuda"), POSE)])
+    assert e.value.code == em.EM_ERR_CAPACITY and m.info()["t_now"] == 3
+    batch.close()
