@@ -4,7 +4,7 @@
 // that forbids allocation after start-up (an allocation can block on the
 // driver for milliseconds), or a host framework whose own caching allocator
 // has already claimed the device memory.  For them this entry point runs the
-// same kernels as em_update (binning, gate + fusion, ray march, removal) on map
+// same kernels as em_update (gate + sums + ray march, fusion, removal) on map
 // layers the caller owns, and keeps every piece of scratch memory in one
 // file-scope __device__ array of fixed size.  The call's
 // descriptor goes to the device as a kernel parameter (no host buffer, no

@@ -173,3 +173,44 @@ def test_batch_of_one_map_equals_update(em, graph):
         batch.update([(m, torch.zeros(9000, 3, device="cuda"), POSE)])
     assert e.value.code == em.EM_ERR_CAPACITY and m.info()["t_now"] == 3
     batch.close()
+
+
+@pytest.mark.parametrize("extra", [dict(), dict(ray_step=0.0), dict(wall_num_thresh=2, time_variance=1e-6),
+                                   dict(drift_flatness=0.9, cleanup_normal_thresh=0.1, overlap_radius=0.5,
+                                        overlap_dz=0.2, excl_b=0.2, excl_c=0.3, excl_theta=0.5, excl_d=1.0,
+                                        flags=1 | 4 | 8 | 32)])
+def test_uploaded_descriptor_equals_parameter(em, extra):
+    """Updates of more than 8 clouds upload their descriptor, the others pass it as
+    a kernel parameter: the same points as 1, 3 and 12 clouds -- strides 3 and 4,
+    rows off a 16-byte boundary, ragged and empty clouds -- leave the same map and
+    counters, over two updates with a shift between them."""
+    import synth
+    W, H, n = 70, 53, 9000
+    pts, pose = synth.scattered_cloud(8, n, 1.3, nan_frac=0.02)
+    prior = synth.random_prior(seed=9, width=W, height=H, t_now=5)
+    P = dict(dict(width=W, height=H, resolution=R, noise_a0=0.005, noise_a2=0.002, mahalanobis_k=2.5,
+                  outlier_variance=1e-4, ray_step=R), **extra)
+    got = []
+    for parts in (1, 3, 12):
+        cuts = np.sort(np.random.default_rng(parts).integers(0, n + 1, parts - 1))
+        if parts > 2:
+            cuts[1] = cuts[0]  # an empty cloud
+        clouds = []
+        for k, c in enumerate(np.split(pts, cuts)):
+            c = np.concatenate([c, np.zeros((len(c), 1), np.float32)], axis=1) if k % 3 == 1 else c
+            flat = torch.zeros(c.size + 1, device="cuda")[1:] if k % 2 else torch.zeros(c.size, device="cuda")
+            flat.copy_(torch.from_numpy(np.ascontiguousarray(c).reshape(-1)))
+            clouds.append((flat.view(c.shape), pose))
+        m = em.Map(em.Params(**P))
+        has_normals = bool(extra.get("flags"))
+        m.set_state(h=prior["h"], var=prior["var"], t_last=prior["t_last"].astype(np.float32), t_now=prior["t_now"],
+                    **({k: prior[k] for k in ("nx", "ny", "nz")} if has_normals else {}))
+        m.update_multi(clouds)
+        m.shift(3, -2)
+        m.update_multi(clouds)
+        got.append((m.state(), m.stats()))
+        m.close()
+    for s, st in got[1:]:
+        for k, v in got[0][0].items():
+            assert np.array_equal(v, s[k], equal_nan=True), k
+        assert st == got[0][1]
