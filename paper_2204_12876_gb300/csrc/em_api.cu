@@ -577,8 +577,10 @@ int em_update_host(em_map* m, const em_cloud* clouds, int32_t n_clouds, em_strea
   rc = set_device(m->device);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
+  // every cloud starts on a 16-byte boundary of the staging buffers, so it takes up to 3 floats more than its own
+  const auto staged = [](const em_cloud& c) { return (c.n * c.stride + 3) & ~int64_t(3); };
   int64_t floats = 0;
-  for (int i = 0; i < n_clouds; ++i) floats += clouds[i].n * clouds[i].stride;
+  for (int i = 0; i < n_clouds; ++i) floats += staged(clouds[i]);
   EM_TRY(cudaEventSynchronize(m->stage_ev), "cudaEventSynchronize");
   if (floats > m->stage_cap) {
     int64_t want = floats + floats / 4 + 1024;
@@ -598,8 +600,7 @@ int em_update_host(em_map* m, const em_cloud* clouds, int32_t n_clouds, em_strea
     if (nf) memcpy(m->host_stage + off, clouds[i].points, nf * sizeof(float));
     local[i] = clouds[i];
     local[i].points = m->dev_stage + off;
-    off += (int64_t)nf;
-    off = (off + 3) & ~int64_t(3);  // keep every cloud 16-byte aligned
+    off += staged(clouds[i]);
   }
   if (off) EM_TRY(cudaMemcpyAsync(m->dev_stage, m->host_stage, (size_t)off * sizeof(float), cudaMemcpyHostToDevice, s),
                   "upload points");

@@ -1,0 +1,75 @@
+"""The library's host side without a GPU: its objects linked with a stand-in
+for the CUDA runtime (fake_cudart.cpp), driven through the Python binding in a
+process of its own.  Kernels are logged, not run; an access past the end of an
+allocation ends that process with SIGSEGV."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CUDA = "/usr/local/cuda/include"
+
+PRELUDE = """
+import ctypes, sys
+import numpy as np
+sys.path.insert(0, {root!r})
+real = ctypes.CDLL
+ctypes.CDLL = lambda path, *a, **k: real({lib!r} if str(path).endswith("libem.so") else path, *a, **k)
+from paper_2204_12876_gb300 import em
+lib = em.lib
+lib.fake_log.restype = ctypes.c_char_p
+lib.fake_fail_launch.argtypes = [ctypes.c_long]
+em._stream_handle = lambda stream: None
+
+def log(clear=True):
+    lines = lib.fake_log().decode().split("\\n")[:-1]
+    if clear:
+        lib.fake_clear()
+    return lines
+
+POSE = np.eye(3, 4, dtype=np.float32)
+"""
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    """Run a program over the stand-in; its output, and the status it ended with."""
+    from paper_2204_12876_gb300 import build
+    if not os.path.exists(os.path.join(CUDA, "cuda_runtime.h")):
+        pytest.skip("no CUDA headers")
+    build.build()
+    objs = [os.path.join(build.BUILD, os.path.basename(s)[:-3] + ".o") for s in build.sources()]
+    if not all(map(os.path.exists, objs)):
+        build.build(force=True)
+    lib = str(tmp_path_factory.mktemp("fake") / "libem_fake.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CUDA, "-o", lib,
+                    os.path.join(ROOT, "tests", "fake_cudart.cpp"), *objs, "-lpthread"], check=True)
+    prelude = PRELUDE.format(root=ROOT, lib=lib)
+
+    def go(program: str):
+        p = subprocess.run([sys.executable, "-c", prelude + program], capture_output=True, text=True, timeout=300)
+        assert p.returncode == 0, (p.returncode, p.stdout, p.stderr[-2000:])
+        return p.stdout
+    return go
+
+
+@pytest.mark.parametrize("sizes", [(1,), (1, 3, 5), (1,) * 63, (0, 7, 2, 0, 9)])
+@pytest.mark.parametrize("stride", [3, 4])
+def test_host_clouds_stay_inside_the_staging_buffers(run, sizes, stride):
+    """The staged clouds start on 16-byte boundaries, so they take more room than
+    their floats: calls whose floats just fit (and the calls around them) neither
+    write past the pinned buffer nor copy past the device one."""
+    run(f"""
+sizes, stride = {sizes!r}, {stride}
+m = em.Map(em.Params(width=8, height=8))
+floats = sum(sizes) * stride
+first = 4 * 1024                       # any first call: its slack decides the capacity
+m.update_host([(np.zeros((first, 4), np.float32), POSE)])
+cap = 4 * first + first + 1024         # floats, with the slack of that call
+for short in (0, 1, 2, 3, 4, 8):       # one big cloud before the odd ones makes their total cap - short
+    big = (cap - floats - short) // 3
+    m.update_host([(np.ones((big, 3), np.float32), POSE)] + [(np.ones((n, stride), np.float32), POSE) for n in sizes])
+m.close()
+""")
