@@ -39,7 +39,9 @@ enum {
   EM_ERR_INVALID_ARG = -1, /* NULL pointer, bad size / stride, non-finite pose, bad parameter */
   EM_ERR_OOM = -2,         /* a device or pinned-host allocation failed */
   EM_ERR_CUDA = -3,        /* a CUDA call failed; the CUDA error is logged by em_last_cuda_error() */
-  EM_ERR_TIMEOUT = -4,     /* a bounded wait ran out (host or device side) */
+  EM_ERR_TIMEOUT = -4,     /* a bounded wait ran out (host or device side).  From em_sync or em_get_stats after
+                              a persistent batch: the map may hold that update in some of its cells and not in
+                              others (its time has advanced); the next update starts clean */
   EM_ERR_REJECTED = -5,    /* admission refused (memory budget or slot limit) */
   EM_ERR_BUSY = -6,        /* the object is in use by work that has not finished */
   EM_ERR_CAPACITY = -7     /* a request exceeds a fixed capacity chosen at creation */
@@ -260,8 +262,9 @@ typedef struct em_batch em_batch;
  * gate, fusion, ray march, removal) over every map, with grid-wide barriers
  * between them, instead of one kernel per pass (the normals, smoothing and
  * in-painting stencils stay kernels of their own).  Every barrier wait is
- * bounded (EM_PERSIST_WAIT_MS): a wait that runs out gives EM_ERR_TIMEOUT at
- * the maps' next em_sync.  Batches with a drift-compensated map, and devices
+ * bounded (EM_PERSIST_WAIT_MS, or fewer microseconds from the environment
+ * variable EM_PERSIST_WAIT_US when the batch is created): a wait that runs out
+ * gives EM_ERR_TIMEOUT at the maps' next em_sync.  Batches with a drift-compensated map, and devices
  * that cannot run the launch, use the kernel sequence.  Same results either
  * way, bit for bit. */
 enum { EM_BATCH_GRAPH = 1u << 0, EM_BATCH_PERSISTENT = 1u << 1 };

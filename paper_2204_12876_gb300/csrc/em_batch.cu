@@ -7,6 +7,7 @@
 // sequence becomes a graph once per descriptor slot (grids sized from the batch
 // capacities), replayed by one cudaGraphLaunch.
 #include <cuda_runtime.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <algorithm>
@@ -325,7 +326,9 @@ int em_batch_create(int device, int32_t max_maps, int32_t max_clouds, int64_t ma
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->desc_dev, b->desc_bytes * kSlots);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->desc_host, b->desc_bytes * kSlots);
   for (int i = 0; i < kSlots && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&b->ev[i], cudaEventDisableTiming);
-  b->wait_budget = clock_budget(EM_PERSIST_WAIT_MS * 1000ll);
+  long long wait_us = EM_PERSIST_WAIT_MS * 1000ll;
+  if (const char* v = getenv("EM_PERSIST_WAIT_US")) wait_us = std::max(0ll, std::min(wait_us, atoll(v)));
+  b->wait_budget = clock_budget(wait_us);
   if (e != cudaSuccess) {
     release(b);
     return map_record_error("em_batch_create", e);

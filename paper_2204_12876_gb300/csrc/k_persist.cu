@@ -17,7 +17,8 @@
 // end of its barrier's range.  The last block to finish the launch sets the
 // counter back to zero.  Every wait is bounded by a clock64 budget: a wait
 // that runs out raises the abort flag, writes EM_ERR_TIMEOUT into the maps'
-// error words, and every block leaves at its next barrier.
+// error words, and every block leaves at its next barrier; the last one to leave
+// then clears the update's scratch, so the next update starts as after a whole one.
 #include "cell_pass.cuh"
 #include "em.h"
 #include "point_pass.cuh"
@@ -88,16 +89,24 @@ __global__ void __launch_bounds__(kPersistThreads, 4) k_persist(const BatchDev* 
     ok = grid_barrier(b, nb, budget, s_ok);
   }
   if (ok) write_pass(b, all);
-  // the last block to leave makes the barrier state ready for the next launch
+  // the last block to leave makes the barrier state ready for the next launch; when a
+  // wait ran out, some blocks left before their share of the sums, the marks and
+  // write_pass, so it also clears what those passes hand on
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    if (atomicAdd(&b.ctl->bar_done, 1) == nb - 1) {
-      b.ctl->bar_ticket = 0ull;
-      b.ctl->bar_done = 0;
-      b.ctl->bar_abort = 0;
-      __threadfence();
-    }
+    s_ok = atomicAdd(&b.ctl->bar_done, 1) == nb - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_ok) return;
+  if (*(const volatile int*)&b.ctl->bar_abort) clear_scratch(b);
+  __syncthreads();  // (every thread has read the abort flag)
+  if (threadIdx.x == 0) {
+    b.ctl->bar_ticket = 0ull;
+    b.ctl->bar_done = 0;
+    b.ctl->bar_abort = 0;
+    __threadfence();
   }
 }
 
