@@ -5,6 +5,7 @@
 // (pinned host + device copies, each guarded by an event) so that em_update
 // returns without waiting for the GPU.
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -106,6 +107,7 @@ struct em_map {
   int64_t work_bytes = 0;
   int ray_group = 8;
   int64_t points_in = 0;
+  bool dirty = false;  // a launch failed half way through an update: the scratch must be cleared
   // per-kernel profiling
   bool prof = false;
   bool prof_pending = false;
@@ -353,7 +355,25 @@ void map_undo_update(em_map* m, int64_t points) {
   m->points_in -= points;
 }
 
+void map_set_dirty(em_map* m) { m->dirty = true; }
+
+int map_clean(em_map* m, cudaStream_t s) {
+  if (!m->dirty) return EM_OK;
+  const size_t nc = (size_t)m->p.width * m->p.height;
+  EM_TRY(cudaMemsetAsync(m->mark, 0, (nc + 31) / 32 * sizeof(uint32_t), s), "clear scratch");
+  EM_TRY(cudaMemsetAsync(m->acc, 0, nc * sizeof(CellAcc), s), "clear scratch");
+  EM_TRY(cudaMemsetAsync(m->rej, 0, nc * sizeof(uint32_t), s), "clear scratch");
+  if (m->cnt) EM_TRY(cudaMemsetAsync(m->cnt, 0, nc * sizeof(uint32_t), s), "clear scratch");
+  if (m->touched) EM_TRY(cudaMemsetAsync(m->touched, 0, (size_t)(pad_tile((int64_t)nc) / kTile), s), "clear scratch");
+  EM_TRY(cudaMemsetAsync(&m->ctl->drift_h, 0, sizeof(MapCtl) - offsetof(MapCtl, drift_h), s), "clear scratch");
+  EM_TRY(cudaMemsetAsync(m->bctl, 0, sizeof(BatchCtl), s), "clear scratch");
+  m->dirty = false;
+  return EM_OK;
+}
+
 int map_update_one(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t total, cudaStream_t s) {
+  int rc = map_clean(m, s);
+  if (rc) return rc;
   m->t_now += 1;
   m->points_in += total;
   UpdateKind kind = map_kind(m, kValueGroup);
@@ -361,7 +381,9 @@ int map_update_one(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t 
   MapDesc desc;
   fill_desc(m, clouds, n_clouds, total, &desc.b, &desc.m, desc.c);
   const Sequence q = update_sequence(kind, total, desc.b.n_cells);
+  m->dirty = true;  // until every launch has gone through
   for (int i = 0; i < q.n; ++i) EM_TRY(run(q.k[i], &desc, s), q.k[i].name);
+  m->dirty = false;
   map_end_update(m, s, 0);
   return EM_OK;
 }
@@ -513,6 +535,8 @@ static int update_impl(em_map* m, const em_cloud* clouds, int32_t n_clouds, cuda
   for (int i = 0; i < n_clouds; ++i) total += clouds[i].n;
   int rc = grow_workspace(m, total);
   if (rc) return rc;
+  rc = map_clean(m, s);
+  if (rc) return rc;
   m->t_now += 1;
   const int64_t ncell = pad_tile((int64_t)m->p.width * m->p.height);
   UpdateKind kind = map_kind(m, m->ray_group);
@@ -531,8 +555,10 @@ static int update_impl(em_map* m, const em_cloud* clouds, int32_t n_clouds, cuda
     }
   }
   const Sequence q = update_sequence(kind, total, ncell);
+  m->dirty = true;  // until every launch has gone through
   for (int i = 0; i < q.n; ++i)
     EM_TRY(timed(m, q.k[i].slot, s, [&] { return run(q.k[i], arg, s); }), q.k[i].name);
+  m->dirty = false;
   if (slot >= 0) EM_TRY(cudaEventRecord(m->desc_ev[slot], s), "cudaEventRecord");
   m->last_stream = s;
   m->last_n = total;

@@ -51,6 +51,7 @@ struct em_batch {
   unsigned char* desc_dev = nullptr;
   cudaEvent_t ev[kSlots] = {};
   int slot = 0;
+  bool dirty = false;  // a launch failed half way through an update: bctl must be cleared
   em_tuning tune{8, 512, 256};
   cudaGraphExec_t graph[kSlots] = {};
   UpdateKind graph_kind[kSlots] = {};
@@ -144,10 +145,22 @@ int group(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t coun
   return EM_OK;
 }
 
+// A failed update may have stopped between its launches.
+void mark_dirty(em_batch* b) {
+  b->dirty = true;
+  for (em_map* m : b->uniq) map_set_dirty(m);
+}
+
 // Build the descriptor of the grouped pairs in the next slot and upload it.
 int prepare(em_batch* b, const em_cloud* clouds, int32_t count, const std::vector<int64_t>& map_pts, int64_t total,
             const em_tuning& tune, cudaStream_t s, Prepared* out) {
   const int nm = (int)b->uniq.size();
+  if (b->dirty) EB_TRY(cudaMemsetAsync(b->bctl, 0, sizeof(BatchCtl), s), "clear scratch");
+  b->dirty = false;
+  for (em_map* m : b->uniq) {
+    int rc = map_clean(m, s);
+    if (rc) return rc;
+  }
   const int slot = b->slot;
   b->slot = (b->slot + 1) % kSlots;
   EB_TRY(cudaEventSynchronize(b->ev[slot]), "cudaEventSynchronize");
@@ -373,6 +386,7 @@ int em_update_batch(em_batch* b, em_map* const* maps, const em_cloud* clouds, in
     cudaError_t e = launch_sequence(b, update_sequence(p.kind, p.points, p.cells), p.bd, s);
     rc = e == cudaSuccess ? EM_OK : map_record_error("batch launches", e);
   }
+  if (rc) mark_dirty(b);
   finish(b, p, s);
   return rc;
 }
@@ -466,7 +480,10 @@ int em_batch_autotune(em_batch* b, em_map* const* maps, const em_cloud* clouds, 
       cudaError_t le = launch_sequence(b, update_sequence(p.kind, p.points, p.cells), p.bd, s);
       cudaEventRecord(e1, s);
       finish(b, p, s);
-      if (le != cudaSuccess) return map_record_error("autotune launches", le);
+      if (le != cudaSuccess) {
+        mark_dirty(b);
+        return map_record_error("autotune launches", le);
+      }
       if (cudaEventSynchronize(e1) != cudaSuccess) return EM_ERR_CUDA;
       float x = 0.f;
       cudaEventElapsedTime(&x, e0, e1);

@@ -23,6 +23,12 @@ MapDev map_begin_update(em_map* m, int64_t points);
 void map_end_update(em_map* m, cudaStream_t s, int64_t points);
 void map_undo_update(em_map* m, int64_t points);
 
+// An update of map m failed after some of its kernels were launched: its scratch
+// (sums, marks, counters) may not be zero.  map_clean clears it before the next
+// update, on that update's stream; nothing to do otherwise.
+void map_set_dirty(em_map* m);
+int map_clean(em_map* m, cudaStream_t s);
+
 // One update of map m from at most kDescClouds clouds (checked by the caller),
 // total points, as a batch of that map alone does it (no trace, no profiling).
 int map_update_one(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t total, cudaStream_t s);

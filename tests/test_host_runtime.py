@@ -73,3 +73,53 @@ for short in (0, 1, 2, 3, 4, 8):       # one big cloud before the odd ones makes
     m.update_host([(np.ones((big, 3), np.float32), POSE)] + [(np.ones((n, stride), np.float32), POSE) for n in sizes])
 m.close()
 """)
+
+
+@pytest.mark.parametrize("form", ["update", "uploaded", "batch", "batch_of_one"])
+def test_an_update_after_a_failed_launch_starts_with_clear_scratch(run, form):
+    """A launch that fails half way leaves sums and marks behind: the next update of
+    those maps clears them on its stream before its first kernel, and only that
+    one does."""
+    run(f"""
+form = {form!r}
+P = em.Params(width=70, height=50, ray_step=0.04, wall_num_thresh=2, drift_flatness=0.9, flags=em.F_NORMALS)
+maps = [em.Map(P), em.Map(P)]
+batch = em.Batch(max_maps=2, max_clouds=16, max_points=1000, max_cells=3500, graph=False)
+pts = np.zeros((20, 3), np.float32)
+clouds = [(pts, POSE)] * (12 if form == "uploaded" else 1)
+
+def update():
+    if form.startswith("batch"):
+        use = maps if form == "batch" else maps[:1]
+        h = (ctypes.c_void_p * len(use))(*[m.handle.value for m in use])
+        c = (em._Cloud * len(use))(*[em._cloud_struct(pts, POSE, True) for _ in use])
+        em._check(lib.em_update_batch(batch._h, h, c, len(use), None), "em_update_batch")
+    else:
+        arr = (em._Cloud * len(clouds))(*[em._cloud_struct(p, q, True) for p, q in clouds])
+        em._check(lib.em_update_multi(maps[0]._h, arr, len(arr), None), "em_update_multi")
+
+log()
+update()
+whole = log()
+n = sum(l.startswith("launch") for l in whole)
+assert n == 5 and not any(l.startswith("memset") for l in whole), whole
+cells = 70 * 50
+for k in range(2, n + 1):  # the first k - 1 kernels are launched, the k-th is not
+    lib.fake_fail_launch(k)
+    try:
+        update()
+        raise SystemExit("the failed launch was not reported")
+    except em.EMError as e:
+        assert e.code == em.EM_ERR_CUDA
+    log()
+    update()
+    lines = log()
+    first = next(i for i, l in enumerate(lines) if l.startswith("launch"))
+    sizes = [int(l.split()[2]) for l in lines[:first] if l.startswith("memset")]
+    assert not any(l.startswith("memset") for l in lines[first:])
+    users = 2 if form == "batch" else 1
+    for want in (cells * 32, cells * 4, (cells + 31) // 32 * 4):  # sums; rejected and counted points; marks
+        assert sizes.count(want) == users * (2 if want == cells * 4 else 1), (k, sizes)
+    update()
+    assert log() == whole  # clean again
+""")
