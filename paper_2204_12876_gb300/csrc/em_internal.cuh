@@ -320,6 +320,8 @@ cudaError_t launch_fill_map(const MapDev& m, cudaStream_t s);
 // Start of every kernel of an update: it may have been launched while the
 // kernel before it on the stream still ran (launch.cu), so it waits for that
 // one's end and memory, then lets the next one be launched in the same way.
+// What the kernel before may have written -- layers, and the caller's points --
+// was not read-only while this one ran, so no kernel reads with __ldg.
 __device__ __forceinline__ void begin_after_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");

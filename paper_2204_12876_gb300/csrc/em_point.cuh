@@ -127,9 +127,9 @@ __device__ __forceinline__ void key_runs(unsigned long long tag, int& head, int&
 // Load point g of cloud c (stride 3 or 4) with scalar loads.
 __device__ __forceinline__ void load_point(const CloudDev& c, int64_t i, float& px, float& py, float& pz) {
   const float* p = c.pts + i * c.stride;
-  px = __ldg(p);
-  py = __ldg(p + 1);
-  pz = __ldg(p + 2);
+  px = p[0];
+  py = p[1];
+  pz = p[2];
 }
 
 // Load the warp's 32 points [wbase, wbase + 32).  When the whole chunk sits in
@@ -151,12 +151,12 @@ __device__ __forceinline__ int load_warp_points(const V& b, int64_t wbase, int64
     const int64_t i0 = wbase - cl0.begin;
     const float* base = cl0.pts + i0 * cl0.stride;
     if (cl0.stride == 4 && ((reinterpret_cast<uintptr_t>(base) & 15) == 0)) {
-      float4 q = __ldg(reinterpret_cast<const float4*>(base) + lane);
+      const float4 q = reinterpret_cast<const float4*>(base)[lane];
       px = q.x; py = q.y; pz = q.z;
       return ci;
     }
     if (cl0.stride == 3 && ((reinterpret_cast<uintptr_t>(base) & 15) == 0)) {
-      if (lane < 24) stage[lane] = __ldg(reinterpret_cast<const float4*>(base) + lane);
+      if (lane < 24) stage[lane] = reinterpret_cast<const float4*>(base)[lane];
       __syncwarp();
       const float* sf = reinterpret_cast<const float*>(stage);
       px = sf[lane * 3];

@@ -248,7 +248,7 @@ __device__ __forceinline__ void inpaint_tile(const MapDev& m, int32_t tx, int32_
     for (int half = 0; half < 2; ++half) {
       const int32_t y = y0 + warp * kPerWarp + k, x = x0 + half * 32 + lane;
       const bool in = y >= 0 && y < m.H && x >= 0 && x < m.W && half * 32 + lane < kIpSpan;
-      empty[k][half] = in && !isfinite(__ldg(m.var + (in ? phys_index(m, x, y) : 0)));
+      empty[k][half] = in && !isfinite(m.var[in ? phys_index(m, x, y) : 0]);
     }
 #pragma unroll
   for (int k = 0; k < kPerWarp; ++k) {
