@@ -31,6 +31,9 @@ static_assert(kPersistThreads == kPointThreads && kPersistThreads == kCellThread
 constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
 // the passes run one after another and share one shared-memory buffer
 constexpr size_t kPersistSmem = cmax(sizeof(PointsSmem<true>), sizeof(PreSmem));
+constexpr size_t kPersistAlign = 32;
+static_assert(kPersistAlign >= alignof(PointsSmem<true>) && kPersistAlign >= alignof(PreSmem),
+              "the buffer starts where the passes' structs may");
 
 // Wait until *word >= target, or until `abort` is raised, for at most budget
 // SM clock cycles; true when the word got there.
@@ -65,7 +68,7 @@ __device__ __forceinline__ bool grid_barrier(const BatchDev& b, int nb, long lon
 
 template <int G, bool kExt>
 __global__ void __launch_bounds__(kPersistThreads, 4) k_persist(const BatchDev* __restrict__ bp) {
-  extern __shared__ __align__(16) unsigned char sm[];
+  extern __shared__ __align__(kPersistAlign) unsigned char sm[];
   __shared__ int s_ok;
   begin_after_previous();
   const BatchDev& b = *bp;
