@@ -605,7 +605,7 @@ class Server:
                 if out.dtype is not f32 or not out.is_contiguous():
                     raise ValueError("read-back buffer must be a contiguous float32 tensor")
                 to_host, dst = 0 if out.is_cuda else 1, out.data_ptr()
-            _REQUEST.pack_into(buf, at, ctypes.c_int32(map_id).value, len(clouds), first, int(mask) & 0xffffffff,
+            _REQUEST.pack_into(buf, at, ctypes.c_int32(int(map_id)).value, len(clouds), first, int(mask) & 0xffffffff,
                                to_host, dst, 1 if on_host else 0)
             at += _REQUEST.size
         tks = (ctypes.c_uint64 * n)()
