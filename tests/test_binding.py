@@ -41,13 +41,12 @@ def test_requests_take_any_map_id_that_is_an_int(monkeypatch, map_id):
             tickets[i] = 10 + i
         return 0
 
-    monkeypatch.setattr(em, "lib", types.SimpleNamespace(em_server_submit_many=submit, em_server_destroy=lambda h: 0))
+    monkeypatch.setattr(em, "lib", types.SimpleNamespace(em_server_submit_many=submit))
     s = object.__new__(em.Server)
-    s._h, s._keep = ctypes.c_void_p(1), {}
+    s._h, s._keep = None, {}
     poses = [np.arange(12.0), np.arange(12, dtype=np.float32).reshape(3, 4) + 1, list(range(2, 14))]
     clouds = [(DeviceCloud(5 + k, 3 + k % 2, 4096 * (k + 1)), q) for k, q in enumerate(poses)]
     assert s.submit_many([(map_id, clouds, None), (0, clouds[1:], None)]) == [10, 11]
     want = ctypes.c_int32(int(map_id)).value
     assert seen == [(want, 3, 0, 0, 4096, 5, 3, [float(v) for v in range(2, 14)]),
                     (0, 2, 0, 0, 8192, 6, 4, [float(v) for v in range(2, 14)])]
-    s._h = None
