@@ -265,6 +265,7 @@ void fill_desc(const em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_
   b->tr_iy = m->tr_iy;
   b->tr_status = m->tr_status;
   b->n_cells = pad_tile((int64_t)m->p.width * m->p.height);
+  if (!use_flags(b->n_cells, total)) md->touched = nullptr;
   b->n_items = (int64_t)md->IW * md->IH;
   b->ctl = m->bctl;
 }
@@ -364,7 +365,7 @@ int map_clean(em_map* m, cudaStream_t s) {
   EM_TRY(cudaMemsetAsync(m->acc, 0, nc * sizeof(CellAcc), s), "clear scratch");
   EM_TRY(cudaMemsetAsync(m->rej, 0, nc * sizeof(uint32_t), s), "clear scratch");
   if (m->cnt) EM_TRY(cudaMemsetAsync(m->cnt, 0, nc * sizeof(uint32_t), s), "clear scratch");
-  if (m->touched) EM_TRY(cudaMemsetAsync(m->touched, 0, (size_t)(pad_tile((int64_t)nc) / kTile), s), "clear scratch");
+  EM_TRY(cudaMemsetAsync(m->touched, 0, (size_t)(pad_tile((int64_t)nc) / kTile), s), "clear scratch");
   EM_TRY(cudaMemsetAsync(&m->ctl->drift_h, 0, sizeof(MapCtl) - offsetof(MapCtl, drift_h), s), "clear scratch");
   EM_TRY(cudaMemsetAsync(m->bctl, 0, sizeof(BatchCtl), s), "clear scratch");
   m->dirty = false;
@@ -480,7 +481,7 @@ int em_create(const em_params* params, int device, em_map** out) {
     EM_ALLOC(m->thr, nc) EM_ALLOC(m->cthr, nb)
   }
   EM_ALLOC(m->acc, nc) EM_ALLOC(m->rej, nc)
-  if ((int64_t)nc > kFlagCells) { EM_ALLOC(m->touched, ntile) }
+  EM_ALLOC(m->touched, ntile)
   if (params->wall_num_thresh > 0) { EM_ALLOC(m->cnt, nc) }
   EM_ALLOC(m->ctl, 1) EM_ALLOC(m->bctl, 1)
   EM_ALLOC(m->desc_dev, kDescBytes * kSlots)
@@ -493,7 +494,7 @@ int em_create(const em_params* params, int device, em_map** out) {
   if (e == cudaSuccess) e = cudaMemset(m->acc, 0, nc * sizeof(CellAcc));
   if (e == cudaSuccess) e = cudaMemset(m->rej, 0, nc * sizeof(uint32_t));
   if (e == cudaSuccess && m->cnt) e = cudaMemset(m->cnt, 0, nc * sizeof(uint32_t));
-  if (e == cudaSuccess && m->touched) e = cudaMemset(m->touched, 0, ntile);
+  if (e == cudaSuccess) e = cudaMemset(m->touched, 0, ntile);
   if (e == cudaSuccess) e = cuda_status(launch_fill_map(make_mapdev(m), nullptr), "fill") ? cudaErrorUnknown : cudaSuccess;
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {

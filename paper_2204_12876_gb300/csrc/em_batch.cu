@@ -218,6 +218,7 @@ int prepare(em_batch* b, const em_cloud* clouds, int32_t count, const std::vecto
   bd->maps = reinterpret_cast<const MapDev*>(db + sizeof(BatchDev));
   bd->clouds = reinterpret_cast<const CloudDev*>(db + sizeof(BatchDev) + (size_t)b->max_maps * sizeof(MapDev));
   bd->n_cells = cells;
+  for (int u = 0; u < nm && !use_flags(cells, total); ++u) md[u].touched = nullptr;
   bd->n_items = items;
   bd->ctl = b->bctl;
   bd->passes = (kind.wall || kind.drift ? kPassPre : 0u) | (kind.ray || kind.drift ? kPassCells : 0u);

@@ -93,12 +93,16 @@ constexpr int kParts = 3;
 constexpr uint32_t kSplitPoints = 1u << 20;
 constexpr int kOrderSamples = 64;
 
-// Maps beyond this many cells keep a flag per tile, so that a cloud on a corner of
-// a huge map does not cost a read of all its accumulators.  Smaller maps' flags
-// would be a few sectors that every warp of the update writes: without them a
-// raw depth image took 45 us instead of 49, four depth cameras 36.8 instead of
-// 38.5, and reading the accumulators of the untouched tiles costs less.
+// Updates of more than kFlagCells cells (all maps together) of which the points can
+// touch half at most keep a flag per tile, so that clouds on a few cells of large maps
+// do not cost a read of all their accumulators (32 maps of 1,000,000 cells, 5,000
+// points each: 214 us without flags, 143 with).  In smaller updates the flags would
+// be a few sectors that every warp writes: without them a raw depth image took 45 us
+// instead of 49, four depth cameras 36.8 instead of 38.5; and where the points are as
+// many as the cells most tiles are touched anyhow (64-map batch, 14 M points on 6.8 M
+// cells: 2196 us without, 2212 with).
 constexpr int64_t kFlagCells = 1 << 20;
+inline bool use_flags(int64_t n_cells, int64_t n_points) { return n_cells > kFlagCells && n_cells >= 2 * n_points; }
 
 constexpr int kItemW = 32, kItemH = 8;  // k_cells: logical cells per warp item
 
@@ -130,8 +134,8 @@ struct MapDev {
   CellAcc* acc;     // per physical cell
   uint32_t* rej;    // rejected points per physical cell, zero between updates
   uint32_t* cnt;    // wall rule: points per physical cell, zero between updates; null without the rule
-  uint8_t* touched; // per tile of kTile cells: some point of this update fell into it; null for maps of at
-                    // most kFlagCells cells, whose tiles all count as touched
+  uint8_t* touched; // per tile of kTile cells: some point of this update fell into it; null when the update
+                    // keeps no flags (use_flags): all tiles count as touched
   int64_t ibegin;   // this map's first item in the batch's item space (maps with the ray march or drift)
   int32_t IW, IH;   // items per row and column; 0 x 0 without the ray march and the drift compensation
   int32_t CW, CH, CS;  // coarse blocks per row and column (0 x 0 without the ray march), row stride
