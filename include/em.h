@@ -131,7 +131,7 @@ typedef struct em_info {
   int32_t t_now;           /* number of updates fused so far */
   int64_t shift_x, shift_y;/* cumulative em_shift in cells; the map centre is (shift_x r, shift_y r) */
   double x0, y0;           /* lower-left corner of the map in the map frame */
-  int64_t point_capacity;  /* points per update reserved for (em_reserve); the trace holds as many */
+  int64_t point_capacity;  /* points per update that need no allocation (em_reserve) */
   int64_t device_bytes;    /* device memory held by the map */
 } em_info;
 
@@ -164,7 +164,9 @@ int em_create(const em_params* params, int device, em_map** out);
 int em_destroy(em_map* map);
 
 /* Grow the workspace so that updates of up to max_points points (all clouds
- * of one update together) need no allocation.  Synchronous. */
+ * of one update together) need no allocation.  Maps of more than 2^19 cells
+ * keep memory per point (their sums, about 80 bytes), smaller ones only with
+ * EM_F_TRACE.  Synchronous. */
 int em_reserve(em_map* map, int64_t max_points);
 
 /* Fuse one point cloud (device pointer, n points, stride 3 or 4 floats) seen
@@ -233,7 +235,8 @@ enum {
                           visibility ray march */
   EM_PROF_ALLOC,       /* (no kernel) */
   EM_PROF_SCATTER,     /* k_pre: points per cell for the wall rule, drift sums */
-  EM_PROF_FUSE,        /* k_write: new state of every cell, removal, overlap clearance */
+  EM_PROF_FUSE,        /* k_write (after k_sums, for maps of more than 2^19 cells): new state of every cell,
+                          removal, overlap clearance */
   EM_PROF_CLEAR,       /* (no kernel) */
   EM_PROF_NORMALS,     /* k_stencils: normals, smoothing, in-painting */
   EM_PROF_SMOOTH,      /* (no kernel) */

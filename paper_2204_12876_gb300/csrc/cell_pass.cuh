@@ -3,8 +3,9 @@
 //   cells_pass  before the points: estimates moved by the drift, ray thresholds
 //               of the pre-update map and their largest per coarse block
 //   refresh_pass  between parts of the points: marked cells out of both
-//   write_pass  after them: every cell's new state from its sums, removal of
-//               marked cells, overlap clearance
+//   sums_pass   after them: new state of the cells whose sums are in the table
+//   write_pass  every cell's new state from its sums, removal of marked cells,
+//               overlap clearance
 //
 // Each pass runs on the blocks of a Grid: its own kernel's, or the persistent
 // kernel's (k_persist.cu).
@@ -205,6 +206,46 @@ __device__ __forceinline__ void clear_acc(CellAcc* p) {
   asm volatile("st.global.v4.u64 [%0], {%1, %1, %1, %1};" ::"l"(p), "l"(0ull) : "memory");
 }
 
+// The cells of maps with keys: a slot of the table per thread and round.  Freed
+// slots, sums and counts go back to zero.  The cells are written now, so write_pass,
+// which runs after this, finds them too young to remove (Section II-E).
+template <class V>
+__device__ __forceinline__ void sums_pass(const V& b, Grid gr) {
+  const SumTable& t = b.tab;
+  const int lane = threadIdx.x & 31;
+  for (int64_t base = (int64_t)gr.bid * kCellThreads; base < t.slots; base += (int64_t)gr.nb * kCellThreads) {
+    const int64_t i = base + threadIdx.x;
+    const unsigned long long key = i < t.slots ? t.keys[i] : 0ull;
+    int updated = -1;  // the map whose cell this lane writes
+    if (key) {
+      const CellAcc a = load_acc(t.acc + i);
+      const uint32_t rej = t.rej[i];
+      const int64_t g = (int64_t)(key - 1ull);
+      const int mi = find_map_cell(b.maps, b.n_maps, g);
+      const MapDev& m = map_at(b, mi);
+      const int32_t c = (int32_t)(g - m.cell_begin);
+      const bool acc = (a.wh | a.wl) != 0;
+      if (acc || rej) {
+        float hn, vn;
+        fused_state(m, m.h[c], m.var[c], m.t_last[c], fix128((long long)a.wh, a.wl & ~kAccTouched),
+                    fix128((long long)a.th, a.tl), acc, rej, hn, vn);
+        m.h[c] = hn;
+        m.var[c] = vn;
+        m.t_last[c] = m.t_now;
+        if (m.upper) m.upper[c] = __int_as_float(0x7f800000);  // observed: no bound (Section II-H)
+        updated = mi;
+      }
+      t.keys[i] = 0ull;
+      if (acc) clear_acc(t.acc + i);
+      if (rej) t.rej[i] = 0;
+      if (m.cnt) t.cnt[i] = 0;
+    }
+    const unsigned same = __match_any_sync(kFull, updated);
+    if (updated >= 0 && lane == __ffs(same) - 1)
+      atomicAdd(&map_at(b, updated).ctl->stats[kStCellsUpdated], (unsigned long long)__popc(same));
+  }
+}
+
 // One block per tile of kTile cells, a cell per thread and round: the sums of
 // the tile's four rounds are in flight together.  Sums, counts, marks and the
 // tile's flag go back to zero for the next update.  Tiles start on multiples of
@@ -225,7 +266,7 @@ __device__ __forceinline__ void write_pass(const V& b, Grid gr) {
       m.ctl->drift_l = 0;
       m.ctl->drift_n = 0;
     }
-    const bool touched = !m.touched || m.touched[tile] != 0;
+    const bool touched = m.acc && !m.keys && (!m.touched || m.touched[tile] != 0);
     const bool overlap = m.ovl_dz > 0.f;
     CellAcc a[kWriteRounds];
     uint32_t rej[kWriteRounds], mark[kWriteRounds];
@@ -313,10 +354,13 @@ __device__ __forceinline__ void clear_scratch(const V& b) {
   for (int mi = 0; mi < b.n_maps; ++mi) {
     const MapDev& m = map_at(b, mi);
     const int32_t ncell = m.W * m.H;
+    const bool flat = m.acc && !m.keys;
     for (int32_t c = threadIdx.x; c < ncell; c += blockDim.x) {
-      clear_acc(m.acc + c);
-      m.rej[c] = 0;
-      if (m.cnt) m.cnt[c] = 0;
+      if (flat) {
+        clear_acc(m.acc + c);
+        m.rej[c] = 0;
+        if (m.cnt) m.cnt[c] = 0;
+      }
       if (c % 32 == 0) m.mark[c / 32] = 0;
       if (m.touched && c % kTile == 0) m.touched[c / kTile] = 0;
     }
@@ -325,6 +369,12 @@ __device__ __forceinline__ void clear_scratch(const V& b) {
       m.ctl->drift_l = 0;
       m.ctl->drift_n = 0;
     }
+  }
+  for (int64_t i = threadIdx.x; i < b.tab.slots; i += blockDim.x) {
+    b.tab.keys[i] = 0ull;
+    clear_acc(b.tab.acc + i);
+    b.tab.rej[i] = 0;
+    if (b.tab.cnt) b.tab.cnt[i] = 0;
   }
 }
 

@@ -15,6 +15,7 @@
 #include <new>
 
 #include "em.h"
+#include "em_host.h"
 #include "em_internal.cuh"
 
 using namespace em;
@@ -77,6 +78,8 @@ struct em_map {
   uint32_t* rej = nullptr;
   uint32_t* cnt = nullptr;       // maps with the wall rule
   uint8_t* touched = nullptr;    // per tile of 1024 cells
+  SumTable tab{};                // maps beyond kFlatCells: acc, rej and cnt are the table's while it has slots
+  int64_t sums_bytes = 0;        // ... and the memory of either
   MapCtl* ctl = nullptr;
   BatchCtl* bctl = nullptr;
   // geometry
@@ -131,7 +134,7 @@ MapDev make_mapdev(const em_map* m) {
   d.h = m->h; d.var = m->var; d.t_last = m->t_last;
   d.nx = m->nx; d.ny = m->ny; d.nz = m->nz; d.smooth = m->smooth; d.inpaint = m->inpaint; d.upper = m->upper;
   d.mark = m->mark; d.thr = m->thr;
-  d.acc = m->acc; d.rej = m->rej; d.cnt = m->cnt; d.touched = m->touched;
+  d.acc = m->acc; d.rej = m->rej; d.cnt = m->cnt; d.keys = m->tab.keys; d.touched = m->touched;
   set_item_grid(d, m->p.width, m->p.height, m->p.ray_step > 0.f, m->p.drift_flatness > 0.f);
   if (m->cthr) d.cthr = m->cthr + coarse_first(m->p.width);
   d.ctl = m->ctl;
@@ -179,6 +182,50 @@ bool params_ok(const em_params* p) {
   return true;
 }
 
+// The sums of a map beyond kFlatCells, for updates of up to `points` points: a
+// table, or an accumulator per cell where that is no larger.
+int grow_sums(em_map* m, int64_t points) {
+  const int64_t nc = (int64_t)m->p.width * m->p.height;
+  if (nc <= kFlatCells || (m->acc && !m->tab.slots)) return EM_OK;
+  const int64_t slots = table_slots(std::min(points, nc));
+  const int64_t cell = sizeof(CellAcc) + 4 + (m->p.wall_num_thresh > 0 ? 4 : 0);
+  if (slots <= m->tab.slots) return EM_OK;
+  EM_TRY(cudaDeviceSynchronize(), "cudaDeviceSynchronize");
+  table_free(&m->tab);
+  m->acc = nullptr;
+  m->rej = m->cnt = nullptr;
+  m->sums_bytes = 0;
+  m->cap = 0;  // (until the new ones are there)
+  if (slots * (cell + 8) < nc * cell) {
+    EM_TRY(table_alloc(&m->tab, slots, m->p.wall_num_thresh > 0, &m->sums_bytes), "alloc sums");
+    m->acc = m->tab.acc;
+    m->rej = m->tab.rej;
+    m->cnt = m->tab.cnt;
+    return EM_OK;
+  }
+  CellAcc* acc = nullptr;
+  uint32_t *rej = nullptr, *cnt = nullptr;
+  int64_t tot = 0;
+  cudaError_t e = dev_alloc(&acc, (size_t)nc, &tot);
+  if (e == cudaSuccess) e = cudaMemset(acc, 0, (size_t)nc * sizeof(CellAcc));
+  if (e == cudaSuccess) e = dev_alloc(&rej, (size_t)nc, &tot);
+  if (e == cudaSuccess) e = cudaMemset(rej, 0, (size_t)nc * 4);
+  if (e == cudaSuccess && m->p.wall_num_thresh > 0) {
+    e = dev_alloc(&cnt, (size_t)nc, &tot);
+    if (e == cudaSuccess) e = cudaMemset(cnt, 0, (size_t)nc * 4);
+  }
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) {
+    cudaFree(acc); cudaFree(rej); cudaFree(cnt);
+    return cuda_status(e, "alloc sums");
+  }
+  m->acc = acc;
+  m->rej = rej;
+  m->cnt = cnt;
+  m->sums_bytes = tot;
+  return EM_OK;
+}
+
 void free_workspace(em_map* m) {
   cudaFree(m->tr_ix); cudaFree(m->tr_iy); cudaFree(m->tr_status);
   m->tr_ix = m->tr_iy = nullptr;
@@ -193,6 +240,8 @@ int grow_workspace(em_map* m, int64_t n) {
   int64_t want = n + n / 4;
   if (want < 4096) want = 4096;
   if (want > (int64_t(1) << 31) - 1) want = (int64_t(1) << 31) - 1;
+  int rc = grow_sums(m, want);
+  if (rc) return rc;
   if (m->p.flags & EM_F_TRACE) {
     EM_TRY(cudaDeviceSynchronize(), "cudaDeviceSynchronize");
     free_workspace(m);
@@ -213,7 +262,9 @@ void release(em_map* m) {
   cudaFree(m->h); cudaFree(m->var); cudaFree(m->t_last);
   cudaFree(m->nx); cudaFree(m->ny); cudaFree(m->nz); cudaFree(m->smooth); cudaFree(m->inpaint); cudaFree(m->upper);
   cudaFree(m->mark); cudaFree(m->thr); cudaFree(m->cthr);
-  cudaFree(m->acc); cudaFree(m->rej); cudaFree(m->cnt); cudaFree(m->touched);
+  if (m->tab.slots) table_free(&m->tab);
+  else { cudaFree(m->acc); cudaFree(m->rej); cudaFree(m->cnt); }
+  cudaFree(m->touched);
   cudaFree(m->ctl); cudaFree(m->bctl);
   free_workspace(m);
   cudaFree(m->desc_dev);
@@ -265,9 +316,10 @@ void fill_desc(const em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_
   b->tr_iy = m->tr_iy;
   b->tr_status = m->tr_status;
   b->n_cells = pad_tile((int64_t)m->p.width * m->p.height);
-  if (!use_flags(b->n_cells, total)) md->touched = nullptr;
+  if (md->keys || !use_flags(b->n_cells, total)) md->touched = nullptr;
   b->n_items = (int64_t)md->IW * md->IH;
   b->ctl = m->bctl;
+  b->tab = m->tab;
 }
 
 // Build and upload the descriptor of a one-map update (more clouds than a
@@ -356,15 +408,57 @@ void map_undo_update(em_map* m, int64_t points) {
   m->points_in -= points;
 }
 
+bool map_has_room(const em_map* m, int64_t points) {
+  return (int64_t)m->p.width * m->p.height <= kFlatCells || (points <= m->cap && m->acc);
+}
+
+cudaError_t table_alloc(SumTable* t, int64_t slots, bool cnt, int64_t* bytes) {
+  SumTable n{};
+  const size_t rows = (size_t)slots + 1;  // with the spare slot
+  int64_t tot = 0;
+  cudaError_t e = dev_alloc(&n.keys, rows, &tot);
+  if (e == cudaSuccess) e = dev_alloc(&n.acc, rows, &tot);
+  if (e == cudaSuccess) e = dev_alloc(&n.rej, rows, &tot);
+  if (e == cudaSuccess && cnt) e = dev_alloc(&n.cnt, rows, &tot);
+  n.slots = (uint32_t)slots;
+  if (e == cudaSuccess) e = table_clear(n, nullptr);
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) {
+    table_free(&n);
+    return e;
+  }
+  *t = n;
+  if (bytes) *bytes += tot;
+  return cudaSuccess;
+}
+
+void table_free(SumTable* t) {
+  cudaFree(t->keys); cudaFree(t->acc); cudaFree(t->rej); cudaFree(t->cnt);
+  *t = SumTable{};
+}
+
+cudaError_t table_clear(const SumTable& t, cudaStream_t s) {
+  const size_t rows = (size_t)t.slots + 1;
+  cudaError_t e = cudaMemsetAsync(t.keys, 0, rows * sizeof(*t.keys), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(t.acc, 0, rows * sizeof(*t.acc), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(t.rej, 0, rows * sizeof(*t.rej), s);
+  if (e == cudaSuccess && t.cnt) e = cudaMemsetAsync(t.cnt, 0, rows * sizeof(*t.cnt), s);
+  return e;
+}
+
 void map_set_dirty(em_map* m) { m->dirty = true; }
 
 int map_clean(em_map* m, cudaStream_t s) {
   if (!m->dirty) return EM_OK;
   const size_t nc = (size_t)m->p.width * m->p.height;
   EM_TRY(cudaMemsetAsync(m->mark, 0, (nc + 31) / 32 * sizeof(uint32_t), s), "clear scratch");
-  EM_TRY(cudaMemsetAsync(m->acc, 0, nc * sizeof(CellAcc), s), "clear scratch");
-  EM_TRY(cudaMemsetAsync(m->rej, 0, nc * sizeof(uint32_t), s), "clear scratch");
-  if (m->cnt) EM_TRY(cudaMemsetAsync(m->cnt, 0, nc * sizeof(uint32_t), s), "clear scratch");
+  if (m->tab.slots) {
+    EM_TRY(table_clear(m->tab, s), "clear scratch");
+  } else if (m->acc) {
+    EM_TRY(cudaMemsetAsync(m->acc, 0, nc * sizeof(CellAcc), s), "clear scratch");
+    EM_TRY(cudaMemsetAsync(m->rej, 0, nc * sizeof(uint32_t), s), "clear scratch");
+    if (m->cnt) EM_TRY(cudaMemsetAsync(m->cnt, 0, nc * sizeof(uint32_t), s), "clear scratch");
+  }
   EM_TRY(cudaMemsetAsync(m->touched, 0, (size_t)(pad_tile((int64_t)nc) / kTile), s), "clear scratch");
   EM_TRY(cudaMemsetAsync(&m->ctl->drift_h, 0, sizeof(MapCtl) - offsetof(MapCtl, drift_h), s), "clear scratch");
   EM_TRY(cudaMemsetAsync(m->bctl, 0, sizeof(BatchCtl), s), "clear scratch");
@@ -379,6 +473,8 @@ int map_update_one(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t 
   m->points_in += total;
   UpdateKind kind = map_kind(m, kValueGroup);
   kind.by_value = true;
+  kind.slots = m->tab.slots;
+  kind.ext |= kind.slots > 0;
   MapDesc desc;
   fill_desc(m, clouds, n_clouds, total, &desc.b, &desc.m, desc.c);
   const Sequence q = update_sequence(kind, total, desc.b.n_cells);
@@ -480,9 +576,10 @@ int em_create(const em_params* params, int device, em_map** out) {
     const size_t nb = (size_t)coarse_size(params->width, params->height);
     EM_ALLOC(m->thr, nc) EM_ALLOC(m->cthr, nb)
   }
-  EM_ALLOC(m->acc, nc) EM_ALLOC(m->rej, nc)
   EM_ALLOC(m->touched, ntile)
-  if (params->wall_num_thresh > 0) { EM_ALLOC(m->cnt, nc) }
+  const bool flat = (int64_t)nc <= kFlatCells;  // larger maps' sums are allocated for their updates' points (grow_sums)
+  if (flat) { EM_ALLOC(m->acc, nc) EM_ALLOC(m->rej, nc) }
+  if (flat && params->wall_num_thresh > 0) { EM_ALLOC(m->cnt, nc) }
   EM_ALLOC(m->ctl, 1) EM_ALLOC(m->bctl, 1)
   EM_ALLOC(m->desc_dev, kDescBytes * kSlots)
 #undef EM_ALLOC
@@ -491,8 +588,8 @@ int em_create(const em_params* params, int device, em_map** out) {
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->stage_ev, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMemset(m->ctl, 0, sizeof(MapCtl));
   if (e == cudaSuccess) e = cudaMemset(m->bctl, 0, sizeof(BatchCtl));
-  if (e == cudaSuccess) e = cudaMemset(m->acc, 0, nc * sizeof(CellAcc));
-  if (e == cudaSuccess) e = cudaMemset(m->rej, 0, nc * sizeof(uint32_t));
+  if (e == cudaSuccess && m->acc) e = cudaMemset(m->acc, 0, nc * sizeof(CellAcc));
+  if (e == cudaSuccess && m->rej) e = cudaMemset(m->rej, 0, nc * sizeof(uint32_t));
   if (e == cudaSuccess && m->cnt) e = cudaMemset(m->cnt, 0, nc * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(m->touched, 0, ntile);
   if (e == cudaSuccess) e = cuda_status(launch_fill_map(make_mapdev(m), nullptr), "fill") ? cudaErrorUnknown : cudaSuccess;
@@ -541,6 +638,8 @@ static int update_impl(em_map* m, const em_cloud* clouds, int32_t n_clouds, cuda
   m->t_now += 1;
   const int64_t ncell = pad_tile((int64_t)m->p.width * m->p.height);
   UpdateKind kind = map_kind(m, m->ray_group);
+  kind.slots = m->tab.slots;
+  kind.ext |= kind.slots > 0;
   kind.by_value = n_clouds <= kDescClouds && m->ray_group == kValueGroup;
   MapDesc desc;
   const BatchDev* bd = nullptr;
@@ -725,7 +824,7 @@ int em_get_info(const em_map* m, em_info* out) {
   out->shift_y = m->shift_y;
   host_origin(m, &out->x0, &out->y0);
   out->point_capacity = m->cap;
-  out->device_bytes = m->layer_bytes + m->work_bytes + (int64_t)m->layer_stage_cap * 4 + m->stage_cap * 4;
+  out->device_bytes = m->layer_bytes + m->work_bytes + m->sums_bytes + (int64_t)m->layer_stage_cap * 4 + m->stage_cap * 4;
   return EM_OK;
 }
 

@@ -45,6 +45,7 @@ struct em_batch {
   int64_t max_points = 0;
   uint32_t flags = 0;
   BatchCtl* bctl = nullptr;
+  SumTable tab{};         // for maps beyond kFlatCells; no slots when max_cells allows none
   long long wait_budget = 0;  // SM clock cycles of EM_PERSIST_WAIT_MS
   size_t desc_bytes = 0;
   unsigned char* desc_host = nullptr;
@@ -156,6 +157,7 @@ int prepare(em_batch* b, const em_cloud* clouds, int32_t count, const std::vecto
             const em_tuning& tune, cudaStream_t s, Prepared* out) {
   const int nm = (int)b->uniq.size();
   if (b->dirty) EB_TRY(cudaMemsetAsync(b->bctl, 0, sizeof(BatchCtl), s), "clear scratch");
+  if (b->dirty && b->tab.slots) EB_TRY(table_clear(b->tab, s), "clear scratch");
   b->dirty = false;
   for (em_map* m : b->uniq) {
     int rc = map_clean(m, s);
@@ -173,11 +175,21 @@ int prepare(em_batch* b, const em_cloud* clouds, int32_t count, const std::vecto
   UpdateKind kind{};
   kind.ray_group = tune.ray_group;
   kind.persistent = (b->flags & EM_BATCH_PERSISTENT) != 0;
-  int64_t cells = 0, items = 0;
+  int64_t cells = 0, flat_cells = 0, items = 0;
   for (int u = 0; u < nm; ++u) {
     md[u] = map_begin_update(b->uniq[u], map_pts[u]);
     md[u].cell_begin = cells;
     cells += pad_tile(map_cells(b->uniq[u]));
+    if (map_cells(b->uniq[u]) > kFlatCells) {
+      md[u].acc = b->tab.acc;
+      md[u].rej = b->tab.rej;
+      md[u].cnt = md[u].wall > 0 ? b->tab.cnt : nullptr;
+      md[u].keys = b->tab.keys;
+      kind.slots = b->tab.slots;
+      kind.ext = true;
+    } else {
+      flat_cells += pad_tile(map_cells(b->uniq[u]));
+    }
     md[u].ibegin = items;
     items += (int64_t)md[u].IW * md[u].IH;
     const UpdateKind k = map_kind(b->uniq[u], tune.ray_group);
@@ -218,9 +230,11 @@ int prepare(em_batch* b, const em_cloud* clouds, int32_t count, const std::vecto
   bd->maps = reinterpret_cast<const MapDev*>(db + sizeof(BatchDev));
   bd->clouds = reinterpret_cast<const CloudDev*>(db + sizeof(BatchDev) + (size_t)b->max_maps * sizeof(MapDev));
   bd->n_cells = cells;
-  for (int u = 0; u < nm && !use_flags(cells, total); ++u) md[u].touched = nullptr;
+  for (int u = 0; u < nm; ++u)
+    if (md[u].keys || !use_flags(flat_cells, total)) md[u].touched = nullptr;
   bd->n_items = items;
   bd->ctl = b->bctl;
+  if (kind.slots) bd->tab = b->tab;
   bd->passes = (kind.wall || kind.drift ? kPassPre : 0u) | (kind.ray || kind.drift ? kPassCells : 0u);
   bd->wait_budget = b->wait_budget;
   // upload header + maps, and the clouds at their fixed offset
@@ -280,6 +294,7 @@ void release(em_batch* b) {
     if (b->ev[i]) cudaEventDestroy(b->ev[i]);
   }
   cudaFree(b->bctl);
+  table_free(&b->tab);
   cudaFree(b->desc_dev);
   cudaFreeHost(b->desc_host);
   delete b;
@@ -337,6 +352,8 @@ int em_batch_create(int device, int32_t max_maps, int32_t max_clouds, int64_t ma
                   ~size_t(255);
   cudaError_t e = cudaMalloc((void**)&b->bctl, sizeof(BatchCtl));
   if (e == cudaSuccess) e = cudaMemset(b->bctl, 0, sizeof(BatchCtl));
+  if (e == cudaSuccess && max_cells > kFlatCells)
+    e = table_alloc(&b->tab, table_slots(std::min(max_points, (int64_t)max_maps * max_cells)), true, nullptr);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->desc_dev, b->desc_bytes * kSlots);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->desc_host, b->desc_bytes * kSlots);
   for (int i = 0; i < kSlots && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&b->ev[i], cudaEventDisableTiming);
@@ -376,7 +393,7 @@ int em_update_batch(em_batch* b, em_map* const* maps, const em_cloud* clouds, in
   // upload and grids of its own size instead of the capacity's; a served request
   // at 2,000 updates/s took 67 us through the graph, em_update 49.
   if (b->uniq.size() == 1 && count <= kDescClouds && b->tune.ray_group == kValueGroup && !b->prof &&
-      !(b->flags & EM_BATCH_PERSISTENT) && !(map_flags(b->uniq[0]) & EM_F_TRACE))
+      !(b->flags & EM_BATCH_PERSISTENT) && !(map_flags(b->uniq[0]) & EM_F_TRACE) && map_has_room(b->uniq[0], total))
     return map_update_one(b->uniq[0], clouds, count, total, s);
   Prepared p;
   rc = prepare(b, clouds, count, map_pts, total, b->tune, s, &p);

@@ -33,6 +33,14 @@ int map_clean(em_map* m, cudaStream_t s);
 // total points, as a batch of that map alone does it (no trace, no profiling).
 int map_update_one(em_map* m, const em_cloud* clouds, int32_t n_clouds, int64_t total, cudaStream_t s);
 
+// Can an update of that many points of this map run without allocating?
+bool map_has_room(const em_map* m, int64_t points);
+
+// Device memory of a table of sums, zeroed; cnt only when the wall rule may count.
+cudaError_t table_alloc(SumTable* t, int64_t slots, bool cnt, int64_t* bytes);
+void table_free(SumTable* t);
+cudaError_t table_clear(const SumTable& t, cudaStream_t s);
+
 // Copy layers, ring offsets, shift and update index of src into dst (same size).
 int map_copy_state(em_map* dst, const em_map* src, cudaStream_t s);
 

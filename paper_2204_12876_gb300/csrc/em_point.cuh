@@ -23,8 +23,8 @@ struct PointGeom {
 
 // Transform by the sensor pose (Section II-A), distance, cell indices
 // ix = floor((x - x0) / r) of the robot-centric grid (as (x - x0) * (1/r)).
-// kExt: kernels built for batches that use the exclusion area or the upper-bound
-// layer; the others carry none of that code (every kernel of one update is
+// kExt: kernels built for batches that use the exclusion area, the upper-bound
+// layer or the table of sums; the others carry none of that code (every kernel of one update is
 // launched with the same kExt, so they all agree on which points are valid).
 template <bool kExt>
 __device__ __forceinline__ PointGeom point_geom(const MapDev& m, const CloudDev& c, float px, float py,

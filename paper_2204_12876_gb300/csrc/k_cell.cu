@@ -27,6 +27,14 @@ __global__ void __launch_bounds__(kCellThreads) k_cells(const __grid_constant__ 
   cells_pass(view(d), own_grid());
 }
 
+// Latency-bound: a slot's key, its sums and its cell's state are dependent reads, the
+// last one scattered (16 us for 491,521 slots, 113,000 of them in use).
+template <class D>
+__global__ void __launch_bounds__(kCellThreads) k_sums(const __grid_constant__ D d) {
+  begin_after_previous();
+  sums_pass(view(d), own_grid());
+}
+
 // DRAM-bound on many maps (427 MB in 135 us for the 64-map batch: 36 bytes of
 // sums and 12 of state per touched cell, read and written); 8-12 us cold on one.
 template <class D>
@@ -54,6 +62,13 @@ Launch cells_launch(int64_t n_cells, bool by_value) {
 }
 Launch refresh_launch(int64_t n_cells, bool by_value) {
   return item_launch(EM_KERNEL(k_refresh, by_value), n_cells, EM_PROF_RAY, "k_refresh");
+}
+
+Launch sums_launch(uint32_t slots, bool by_value) {
+  if (!slots) return {};
+  const int64_t blocks = ((int64_t)slots + kCellThreads - 1) / kCellThreads, cap = (int64_t)sm_count() * 8;
+  return {EM_KERNEL(k_sums, by_value), (unsigned)(blocks < cap ? blocks : cap), kCellThreads, 0, false, EM_PROF_FUSE,
+          "k_sums", 0};
 }
 
 Launch write_launch(int64_t n_cells, bool by_value) {

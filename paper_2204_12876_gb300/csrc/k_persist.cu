@@ -7,6 +7,7 @@
 //   points per cell (maps with the wall rule), thresholds and coarse grids
 //   | points: gate, sums, ray march (blocks take runs from the work counter); for
 //   |   scattered points in parts, the thresholds refreshed between them
+//   | new state of the table's cells (maps beyond kFlatCells)
 //   | new state of every cell, removal of marked cells, overlap clearance
 //
 // The stencils (normals, smoothing, in-painting) follow as their own kernels.
@@ -89,6 +90,10 @@ __global__ void __launch_bounds__(kPersistThreads, 4) k_persist(const BatchDev* 
       if (!ok) break;
     }
     points_pass<G, true, kExt>(b, all, i, *reinterpret_cast<PointsSmem<true>*>(sm));
+    ok = grid_barrier(b, nb, budget, s_ok);
+  }
+  if (ok && b.tab.slots) {
+    sums_pass(b, all);
     ok = grid_barrier(b, nb, budget, s_ok);
   }
   if (ok) write_pass(b, all);

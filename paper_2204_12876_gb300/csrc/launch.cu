@@ -20,6 +20,7 @@ Sequence update_sequence(const UpdateKind& k, int64_t n_points, int64_t n_cells)
       if (i > 0) q.add(refresh_launch(n_cells, k.by_value));
       q.add(points_launch(n_points, k.ray_group, k.ray, k.ext, i, k.by_value));
     }
+    if (n_points > 0) q.add(sums_launch(k.slots, k.by_value));
     q.add(write_launch(n_cells, k.by_value));
   }
   if (k.stencils) q.add(stencils_launch(n_cells, k.by_value));

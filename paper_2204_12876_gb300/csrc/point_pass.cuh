@@ -82,7 +82,13 @@ __device__ __forceinline__ void pre_pass(const V& b, Grid gr, PreSmem& S) {
     // one count per run of lanes in the same cell
     int head, len;
     key_runs(inm && m.cnt ? (unsigned long long)(uint32_t)c.map << 32 | (uint32_t)key : ~0ull, head, len);
-    if (inm && m.cnt && lane == head) atomicAdd(&m.cnt[key], (uint32_t)len);
+    const bool counts = inm && m.cnt && lane == head;
+    uint32_t q = (uint32_t)key;
+    if (kExt && b.tab.slots) {
+      const uint32_t s = slot_of(counts && m.keys, b.tab, m, m.cell_begin + key);
+      if (m.keys) q = s;
+    }
+    if (counts) atomicAdd(&m.cnt[q], (uint32_t)len);
     if (inm && m.drift_flat > 0.f) {
       // the three loads are independent: all in flight at once
       const float var = m.var[key], nz = m.nz[key], hc = m.h[key];
@@ -155,15 +161,24 @@ struct AccStage {
 // the accumulators: runs of equal cells in consecutive lanes are first reduced
 // by a segmented scan of the exact sums.  Every lane takes part; returns the
 // lane's status (meaningful where inm).
-__device__ __forceinline__ uint8_t add_points(const MapDev& m, int map, bool one_map, bool inm, uint32_t p, float z,
-                                              float d, AccStage& A) {
+template <bool kExt, class V>
+__device__ __forceinline__ uint8_t add_points(const V& b, const MapDev& m, int map, bool one_map, bool inm, uint32_t p,
+                                              float z, float d, AccStage& A) {
   const int lane = threadIdx.x & 31;
   Fix fw{0, 0u}, ft{0, 0u};
   uint8_t st = kPtOutside;
+  uint32_t q = p;  // where the cell's sums are
+  if (kExt && b.tab.slots) {  // the first lane of a run looks its slot up
+    const bool keyed = inm && m.keys;
+    int head, len;
+    key_runs(keyed ? (unsigned long long)(m.cell_begin + p) : ~0ull, head, len);
+    const uint32_t s = __shfl_sync(kFull, slot_of(keyed && lane == head, b.tab, m, m.cell_begin + p), head);
+    if (keyed) q = s;
+  }
   if (inm) {
     const float var = m.var[p], h = m.h[p];  // the loads are independent: all in flight at once
     const int32_t tl = m.t_last[p];
-    const int32_t cnt = m.cnt ? (int32_t)m.cnt[p] : 0;
+    const int32_t cnt = m.cnt ? (int32_t)m.cnt[q] : 0;
     const bool valid = isfinite(var);
     const float ve = valid ? var_eff(m, var, tl) : 0.f;
     const float vp = point_variance(m, d);
@@ -184,7 +199,7 @@ __device__ __forceinline__ uint8_t add_points(const MapDev& m, int map, bool one
   // needs; within a run of at most 32 lanes the 27-bit low parts and the counts
   // (accepted | rejected << 16) fit 32 bits
   uint32_t nn = st == kPtFused ? 1u : st == kPtRejected ? (1u << 16) : 0u;
-  const uint32_t tag = inm ? p : 0xffffffffu;
+  const uint32_t tag = inm ? q : 0xffffffffu;
   const uint32_t prev = __shfl_up_sync(kFull, tag, 1);  // (every lane takes part in the shuffles)
   bool first = lane == 0 || prev != tag;
   if (!one_map) {
@@ -211,9 +226,9 @@ __device__ __forceinline__ uint8_t add_points(const MapDev& m, int map, bool one
   }
   // the run's last lane holds its sums
   if (tail) {
-    if (m.touched) m.touched[p / kTile] = 1;  // every writer stores the same
-    if (nn >> 16) atomicAdd(&m.rej[p], nn >> 16);
-    if ((nn & 0xffffu) && (wh | (long long)wl) == 0) atomicOr(&m.acc[p].wl, kAccTouched);
+    if (m.touched) m.touched[q / kTile] = 1;  // every writer stores the same (maps with keys have no flags)
+    if (nn >> 16) atomicAdd(&m.rej[q], nn >> 16);
+    if ((nn & 0xffffu) && (wh | (long long)wl) == 0) atomicOr(&m.acc[q].wl, kAccTouched);
   }
   const bool add = tail && (nn & 0xffffu);
   const unsigned am = __ballot_sync(kFull, add);
@@ -221,7 +236,7 @@ __device__ __forceinline__ uint8_t add_points(const MapDev& m, int map, bool one
   if (add) {
     const int k = __popc(am & ((1u << lane) - 1u));
     A.sum[k] = CellAcc{(unsigned long long)wh, wl, (unsigned long long)th, tl};
-    A.dst[k] = m.acc + p;
+    A.dst[k] = m.acc + q;
   }
   __syncwarp();
   for (int k = lane >> 2; k < runs; k += 8)
@@ -442,7 +457,7 @@ __device__ __forceinline__ void points_pass(const V& b, Grid gr, int part, Point
     const uint32_t cell = inm ? (uint32_t)phys_index(m, pg.ix, pg.iy) : 0u;
     const int map0 = __shfl_sync(kFull, map, 0);
     const bool one_map = __all_sync(kFull, map == map0);
-    const uint8_t st = add_points(m, map, one_map, inm, cell, pg.z, pg.d, SM.w[warp].acc);
+    const uint8_t st = add_points<kExt>(b, m, map, one_map, inm, cell, pg.z, pg.d, SM.w[warp].acc);
     if (b.tr_status && live) {
       b.tr_ix[g] = pg.finite ? pg.ix : INT32_MIN;
       b.tr_iy[g] = pg.finite ? pg.iy : INT32_MIN;

@@ -29,7 +29,7 @@ void note(const std::string& line) {
 
 cudaError_t alloc(void** p, size_t bytes, bool host) {
   const size_t page = (size_t)sysconf(_SC_PAGESIZE), room = (bytes + page - 1) / page * page;
-  char* m = (char*)mmap(nullptr, room + page, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS, -1, 0);
+  char* m = (char*)mmap(nullptr, room + page, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
   if (m == MAP_FAILED) return cudaErrorMemoryAllocation;
   mprotect(m + room, page, PROT_NONE);
   *p = m + (room - bytes) / 4 * 4;  // (ends within 3 bytes of the guard)

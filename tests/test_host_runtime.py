@@ -123,3 +123,35 @@ for k in range(2, n + 1):  # the first k - 1 kernels are launched, the k-th is n
     update()
     assert log() == whole  # clean again
 """)
+
+
+@pytest.mark.parametrize("wall", [0, 2])
+@pytest.mark.parametrize("ray", [0.0, 0.04])
+def test_large_maps_hold_memory_for_their_points_not_for_every_cell(run, ray, wall):
+    """A map holds, besides its layers, marks and ray thresholds, at most 40 bytes a
+    cell for the sums of 512 tiles of 1024 cells (21 MB), and about 80 bytes for
+    each point of its largest update, at most 48 a cell: 120 maps of 4096 x 4096
+    cells are admitted to 40 GB."""
+    run(f"""
+for side in (64, 500, 724, 725, 1000, 4096):
+    P = em.Params(width=side, height=side, ray_step={ray}, wall_num_thresh={wall})
+    m = em.Map(P)
+    nc = side * side
+    coarse = (side // 8 + 4) ** 2
+    layers = nc * (12 + 4 + 1 / 8) + 4 * coarse + 80 * (nc / 1024 + 1) + (1 << 16)
+    sums = 40 * min(nc, 1 << 19)
+    assert m.info()["device_bytes"] <= layers + sums, (side, m.info())
+    for n in (0, 20000, 300000):
+        m.reserve(n)
+        points = min(80 * 1.25 * n, 48 * nc) if nc > 1 << 19 else 0
+        assert m.info()["device_bytes"] <= layers + sums + points, (side, n, m.info())
+    m.reserve(5 * nc)  # more points than cells: a sum per cell
+    assert m.info()["device_bytes"] <= layers + max(sums, 48 * nc)
+    m.close()
+
+srv = em.Server(budget_bytes=40 << 30, max_slots=16, n_streams=1, max_batch_maps=4, max_batch_points=1 << 20,
+                max_map_cells=1 << 24, graph=False)
+for _ in range(120):
+    srv.add_map(em.Params(width=4096, height=4096, ray_step={ray}, wall_num_thresh={wall}))
+srv.close()
+""")
