@@ -146,6 +146,15 @@ int group(em_batch* b, em_map* const* maps, const em_cloud* clouds, int32_t coun
   return EM_OK;
 }
 
+// Does an update of `count` clouds of the one map m run as em_update does?  With
+// nothing to upload and grids of its own size instead of the capacity's; a served
+// request at 2,000 updates/s (a lightly loaded server's batches are of one map)
+// took 67 us through the graph, em_update 49.
+bool runs_alone(const em_batch* b, const em_map* m, const em_tuning& tune, int32_t count, int64_t total) {
+  return count <= kDescClouds && tune.ray_group == kValueGroup && !b->prof && !(b->flags & EM_BATCH_PERSISTENT) &&
+         !(map_flags(m) & EM_F_TRACE) && map_has_room(m, total);
+}
+
 // A failed update may have stopped between its launches.
 void mark_dirty(em_batch* b) {
   b->dirty = true;
@@ -389,11 +398,7 @@ int em_update_batch(em_batch* b, em_map* const* maps, const em_cloud* clouds, in
   int64_t total = 0;
   rc = group(b, maps, clouds, count, &map_pts, &total);
   if (rc) return rc;
-  // One map (a lightly loaded server's batches): as em_update, with nothing to
-  // upload and grids of its own size instead of the capacity's; a served request
-  // at 2,000 updates/s took 67 us through the graph, em_update 49.
-  if (b->uniq.size() == 1 && count <= kDescClouds && b->tune.ray_group == kValueGroup && !b->prof &&
-      !(b->flags & EM_BATCH_PERSISTENT) && !(map_flags(b->uniq[0]) & EM_F_TRACE) && map_has_room(b->uniq[0], total))
+  if (b->uniq.size() == 1 && runs_alone(b, b->uniq[0], b->tune, count, total))
     return map_update_one(b->uniq[0], clouds, count, total, s);
   Prepared p;
   rc = prepare(b, clouds, count, map_pts, total, b->tune, s, &p);
@@ -483,6 +488,14 @@ int em_batch_autotune(em_batch* b, em_map* const* maps, const em_cloud* clouds, 
   cudaEventCreate(&e1);
   auto time_one = [&](const em_tuning& t, float* ms_out) -> int {
     std::vector<float> ms;
+    auto timed = [&]() -> int {
+      cudaEventRecord(e1, s);
+      if (cudaEventSynchronize(e1) != cudaSuccess) return EM_ERR_CUDA;
+      float x = 0.f;
+      cudaEventElapsedTime(&x, e0, e1);
+      ms.push_back(x);
+      return EM_OK;
+    };
     for (int r = 0; r < reps + 1; ++r) {
       for (size_t j = 0; j < uniq.size(); ++j) {
         int c = map_copy_state(clones[j], uniq[j], s);
@@ -492,21 +505,29 @@ int em_batch_autotune(em_batch* b, em_map* const* maps, const em_cloud* clouds, 
       std::vector<int64_t> map_pts;
       int64_t total = 0;
       int c = group(b, cmaps.data(), clouds, count, &map_pts, &total);
+      // one map: each shape the way em_update_batch would run it
+      const bool alone = uniq.size() == 1 && runs_alone(b, uniq[0], t, count, total);
+      if (c == EM_OK && alone) c = em_reserve(clones[0], total);
+      if (c == EM_OK && alone) {
+        cudaEventRecord(e0, s);
+        c = map_update_one(clones[0], clouds, count, total, s);
+        if (c == EM_OK) c = timed();
+        if (c) return c;
+        continue;
+      }
       if (c == EM_OK) c = prepare(b, clouds, count, map_pts, total, t, s, &p);
       if (c) return c;
       cudaEventRecord(e0, s);
       cudaError_t le = launch_sequence(b, update_sequence(p.kind, p.points, p.cells), p.bd, s);
-      cudaEventRecord(e1, s);
       finish(b, p, s);
       if (le != cudaSuccess) {
         mark_dirty(b);
         return map_record_error("autotune launches", le);
       }
-      if (cudaEventSynchronize(e1) != cudaSuccess) return EM_ERR_CUDA;
-      float x = 0.f;
-      cudaEventElapsedTime(&x, e0, e1);
-      if (r > 0) ms.push_back(x);  // the first run warms up
+      c = timed();
+      if (c) return c;
     }
+    ms.erase(ms.begin());  // the first run warms up
     std::sort(ms.begin(), ms.end());
     *ms_out = ms[ms.size() / 2];
     return EM_OK;

@@ -155,3 +155,28 @@ for _ in range(120):
     srv.add_map(em.Params(width=4096, height=4096, ray_step={ray}, wall_num_thresh={wall}))
 srv.close()
 """)
+
+
+@pytest.mark.parametrize("maps, clouds, alone", [(1, 1, True), (1, 8, True), (1, 9, False), (2, 1, False)])
+def test_autotune_times_the_path_an_update_takes(run, maps, clouds, alone):
+    """A batch of one map with the default shape runs as em_update does, with nothing
+    to upload; the autotuner times that shape so, and the others as they would run."""
+    run(f"""
+n_maps, n_clouds, alone, reps = {maps}, {clouds}, {alone}, 3
+maps = [em.Map(em.Params(width=40, height=30, ray_step=0.04)) for _ in range(n_maps)]
+batch = em.Batch(max_maps=2, max_clouds=16, max_points=1000, max_cells=1200, graph=False)
+pts = np.zeros((20, 3), np.float32)
+count = n_maps * n_clouds
+h = (ctypes.c_void_p * count)(*[maps[i % n_maps].handle.value for i in range(count)])
+c = (em._Cloud * count)(*[em._cloud_struct(pts, POSE, True) for _ in range(count)])
+uploads = lambda lines: sum(l.startswith("copy 1 ") for l in lines)  # host to device
+log()
+em._check(lib.em_update_batch(batch._h, h, c, count, None), "em_update_batch")
+per_update = uploads(log())
+assert per_update == (0 if alone else 2)
+t = em._Tuning()
+em._check(lib.em_batch_autotune(batch._h, h, c, count, None, reps, ctypes.byref(t)), "em_batch_autotune")
+lines = log()
+assert sum("k_write" in l for l in lines) == 5 * (reps + 1)  # ray_group 1, 2, 4, 8 and 16
+assert uploads(lines) == 2 * (reps + 1) * (4 if alone else 5), uploads(lines)
+""")
