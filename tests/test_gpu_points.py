@@ -214,3 +214,31 @@ def test_uploaded_descriptor_equals_parameter(em, extra):
         for k, v in got[0][0].items():
             assert np.array_equal(v, s[k], equal_nan=True), k
         assert st == got[0][1]
+
+
+@pytest.mark.parametrize("ray_group", [1, 2, 8, 32])
+@pytest.mark.parametrize("order", ["runs", "alternating", "random"])
+def test_many_points_in_few_cells(em, ray_group, order):
+    """150,000 points of one cell and 60,000 of three others, in runs, in turn and in
+    random order among points of other cells: the accumulators' sums, with every
+    kind of launch shape, against the float64 means."""
+    rng = np.random.default_rng(12)
+    W, H = 60, 50
+    cells = np.concatenate([np.tile([[17, 20]], (150_000, 1)), np.tile([[18, 20], [0, 0], [59, 49]], (20_000, 1)),
+                            np.stack([rng.integers(W, size=30_000), rng.integers(H, size=30_000)], axis=1)])
+    if order == "random":
+        cells = cells[rng.permutation(len(cells))]
+    elif order == "alternating":  # neighbours in a warp in different cells
+        cells = cells.reshape(30, -1, 2).transpose(1, 0, 2).reshape(-1, 2)
+    xy = (cells + 0.5 + rng.uniform(-0.3, 0.3, cells.shape) - np.array([W, H]) / 2) * R
+    p = np.concatenate([xy, rng.uniform(-0.8, -0.3, (len(cells), 1))], axis=1).astype(np.float32)
+    maps = [em.Map(em.Params(width=W, height=H, resolution=R, noise_a0=0.005, noise_a2=0.002, ray_step=R)) for _ in range(2)]
+    batch = em.Batch(max_maps=2, max_clouds=2, max_points=2 * len(p), max_cells=W * H)
+    batch.set_tuning(ray_group=ray_group, fuse_chunk=512, big_thresh=256)
+    d = torch.from_numpy(p).cuda()
+    batch.update([(m, d, POSE) for m in maps])
+    for m in maps:
+        m.sync()
+        check(m.state(), [(p, cells)], W, H)
+        assert m.stats()["points_accepted"] == len(p)
+    batch.close()

@@ -82,3 +82,70 @@ def test_parts_equal_one_part(em, upper, batched):
     for k in ("h", "var", "t_last") + (("upper",) if upper else ()):
         assert np.array_equal(a[k], c[k], equal_nan=True), k
     assert sa == sc and sa["cells_cleared"] > 0 and sa["ray_samples"] > 0
+
+
+@pytest.mark.parametrize("graph, persistent", [(False, False), (True, False), (True, True)])
+@pytest.mark.parametrize("upper", [False, True])
+def test_batches_in_parts_equal_separate_updates(em, upper, graph, persistent):
+    """Two maps of different sizes whose clouds together reach the size from which
+    scattered points go in parts, each below it by itself: the batch, in parts with
+    refreshed thresholds, leaves what the maps' own updates leave, bit for bit --
+    with the wall rule, the time variance, the Eq. 4 guard, the upper-bound layer."""
+    specs = [dict(width=300, height=290, cleanup_normal_thresh=0.3, flags=em.F_NORMALS | (em.F_UPPER if upper else 0)),
+             dict(width=211, height=333, wall_num_thresh=3, time_variance=1e-6, ray_step=0.06)]
+    counts = (620_000, 480_000)
+    assert sum(counts) > 1 << 20 > max(counts)
+    base = dict(resolution=R, noise_a0=0.005, noise_a2=0.002, mahalanobis_k=2.5, outlier_variance=1e-4, ray_step=R)
+    both = []
+    for _ in range(2):
+        maps = [em.Map(em.Params(**{**base, **s})) for s in specs]
+        for j, m in enumerate(maps):
+            parity.prior_to_gpu(m, synth.random_prior(seed=95 + j, width=specs[j]["width"], height=specs[j]["height"],
+                                                      t_now=5, with_normals=j == 0))
+            m.shift(17, -40 * j)
+        both.append(maps)
+    b = em.Batch(max_maps=2, max_clouds=2, max_points=sum(counts), max_cells=300 * 300, graph=graph, persistent=persistent)
+    for k in range(2):
+        clouds = []
+        for j, n in enumerate(counts):
+            pts, pose = synth.scattered_cloud(97 + 2 * k + j, n, 6.3, nan_frac=0.01)
+            clouds.append((torch.from_numpy(pts).cuda(), pose))
+        b.update([(m, *c) for m, c in zip(both[0], clouds)])
+        for m, c in zip(both[1], clouds):
+            m.update(*c)
+        for x, y in zip(*both):
+            x.sync()
+            s, t = x.state(), y.state()
+            for key in s:
+                assert np.array_equal(s[key], t[key], equal_nan=True), (k, key)
+            assert x.stats() == y.stats()
+    assert both[0][0].stats()["cells_cleared"] > 0 and both[0][1].stats()["points_wall"] > 0
+    b.close()
+
+
+@pytest.mark.parametrize("W, H", [(1, 1), (7, 9), (8, 8), (9, 1)])
+def test_cells_of_tiny_maps_are_compared(em, W, H):
+    """Few points, so that few cells are marginal: over several scenes most cells of
+    maps of one and a few cells agree with the oracle, none of them excluded."""
+    compared = valid = 0
+    for seed in range(24):
+        rng = np.random.default_rng(seed)
+        P = dict(width=W, height=H, resolution=R, noise_a0=0.005, noise_a2=0.002, var_min=1e-8, mahalanobis_k=2.5,
+                 outlier_variance=1e-4, ray_step=(0.02, 0.04, 0.13)[seed % 3])
+        prior = synth.random_prior(seed=seed, width=W, height=H, t_now=5, obstacle_frac=0.3, with_normals=False)
+        half, t = np.array([W, H]) * R / 2, np.array([0.3 * (seed % 2), -0.2 * (seed % 2), 0.5])
+        pw = np.concatenate([rng.uniform(-1.5, 1.5, (40, 2)) * (half + 0.1), rng.normal(0.0, 0.1, (40, 1))], axis=1)
+        pts, pose = (pw - t).astype(np.float32), synth.pose_matrix(np.eye(3), t)
+        om = oracle.OracleMap(parity.oracle_params(P))
+        parity.prior_to_oracle(om, prior)
+        prior_valid = np.isfinite(om.state()["var"])
+        tr = om.update((pts, pose), trace=True, unit=oracle.FP32_UNIT, abs_band=parity.ABS_BAND)
+        m = em.Map(em.Params(**P, flags=em.F_TRACE))
+        parity.prior_to_gpu(m, prior)
+        m.update(torch.from_numpy(pts).cuda(), pose)
+        cmp = parity.compare_update(tr, om.state(), m.state(), m.trace(40), check_stencils=(), prior_valid=prior_valid,
+                                    max_excluded=1.0)
+        m.close()
+        compared += cmp.notes["cells_compared"]
+        valid += int(np.isfinite(om.state()["var"]).sum())
+    assert valid > 0 and compared > valid / 2, (compared, valid)
