@@ -17,8 +17,8 @@
  *   - Map layers are float32.  Layer arrays exchanged with the caller are in
  *     logical row-major order [iy][ix], cell (ix, iy) covering
  *     [x0 + ix r, x0 + (ix+1) r) x [y0 + iy r, y0 + (iy+1) r) of the map frame.
- *   - Errors found by a kernel (a capacity overflow, a bounded wait that ran
- *     out) are recorded on the device and reported by the next em_sync() or
+ *   - Errors found by a kernel (a bounded wait that ran out, an internal check
+ *     that failed) are recorded on the device and reported by the next em_sync() or
  *     em_get_stats() of that map.
  */
 #ifndef EM_H
@@ -247,8 +247,10 @@ enum {
   EM_PROF_SLOTS
 };
 int em_profile(em_map* map, int enable);
-/* Accumulated milliseconds and launch counts per slot since profiling was
- * enabled (both arrays EM_PROF_SLOTS long, host memory); waits for the map. */
+/* Accumulated milliseconds per slot since profiling was enabled, and the number
+ * of updates they were taken over: a slot's launches of one update count once (the
+ * parts of k_points and k_refresh between them).  Both arrays EM_PROF_SLOTS long,
+ * host memory; waits for the map. */
 int em_profile_read(em_map* map, double* ms, int64_t* launches);
 
 /* ---- Batched form: many maps (each with one or more clouds) updated by one
@@ -335,12 +337,16 @@ typedef struct em_server em_server;
 enum { EM_SERVE_BATCHED = 0, EM_SERVE_PLAIN = 1 };
 
 /* Admission accounting: each admitted request counts this many bytes per point,
- * and each batch stream as many for max_batch_points points. */
+ * and each batch stream as many for max_batch_points points.  A nominal charge that
+ * bounds the load, not memory of that size: requests hold nothing per point but
+ * their host clouds' room in the input arena, and a batch stream a table of about 72
+ * bytes per point when max_map_cells is above 2^19, else nothing. */
 enum { EM_SERVE_RECORD_BYTES = 16 };
 
 typedef struct em_server_cfg {
   int32_t device;
-  int64_t budget_bytes;     /* device bytes for resident maps + batch workspaces + admitted requests */
+  int64_t budget_bytes;     /* resident maps, stage buffers and the input arena (device bytes), and the nominal
+                               charges of batch streams and admitted requests (EM_SERVE_RECORD_BYTES) */
   int32_t max_slots;        /* requests admitted at a time */
   int32_t n_streams;        /* batches in flight at a time (batched mode) */
   int32_t max_batch_maps;   /* maps per batch */

@@ -39,7 +39,6 @@ int cuda_status(cudaError_t e, const char* what) {
 constexpr int kSlots = 4;
 constexpr int kMaxClouds = 64;
 constexpr size_t kDescBytes = sizeof(BatchDev) + sizeof(MapDev) + kMaxClouds * sizeof(CloudDev) + 64;
-static_assert(kDescBytes >= sizeof(MapDesc), "the descriptor ring");
 
 template <class T>
 cudaError_t dev_alloc(T** p, size_t count, int64_t* total) {

@@ -18,8 +18,8 @@
 namespace em {
 
 // Latency-bound on one map (9 us cold for 250 x 250 cells: two dependent loads
-// and the square roots), DRAM-bound on many (31 us for the 64-map batch's 6.8 M
-// cells).  It takes the place of a threshold pass in the point kernel and a
+// and the square roots), DRAM-bound on many (37 us for the 64-map batch's 6.8 M
+// cells, 43 cold).  It takes the place of a threshold pass in the point kernel and a
 // one-thread-per-block coarse kernel (12 us alone on one map).
 template <class D>
 __global__ void __launch_bounds__(kCellThreads) k_cells(const __grid_constant__ D d) {
@@ -35,8 +35,9 @@ __global__ void __launch_bounds__(kCellThreads) k_sums(const __grid_constant__ D
   sums_pass(view(d), own_grid());
 }
 
-// DRAM-bound on many maps (427 MB in 135 us for the 64-map batch: 36 bytes of
-// sums and 12 of state per touched cell, read and written); 8-12 us cold on one.
+// DRAM-bound on many maps (106 us for the 64-map batch; 556 MB in 132 us cold: 36
+// bytes of sums and 12 of state per touched cell, read and written); 8-12 us cold
+// on one.
 template <class D>
 __global__ void __launch_bounds__(kCellThreads) k_write(const __grid_constant__ D d) {
   begin_after_previous();

@@ -28,7 +28,8 @@ __device__ __forceinline__ float pinf() { return __int_as_float(0x7f800000); }
 // share the staged heights).  They only read heights and variances and write
 // layers of their own, so no order between them is needed, and the tiles of the
 // quick ones fill the SMs beside the in-painting's long searches (three kernels
-// one after the other: 28.7 + 10.4 + 8.8 us on a 500 x 500 map).
+// one after the other: 28.7 + 10.4 + 8.8 us on a 500 x 500 map).  The build with an
+// uploaded descriptor spills 28 bytes a thread at its two blocks per SM.
 constexpr int kStThreads = 512, kStWarps = kStThreads / 32;
 constexpr int kStT = 32, kStRim = 2, kStSpan = kStT + 2 * kStRim;
 constexpr int kStRounds = kStT * kStT / kStThreads;  // cells per thread of a tile

@@ -8,8 +8,8 @@
 // reductions of a 407,040-point depth image, or of 14 M points in random order
 // over 64 maps, cost less than a counting sort by tile and a fusion from shared
 // memory did (count, range, scatter and fusion kernels: 1130 us of the 64-map
-// batch, where the sums now add about 560 us; 174 us of the depth image's 240 us,
-// now under 15 us), and one launch takes the place of four.
+// batch, where gate and sums without rays take 380; 184 us of the depth image's
+// kernels, now 18), and one launch takes the place of four.
 //
 // Visibility (Section II-E): one ray per valid point.  The ray from the sensor
 // origin o (the pose translation) to the point is sampled at s_k = o + (k step / d) (R p_s) for
@@ -38,7 +38,8 @@
 // points the gathers of thresholds from L2 (1.4 G sectors for the 64-map batch,
 // which the parts with refreshed thresholds cut to about a third).  256 threads
 // and 64 registers, four blocks per SM: one resident wave that takes runs of
-// batches from a counter.  Measured and not kept: one test for the beam of a warp's
+// batches from a counter (the builds that read an uploaded descriptor spill 32 bytes
+// a thread at that, those with the descriptor as a parameter none).  Measured and not kept: one test for the beam of a warp's
 // 32 rays before the rays' own (no fewer instructions: rays of an image row
 // have 4 to 8 chunks); thresholds or block maxima updated in place by the march
 // (mark_sample).
