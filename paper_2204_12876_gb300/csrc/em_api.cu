@@ -27,6 +27,7 @@ thread_local char g_cuda_msg[256] = "";
 int cuda_status(cudaError_t e, const char* what) {
   if (e == cudaSuccess) return EM_OK;
   snprintf(g_cuda_msg, sizeof(g_cuda_msg), "%s: %s", what, cudaGetErrorString(e));
+  cudaGetLastError();  // reported here: not again by the next launch that asks for it
   return e == cudaErrorMemoryAllocation ? EM_ERR_OOM : EM_ERR_CUDA;
 }
 

@@ -19,6 +19,8 @@ std::string g_log;
 std::map<const void*, std::string> g_names;        // host stub -> kernel name
 struct Block { void* map; size_t len, bytes; bool host; };
 std::map<uintptr_t, Block> g_blocks;
+cudaError_t g_last = cudaSuccess;  // what cudaGetLastError returns next
+long g_fail_alloc = 0;   // fails the n-th device allocation from now on (1-based); 0: none
 long g_fail_launch = 0;  // fails the n-th launch from now on (1-based); 0: none
 float g_ms = 1.f;
 
@@ -54,7 +56,7 @@ cudaError_t launched(const void* fn) {
     name = g_names[fn];
     if (g_fail_launch > 0 && --g_fail_launch == 0) {
       g_log += "failed " + name + "\n";
-      return cudaErrorLaunchOutOfResources;
+      return g_last = cudaErrorLaunchOutOfResources;
     }
     g_log += "launch " + name + "\n";
   }
@@ -75,9 +77,13 @@ extern "C" {
 const char* fake_log() { return g_log.c_str(); }
 void fake_clear() { g_log.clear(); }
 void fake_fail_launch(long n) { g_fail_launch = n; }
+void fake_fail_alloc(long n) { g_fail_alloc = n; }
 
 // ---- the runtime
-cudaError_t cudaMalloc(void** p, size_t n) { return alloc(p, n, false); }
+cudaError_t cudaMalloc(void** p, size_t n) {
+  if (g_fail_alloc > 0 && --g_fail_alloc == 0) return g_last = cudaErrorMemoryAllocation;
+  return alloc(p, n, false);
+}
 cudaError_t cudaMallocHost(void** p, size_t n) { return alloc(p, n, true); }
 cudaError_t cudaFree(void* p) { return release(p); }
 cudaError_t cudaFreeHost(void* p) { return release(p); }
@@ -101,7 +107,11 @@ cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
   *v = a == cudaDevAttrMultiProcessorCount ? 152 : a == cudaDevAttrClockRate ? 2070000 : 1;
   return cudaSuccess;
 }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() {
+  const cudaError_t e = g_last;
+  g_last = cudaSuccess;
+  return e;
+}
 const char* cudaGetErrorString(cudaError_t) { return "injected"; }
 cudaError_t cudaGetSymbolAddress(void** p, const void* s) { *p = const_cast<void*>(s); return cudaSuccess; }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {

@@ -20,7 +20,7 @@ ctypes.CDLL = lambda path, *a, **k: real({lib!r} if str(path).endswith("libem.so
 from paper_2204_12876_gb300 import em
 lib = em.lib
 lib.fake_log.restype = ctypes.c_char_p
-lib.fake_fail_launch.argtypes = [ctypes.c_long]
+lib.fake_fail_launch.argtypes = lib.fake_fail_alloc.argtypes = [ctypes.c_long]
 em._stream_handle = lambda stream: None
 
 def log(clear=True):
@@ -179,4 +179,45 @@ em._check(lib.em_batch_autotune(batch._h, h, c, count, None, reps, ctypes.byref(
 lines = log()
 assert sum("k_write" in l for l in lines) == 5 * (reps + 1)  # ray_group 1, 2, 4, 8 and 16
 assert uploads(lines) == 2 * (reps + 1) * (4 if alone else 5), uploads(lines)
+""")
+
+
+def test_a_refused_allocation_leaves_no_error_for_the_next_call(run):
+    """Every allocation of a map, and of a large map's table, fails in turn: the call
+    says so, and the next ones work, those included that ask the runtime for its
+    last error after a launch."""
+    run("""
+large = em.Map(em.Params(width=900, height=900, wall_num_thresh=1))
+for k in range(1, 5):
+    lib.fake_fail_alloc(k)
+    try:
+        large.reserve(1000)
+        raise SystemExit("a refused allocation was not reported")
+    except em.EMError as e:
+        assert e.code == em.EM_ERR_OOM
+    assert large.info()["point_capacity"] == 0
+    em.Map(em.Params(width=20, height=10, ray_step=0.04)).close()
+large.reserve(1000)
+before = large.info()["device_bytes"]
+lib.fake_fail_alloc(2)
+try:
+    large.reserve(100000)
+    raise SystemExit("a refused allocation was not reported")
+except em.EMError as e:
+    assert e.code == em.EM_ERR_OOM
+assert large.info()["point_capacity"] == 0 and large.info()["device_bytes"] < before  # (given back, not half there)
+large.update_host([(np.zeros((2000, 3), np.float32), POSE)])
+large.close()
+k = 0
+while True:
+    k += 1
+    lib.fake_fail_alloc(k)
+    try:
+        em.Map(em.Params(width=20, height=10, ray_step=0.04, wall_num_thresh=1, flags=em.F_NORMALS)).close()
+        break
+    except em.EMError as e:
+        assert e.code == em.EM_ERR_OOM
+    lib.fake_fail_alloc(0)
+    em.Map(em.Params(width=20, height=10)).close()
+assert k > 10
 """)
