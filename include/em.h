@@ -257,9 +257,11 @@ int em_profile_read(em_map* map, double* ms, int64_t* launches);
  * sequence of kernels over all of them -- the per-point and per-cell work of
  * every map shares each launch, so small updates no longer pay a launch
  * sequence each.  The arithmetic per map is exactly em_update's.
- * A batch object owns a ring of device descriptors and -- with EM_BATCH_GRAPH -- one CUDA graph
- * per descriptor slot, replayed with a single cudaGraphLaunch per batch (grids
- * are sized from the capacities; actual sizes are read from the descriptor). */
+ * A batch object owns a ring of device descriptors, a table of sums when max_cells
+ * is above 2^19 (about 72 bytes per point of max_points, or per cell if they are
+ * fewer), and -- with EM_BATCH_GRAPH -- one CUDA graph per descriptor slot, replayed
+ * with a single cudaGraphLaunch per batch (grids are sized from the capacities;
+ * actual sizes are read from the descriptor). */
 typedef struct em_batch em_batch;
 
 /* EM_BATCH_PERSISTENT: one cooperative launch of all blocks that fit on the
