@@ -96,8 +96,8 @@ constexpr int kOrderSamples = 64;
 
 // Updates of more than kFlagCells cells (all maps together) of which the points can
 // touch half at most keep a flag per tile, so that clouds on a few cells of large maps
-// do not cost a read of all their accumulators (32 maps of 1,000,000 cells, 5,000
-// points each: 214 us without flags, 143 with).  In smaller updates the flags would
+// do not cost a read of all their accumulators (64 maps of 250,000 cells, 2,000
+// points each, with rays: 213 us without flags, 190 with).  In smaller updates the flags would
 // be a few sectors that every warp writes: without them a raw depth image took 45 us
 // instead of 49, four depth cameras 36.8 instead of 38.5; and where the points are as
 // many as the cells most tiles are touched anyhow (64-map batch, 14 M points on 6.8 M
